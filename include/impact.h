@@ -23,8 +23,9 @@
  * edge N_d is hi_d itself. Input points are points (no input cells).
  *
  * Precisions:
- *   IMPACT_FP64_PLAIN  every factor of every pair evaluated in FP64 (erfc per
- *                      pair and dimension); lo/up stored as double.
+ *   IMPACT_FP64_PLAIN  every pair's factors and products in FP64 round-to-
+ *                      nearest (each distinct image's factors evaluated
+ *                      once); lo/up stored as double.
  *   IMPACT_FP32_SOUND  factors from per-row FP32 tables with outward rounding:
  *                      lo32 <= lo64 and up32 >= up64 for the FP64 values of
  *                      the definition above; lo/up stored as float. The row

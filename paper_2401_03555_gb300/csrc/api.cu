@@ -117,6 +117,23 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
                 B.work_max[c] = std::max(B.work_max[c],
                                          impact::walk_work_bytes(P.desc.n, P.desc.leaf_cap, c == 1));
         }
+        if (precision == IMPACT_FP64_PLAIN) {
+            const ImpactDesc &D = P.desc;
+            if (q == 0) B.item_begin.assign((size_t)count * IMPACT_MAX_DIM + 1, 0);
+            for (int d = 0; d < IMPACT_MAX_DIM; ++d) {
+                const size_t i = (size_t)q * IMPACT_MAX_DIM + d;
+                int64_t units = 0;
+                if (D.walk64 && d < D.n) {
+                    const int ipw = 32 / D.dim[d].group;
+                    units = (D.dim[d].n_items + ipw - 1) / ipw;
+                }
+                B.item_begin[i + 1] = B.item_begin[i] + units;
+            }
+            if (D.walk64) {
+                ++B.any64;
+                B.warp64 = std::max(B.warp64, (int)impact::walk64_bytes(D));
+            }
+        }
         h = mix(h, P.hash);
     }
     B.rows = B.row_begin[count];
@@ -148,6 +165,7 @@ BatchLayout batch_layout(const Batch &B)
     L.unit_begin = put((size_t)(count + 1) * 8);
     L.descs = put((size_t)count * 8);
     L.recs = put((size_t)count * 8);
+    L.item_begin = put(B.item_begin.size() * 8);
     L.tables.resize(count);
     L.tl.resize(count);
     for (int q = 0; q < count; ++q) {
@@ -162,7 +180,9 @@ BatchLayout batch_layout(const Batch &B)
     L.rec.resize(count);
     for (int q = 0; q < count; ++q) {
         const Plan &P = B.plans[q];
-        L.rec[q] = put(B.prec == PREC_FP32_SOUND ? (size_t)P.rows * P.desc.rec_stride : 0);
+        L.rec[q] = put(!B.walks                    ? 0
+                       : B.prec == PREC_FP32_SOUND ? (size_t)P.rows * P.desc.rec_stride
+                                                   : (size_t)P.item_bytes);
     }
     L.total = o;
     return L;
@@ -250,12 +270,16 @@ impact_status upload(const Batch &B, Work &W, cudaStream_t st)
     bi.desc = (const ImpactDesc *const *)(W.base + L.descs);
     bi.rec = (unsigned char *const *)(W.base + L.recs);
     bi.next_row = W.counter();
+    bi.item_units = B.item_begin.empty() ? 0 : B.item_begin.back();
+    bi.item_begin = (const int64_t *)(W.base + L.item_begin);
     memcpy(host.data() + L.index, &bi, sizeof(bi));
     memcpy(host.data() + L.row_begin, B.row_begin.data(), (size_t)(count + 1) * 8);
     memcpy(host.data() + L.unit_begin, B.unit_begin.data(), (size_t)(count + 1) * 8);
+    if (!B.item_begin.empty())
+        memcpy(host.data() + L.item_begin, B.item_begin.data(), B.item_begin.size() * 8);
     for (int q = 0; q < count; ++q) {
         const ImpactDesc *d = W.desc(q);
-        unsigned char *r = B.prec == PREC_FP32_SOUND ? W.base + L.rec[q] : nullptr;
+        unsigned char *r = W.base + L.rec[q];
         memcpy(host.data() + L.descs + 8 * (size_t)q, &d, 8);
         memcpy(host.data() + L.recs + 8 * (size_t)q, &r, 8);
         impact::pack_tables(B.plans[q], host.data() + L.tables[q], W.base + L.tables[q],
@@ -351,9 +375,24 @@ cudaError_t walk_pass(const Batch &B, const Work &W, int mode, int warps,
     return cudaSuccess;
 }
 
+// FP64 walk launches of one pass, as walk_pass.
+cudaError_t walk_pass64(const Batch &B, const Work &W, bool emit, const impact::RowOutputs &o,
+                        unsigned long long *counter, int64_t chunk_rows, cudaStream_t st)
+{
+    const int64_t step = chunk_rows > 0 ? chunk_rows : std::max<int64_t>(B.rows, 1);
+    for (int64_t r0 = 0; r0 < B.rows; r0 += step) {
+        cudaError_t e = cudaMemsetAsync(counter, 0, 8, st);
+        if (e == cudaSuccess)
+            e = impact::launch_walk64(W.index(), r0, std::min(B.rows, r0 + step), B.warp64, emit, o,
+                                      counter, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // count pass: row_ptr (row pointers and the total), sink_lo, sink_up, trunc,
-// row_flags. FP32: one walk whose look-back writes the row pointers; FP64:
-// per-row counts, then the scan.
+// row_flags: per-row counts, then the scan. FP64 builds whose tables are too
+// large for the walk (ImpactDesc.walk64) are counted by the per-pair kernel.
 impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cudaStream_t st,
                         int64_t chunk_rows)
 {
@@ -367,9 +406,15 @@ impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cu
         CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st));
         return IMPACT_OK;
     }
+    if (B.any64) {
+        CK(impact::launch_items64(W.index(), B.item_begin.back(), W.status(), st));
+        CK(impact::launch_terms64(W.index(), B.rows, out->sink_lo, out->sink_up, out->trunc, st));
+        CK(walk_pass64(B, W, false, o, W.counter(), chunk_rows, st));
+    }
     for (int q = 0; q < B.count(); ++q)
-        CK(impact::launch_rows(W.desc(q), B.prec, false, 0, B.plans[q].rows,
-                               shifted(o, B.row_begin[q], B.rows), st));
+        if (!B.plans[q].desc.walk64)
+            CK(impact::launch_rows(W.desc(q), B.prec, false, 0, B.plans[q].rows,
+                                   shifted(o, B.row_begin[q], B.rows), st));
     CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st));
     return IMPACT_OK;
 }
@@ -386,9 +431,15 @@ impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int
                                          nullptr, st));
         CK(walk_pass(B, W, WALK_EMIT, B.tune.emit_warps, o, W.counter() + 1, chunk_rows, st));
     } else {
+        if (B.any64) {
+            if (!records_ready)
+                CK(impact::launch_items64(W.index(), B.item_begin.back(), W.status(), st));
+            CK(walk_pass64(B, W, true, o, W.counter() + 1, chunk_rows, st));
+        }
         for (int q = 0; q < B.count(); ++q)
-            CK(impact::launch_rows(W.desc(q), B.prec, true, 0, B.plans[q].rows,
-                                   shifted(o, B.row_begin[q], B.rows), st));
+            if (!B.plans[q].desc.walk64)
+                CK(impact::launch_rows(W.desc(q), B.prec, true, 0, B.plans[q].rows,
+                                       shifted(o, B.row_begin[q], B.rows), st));
     }
     return IMPACT_OK;
 }
@@ -1052,6 +1103,7 @@ impact_status impact_region_vectors(const impact_system *sys, const impact_grid 
     Batch batch;
     s = make_batch(&req, 1, IMPACT_FP64_PLAIN, nullptr, batch);
     if (s != IMPACT_OK) return s;
+    batch.walks = false;
     Work W;
     s = get_work(batch, nullptr, st, W);
     if (s != IMPACT_OK) return s;

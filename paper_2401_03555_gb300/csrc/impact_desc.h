@@ -27,6 +27,19 @@ struct ImpactDim {
     float delta_cells;    // delta / h
     uint32_t div_m;       // fast division by N: q = (umulhi(x, div_m) + x) >> div_s
     int div_s;
+    // Distinct images of the dimension. The image in dimension d depends on
+    // the cell's index in the dimensions f_d reads (A_dk != 0) and on the class
+    // of the input (inputs with the same offset): rows that agree in these
+    // share one item, numbered sum_k idx_k item_mul[k] + class (caller images:
+    // the row itself). Everything the kernels derive from an image alone is
+    // made once per item.
+    int64_t n_items;
+    int64_t item_mul[IMPACT_MAX_DIM];   // 0: the image does not read dimension k
+    int n_classes;        // classes of inputs
+    int w64;              // FP64: targets an item's table holds (largest window)
+    int group;            // FP64: lanes that make one item (8, 16 or 32)
+    int item_stride;      // FP64: bytes of one item
+    int64_t item_off;     // FP64: bytes of the build's items before this dimension's
 };
 
 // Kinds (match impact_kind) and precisions (match impact_precision).
@@ -67,7 +80,9 @@ struct ImpactDesc {
     const double *inputs;     // [n_inputs][m]
     const double *images;     // IMAGES: [rows][n][2], caller's device array
     int n_max;                // max N_d
-    int pad1;
+    int walk64;               // FP64: built by the item tables and the tree walk
+    const int *cls;           // [n][n_inputs] class of an input in dimension d
+    const int *cls_rep;       // [n][n_inputs] an input of each class
 
     // FP32-sound table path. Values "in erf units" of dimension d are
     // multiplied by 1/(sigma_d sqrt2) on the host in FP64 and stored as FP32
@@ -103,6 +118,8 @@ struct BatchIndex {
     const int64_t *row_begin;           // [count + 1]
     const int64_t *unit_begin;          // [count + 1]
     const ImpactDesc *const *desc;      // [count] device descriptors
-    unsigned char *const *rec;          // [count] FP32 per-row records
+    unsigned char *const *rec;          // [count] FP32: per-row records, FP64: items
+    int64_t item_units;                 // FP64: warps' worth of items, all builds
+    const int64_t *item_begin;          // [count * IMPACT_MAX_DIM + 1] first unit per dimension
     unsigned long long *next_row;       // [2] row counters of the count / emit walk
 };

@@ -1,19 +1,16 @@
-// kernels.cu -- the FP64-plain path and the row-pointer scan.
+// kernels.cu -- the row-pointer scan, the region vectors, the sampled-noise
+// kernels and the per-pair FP64 kernel.
 //
-// FP64 plain: one warp builds one row (source cell x input) at a time (Alg. 2:
-// rows are independent) and evaluates every factor of every candidate pair in
-// FP64 (the comparison baseline; the FP32-sound path is in tree_fp32.cu).
+// FP64 builds are made by walk_fp64.cu; rows_fp64 here builds those whose
+// tables do not fit it (a window box of more than 2048 targets): one warp per
+// row evaluates every factor of every candidate pair.
 // Per row:
 //   1. interval image [m_lo, m_hi] of f over the cell (table lookups + sums)
 //   2. per dimension, a window of target cells outside of which every upper
 //      factor is below cutoff/2 (Sec. 4.4: entries whose upper bound is
-//      negligible are not stored), then the per-dimension factor table
-//      U_d[t] (upper, Def. 3.1 T_max relaxed) and L_d[t] (lower, T_min)
-//   3. the window box is enumerated in C order: an outer prefix of
-//      dimensions is pruned as a whole when even the largest remaining
-//      factors cannot lift it to the cutoff, the surviving prefixes are
-//      expanded over the inner dimensions, lanes test up >= cutoff and the
-//      warp compacts the kept targets with ballot/popc
+//      negligible are not stored), trimmed to the targets that pass alone
+//   3. the window box is enumerated in C order, lanes test up >= cutoff and
+//      the warp compacts the kept targets with ballot/popc
 //   4. per-row terms: the out-of-domain sink bounds (Remark 4.1), the
 //      truncated mass and the row-sum checks of Def. 3.1, combined in FP64.
 // The count pass runs 1-4 without storing pairs; a scan turns the counts into
@@ -26,9 +23,12 @@
 
 #include "impact_desc.h"
 #include "kernels.h"
+#include "rowmath.cuh"
 #include "sound_fp32.cuh"
 
 namespace {
+
+using namespace rowmath;
 
 constexpr int kWarpsPerBlock = 8;
 constexpr int kThreads = kWarpsPerBlock * 32;
@@ -48,111 +48,9 @@ __device__ __forceinline__ double warp_sum_d(double v)
     return v;
 }
 
-// Cell digits (C order) of a row, and the input index.
-__device__ __forceinline__ void decode_row(const ImpactDesc &D, int64_t row, int *idx, int &j)
-{
-    int64_t cell = row / D.n_inputs;
-    j = (int)(row - cell * D.n_inputs);
-    uint32_t c = (uint32_t)cell;
-#pragma unroll
-    for (int d = IMPACT_MAX_DIM - 1; d >= 0; --d) {
-        if (d < D.n) {
-            uint32_t N = (uint32_t)D.dim[d].N;
-            uint32_t q = c / N;
-            idx[d] = (int)(c - q * N);
-            c = q;
-        }
-    }
-}
-
-// Interval image of f(., u_j) over the cell in dimension d.
-//   SOUND: outward-rounded bounds of the exact image.
-//   plain: round-to-nearest in the same operation order as the definition
-//          (sum over k of the per-term range, then the input offset).
-template <bool SOUND>
-__device__ __forceinline__ void image_dim(const ImpactDesc &D, int64_t row, const int *idx, int j,
-                                          int d, double &mlo, double &mhi)
-{
-    const int n = D.n;
-    if (D.kind == KIND_AFFINE) {
-        const int NM = D.n_max;
-        if (SOUND) {
-            double slo = 0.0, shi = 0.0;
-            for (int k = 0; k < n; ++k) {
-                int t = (d * n + k) * NM + idx[k];
-                slo = __dadd_rd(slo, D.term_dn[t]);
-                shi = __dadd_ru(shi, D.term_up[t]);
-            }
-            mlo = __dadd_rd(slo, D.off_dn[j * n + d]);
-            mhi = __dadd_ru(shi, D.off_up[j * n + d]);
-        } else {
-            double slo = 0.0, shi = 0.0;
-            for (int k = 0; k < n; ++k) {
-                int t = ((d * n + k) * NM + idx[k]) * 2;
-                slo = __dadd_rn(slo, D.term_rn[t]);
-                shi = __dadd_rn(shi, D.term_rn[t + 1]);
-            }
-            mlo = __dadd_rn(slo, D.off_rn[j * n + d]);
-            mhi = __dadd_rn(shi, D.off_rn[j * n + d]);
-        }
-    } else if (D.kind == KIND_UNICYCLE) {
-        const double *E = D.edges + D.dim[d].edge_off;
-        double xlo = E[idx[d]], xhi = E[idx[d] + 1];
-        if (d == 2) {
-            double om = D.inputs[j * D.m + 1];
-            if (SOUND) { mlo = __dadd_rd(xlo, om); mhi = __dadd_ru(xhi, om); }
-            else { mlo = __dadd_rn(xlo, om); mhi = __dadd_rn(xhi, om); }
-        } else {
-            const double *u = (SOUND ? D.uni_sd : D.uni_rn) + ((int64_t)idx[2] * D.n_inputs + j) * 4;
-            double vlo = u[d * 2 + 0], vhi = u[d * 2 + 1];
-            if (SOUND) { mlo = __dadd_rd(xlo, vlo); mhi = __dadd_ru(xhi, vhi); }
-            else { mlo = __dadd_rn(xlo, vlo); mhi = __dadd_rn(xhi, vhi); }
-        }
-    } else {
-        const double *im = D.images + (row * n + d) * 2;
-        mlo = im[0];
-        mhi = im[1];
-    }
-}
-
-// Conservative window [a, b] of target cells in dimension d: any target whose
-// cell lies entirely more than delta beyond the image has every upper factor
-// below cutoff/2. One extra cell of slack on each side absorbs rounding.
-__device__ __forceinline__ void window_dim(const ImpactDim &g, double mlo, double mhi, int &a,
-                                           int &b)
-{
-    if (!(g.delta < INFINITY)) {
-        a = 0;
-        b = g.N - 1;
-        return;
-    }
-    double xa = floor((mlo - g.delta - g.lo) * g.inv_h) - 1.0;
-    double xb = floor((mhi + g.delta - g.lo) * g.inv_h) + 1.0;
-    xa = fmin(fmax(xa, 0.0), (double)(g.N - 1));
-    xb = fmin(fmax(xb, 0.0), (double)(g.N - 1));
-    a = (int)xa;
-    b = (int)xb;
-    if (b < a) b = a - 1;   // empty
-}
-
 // ---------------------------------------------------------------------------
 // FP64 plain row kernel: every factor of every candidate pair in FP64
 // ---------------------------------------------------------------------------
-
-// g(c, e; m) = Phi((e-m)/sigma) - Phi((c-m)/sigma), inv_s = 1/(sigma sqrt 2).
-__device__ __forceinline__ double g64(double c, double e, double m, double inv_s)
-{
-    double a = (c - m) * inv_s;
-    double b = (e - m) * inv_s;
-    if (a >= 0.0) return 0.5 * (erfc(a) - erfc(b));
-    if (b <= 0.0) return 0.5 * (erfc(-b) - erfc(-a));
-    return 1.0 - 0.5 * erfc(-a) - 0.5 * erfc(b);
-}
-
-__device__ __forceinline__ double clampd(double x, double lo, double hi)
-{
-    return x < lo ? lo : (x > hi ? hi : x);
-}
 
 // Upper factor of target cell t of dimension d.
 __device__ __forceinline__ double up64(const ImpactDim &g, const double *E, int t, double mlo,

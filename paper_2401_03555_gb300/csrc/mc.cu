@@ -69,6 +69,7 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     Batch B;
     impact_status s = make_batch(&req, 1, IMPACT_FP64_PLAIN, nullptr, B);
     if (s != IMPACT_OK) return s;
+    B.walks = false;
     B.plans[0].desc.cutoff = cutoff;
     B.plans[0].desc.prec = precision;
     configure_pool_once();

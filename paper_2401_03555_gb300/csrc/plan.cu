@@ -72,6 +72,63 @@ float2 pair_of(double v)
     return make_float2(hi, lo);
 }
 
+// Distinct images of every dimension (impact_desc.h): which coordinates and
+// which input classes the image in dimension d depends on. Inputs are of one
+// class when everything they bring to the image is bitwise the same.
+void number_items(const impact_system *sys, const impact_inputs *inputs, Plan &P)
+{
+    ImpactDesc &D = P.desc;
+    const int n = D.n, ni = D.n_inputs, m = D.m;
+    P.cls.assign((size_t)n * ni, 0);
+    P.cls_rep.assign((size_t)n * ni, 0);
+    std::vector<int> order((size_t)ni);
+    for (int d = 0; d < n; ++d) {
+        ImpactDim &g = D.dim[d];
+        bool reads[IMPACT_MAX_DIM] = {false};
+        auto less = [&](int a, int b) -> int {   // -1, 0, 1: input a before, like, after b
+            auto cmp = [](double x, double y) { return memcmp(&x, &y, sizeof(double)); };
+            if (D.kind == KIND_AFFINE) {
+                const size_t i = (size_t)a * n + d, k = (size_t)b * n + d;
+                int c = cmp(P.off_rn[i], P.off_rn[k]);
+                if (!c) c = cmp(P.off_dn[i], P.off_dn[k]);
+                if (!c) c = cmp(P.off_up[i], P.off_up[k]);
+                return c;
+            }
+            const int u = d == 2 ? 1 : 0;   // unicycle: v moves x and y, om the heading
+            return cmp(inputs->points[(int64_t)a * m + u], inputs->points[(int64_t)b * m + u]);
+        };
+        if (D.kind == KIND_AFFINE) {
+            for (int k = 0; k < n; ++k) reads[k] = sys->A[d * n + k] != 0.0;
+        } else if (D.kind == KIND_UNICYCLE) {
+            reads[d] = true;
+            reads[2] = true;
+        }
+        int classes = 0;
+        if (D.kind != KIND_IMAGES) {
+            for (int j = 0; j < ni; ++j) order[j] = j;
+            std::sort(order.begin(), order.end(), [&](int a, int b) {
+                const int c = less(a, b);
+                return c != 0 ? c < 0 : a < b;
+            });
+            for (int i = 0; i < ni; ++i) {
+                if (i == 0 || less(order[i - 1], order[i]) != 0)
+                    P.cls_rep[(size_t)d * ni + classes++] = order[i];
+                P.cls[(size_t)d * ni + order[i]] = classes - 1;
+            }
+            g.n_classes = classes;
+            int64_t c = classes;
+            for (int k = n - 1; k >= 0; --k) {
+                g.item_mul[k] = reads[k] ? c : 0;
+                if (reads[k]) c *= D.dim[k].N;
+            }
+            g.n_items = c;
+        } else {
+            g.n_classes = 1;
+            g.n_items = D.rows;
+        }
+    }
+}
+
 uint64_t fnv(uint64_t h, const void *p, size_t bytes)
 {
     const unsigned char *c = (const unsigned char *)p;
@@ -117,6 +174,8 @@ TableLayout table_layout(const Plan &p)
     L.mo = put(p.mo.size() * 4);
     L.um = put(p.um.size() * 4);
     L.omm = put(p.omm.size() * 4);
+    L.cls = put(p.cls.size() * 4);
+    L.cls_rep = put(p.cls_rep.size() * 4);
     L.total = o;
     return L;
 }
@@ -329,6 +388,7 @@ impact_status make_plan(const impact_system *sys, const impact_grid *grid,
         }
         box = std::min<int64_t>(box * w, cells);
         need += w;
+        g.w64 = (int)w;
         g.wcap = (int)(sys->kind == IMPACT_IMAGES ? std::min<int64_t>(w, 128) : w);
         g.delta_cells = isfinite(g.delta) ? (float)(g.delta * g.inv_h) : INFINITY;
         div_magic((uint32_t)g.N, g.div_m, g.div_s);
@@ -415,6 +475,8 @@ impact_status make_plan(const impact_system *sys, const impact_grid *grid,
             }
         }
     }
+    number_items(sys, inputs, P);
+    if (precision == IMPACT_FP64_PLAIN) P.item_bytes = impact::size_items64(D, P.nnz_bound);
     // identity of the arguments, for reusing a caller's workspace
     uint64_t h = 1469598103934665603ull;
     int hdr[5] = {sys->kind, n, m, (int)precision, n_inputs};
@@ -465,6 +527,8 @@ void pack_tables(const Plan &P, unsigned char *host, unsigned char *dev_base,
     D.mo = (const float *)dp(L.mo, P.mo.size());
     D.um = (const float *)dp(L.um, P.um.size());
     D.omm = (const float *)dp(L.omm, P.omm.size());
+    D.cls = (const int *)dp(L.cls, P.cls.size());
+    D.cls_rep = (const int *)dp(L.cls_rep, P.cls_rep.size());
     D.images = dev_images;
     memcpy(host + L.desc, &D, sizeof(D));
     auto put = [&](size_t off, const void *src, size_t bytes) {
@@ -491,6 +555,8 @@ void pack_tables(const Plan &P, unsigned char *host, unsigned char *dev_base,
     put(L.mo, P.mo.data(), P.mo.size() * 4);
     put(L.um, P.um.data(), P.um.size() * 4);
     put(L.omm, P.omm.data(), P.omm.size() * 4);
+    put(L.cls, P.cls.data(), P.cls.size() * 4);
+    put(L.cls_rep, P.cls_rep.data(), P.cls_rep.size() * 4);
 }
 
 }  // namespace impact

@@ -32,6 +32,9 @@ struct Plan {
     // FP32-sound table path
     std::vector<float2> ea, ta_lo, ta_hi, oa, ua, oma;
     std::vector<float> mu_lo, mu_hi, mo, um, omm;
+    // distinct images (impact_desc.h): input classes per dimension
+    std::vector<int> cls, cls_rep;
+    int64_t item_bytes = 0;   // FP64: the build's item tables
     int64_t rows = 0;
     int64_t nnz_bound = 0;
     int table_need = 0;   // upper bound of the staged entries per row (-1: unknown)
@@ -41,7 +44,8 @@ struct Plan {
 // Offsets (in bytes, 256-aligned) of the descriptor and tables of one build.
 struct TableLayout {
     size_t desc, edges, term_rn, term_dn, term_up, off_rn, off_dn, off_up, uni_rn, uni_sd,
-        inputs, ea, ta_lo, ta_hi, oa, ua, oma, mu_lo, mu_hi, mo, um, omm, total;
+        inputs, ea, ta_lo, ta_hi, oa, ua, oma, mu_lo, mu_hi, mo, um, omm, cls, cls_rep,
+        total;
 };
 
 size_t align256(size_t x);

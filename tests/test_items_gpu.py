@@ -1,0 +1,84 @@
+"""Shared image tables against the oracle where they can go wrong (needs a GPU):
+window widths around the lane groups and around the widest sorted window,
+dimensions that read few coordinates or none, repeated inputs, windows too wide
+for the tables. Tolerances are those of parity.py."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import parity as PA
+from paper_2401_03555_gb300 import impact, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def linear(cells, A, sigma_cells, cutoff, inputs, B=None, seed=0):
+    """x+ = A x + B u + w on [-1,1]^n with sigma in cell widths."""
+    n = len(cells)
+    A = np.asarray(A, np.float64)
+    rng = np.random.default_rng(seed)
+    U = np.asarray(inputs, np.float64)
+    return W.Problem(
+        name="items", kind=W.AFFINE, lo=np.full(n, -1.0), hi=np.full(n, 1.0),
+        cells=np.asarray(cells, np.int32), inputs=U,
+        sigma=2.0 / np.asarray(cells) * np.asarray(sigma_cells, np.float64), cutoff=cutoff, A=A,
+        B=rng.normal(0.0, 0.2, (n, U.shape[1])) if B is None else np.asarray(B, np.float64),
+        c=rng.uniform(-0.05, 0.05, n))
+
+
+def images_of(prob, seed):
+    rng = np.random.default_rng(seed)
+    m = rng.uniform(-1.2, 1.2, (prob.rows, prob.n))
+    return W.with_images(prob, np.stack([m, m + rng.uniform(0.0, 0.3, m.shape)], axis=2))
+
+
+U1, U2 = [[-0.3], [0.4]], [[-0.3, 0.1], [0.4, 0.1], [0.4, 0.1], [0.0, -0.5]]
+PROBLEMS = {
+    # windows as wide as the grid: one below, at and above 8, 16 and 32 edges
+    "width-7-8": lambda: linear([7, 8], np.eye(2) * 0.9, [4, 4], 1e-8, U1),
+    "width-15-16": lambda: linear([15, 16], [[0.9, 0.1], [0.0, 0.8]], [6, 6], 1e-8, U1),
+    "width-31-32": lambda: linear([31, 32], [[0.9, 0.0], [0.1, 0.8]], [9, 9], 1e-8, U1),
+    "width-33-3": lambda: linear([33, 3], np.eye(2) * 0.9, [9, 2], 1e-8, U1),
+    # the last dimension's window at and beyond the widest sorted one
+    "sorted-256": lambda: linear([3, 256], np.eye(2) * 0.9, [2, 60], 1e-8, U1),
+    "sorted-257": lambda: linear([3, 257], np.eye(2) * 0.9, [2, 60], 1e-8, U1),
+    # windows wider than the FP64 tables (cutoff 0 keeps every cell)
+    "wide-2049": lambda: linear([2049], [[0.9]], [50], 0.0, U1),
+    "wide-2048": lambda: linear([2048], [[0.9]], [50], 0.0, U1),
+    # a dimension that reads no coordinate, signed zeros, repeated inputs
+    "no-reads": lambda: linear([6, 5, 4], [[0, 0, 0], [-0.0, 0.9, 0], [0.2, 0, 0.7]],
+                               [0.8, 0.6, 0.5], 1e-8, U2),
+    "crossed": lambda: linear([5, 4, 3, 4], np.roll(np.eye(4) * 0.9, 1, axis=1),
+                              [0.5, 0.9, 0.4, 0.6], 1e-6, U2,
+                              B=[[0.1, 0], [0, 0.1], [0, 0], [-0.0, 0]]),
+    "dense-6d": lambda: linear([3, 2, 3, 2, 3, 2], np.eye(6) * 0.8 + 0.02, [0.5] * 6, 0.0, U1),
+    "images": lambda: images_of(linear([9, 12], np.eye(2), [0.7, 0.5], 1e-8, U2), 3),
+    "one-cell": lambda: linear([1, 1, 5], np.eye(3) * 0.5, [0.3, 1.0, 0.6], 1e-8, U1),
+}
+
+
+@pytest.fixture(scope="module")
+def orc():
+    return oracle.default()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("name", list(PROBLEMS))
+def test_tables_match_the_oracle(orc, name, precision):
+    prob = PROBLEMS[name]()
+    csr = impact.build(prob, precision)
+    torch.cuda.synchronize()
+    rows = np.arange(prob.rows) if prob.rows <= 2000 else W.sample_rows(prob, 200, seed=2)
+    PA.compare(prob, csr, orc.build_rows(prob, rows), orc, precision).assert_ok()
+
+
+def test_mixed_batch_equals_its_builds(orc):
+    """Builds on and off the FP64 tables in one batch: bitwise as alone."""
+    probs = [PROBLEMS[k]() for k in ("no-reads", "wide-2049", "images", "width-33-3")]
+    batch = impact.Batch(probs, "fp64").build()
+    for q, p in enumerate(probs):
+        one, part = impact.build(p, "fp64"), batch.part(q)
+        for k in ("row_ptr", "col", "lo", "up", "sink_lo", "sink_up", "trunc", "row_flags"):
+            assert torch.equal(getattr(one, k), getattr(part, k)), (q, k)
