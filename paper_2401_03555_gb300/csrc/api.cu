@@ -184,6 +184,7 @@ BatchLayout batch_layout(const Batch &B)
                        : B.prec == PREC_FP32_SOUND ? (size_t)P.rows * P.desc.rec_stride
                                                    : (size_t)P.item_bytes);
     }
+    L.extra = put((size_t)B.extra);
     L.total = o;
     return L;
 }
@@ -1104,14 +1105,17 @@ impact_status impact_region_vectors(const impact_system *sys, const impact_grid 
     s = make_batch(&req, 1, IMPACT_FP64_PLAIN, nullptr, batch);
     if (s != IMPACT_OK) return s;
     batch.walks = false;
+    batch.extra = region_scratch(batch.plans[0].desc, B);
     Work W;
     s = get_work(batch, nullptr, st, W);
     if (s != IMPACT_OK) return s;
     WorkHold hold{W, st};
     s = upload(batch, W, st);
     if (s == IMPACT_OK) {
-        cudaError_t e = launch_regions(W.desc(0), batch.rows, B, mode == IMPACT_REGION_CELL_SUM,
-                                       precision == IMPACT_FP32_SOUND, r_lo, r_up, a_lo, a_up, st);
+        cudaError_t e = launch_regions(batch.plans[0].desc, W.desc(0), batch.rows, B,
+                                       mode == IMPACT_REGION_CELL_SUM,
+                                       precision == IMPACT_FP32_SOUND, W.base + W.L.extra, r_lo,
+                                       r_up, a_lo, a_up, st);
         if (e != cudaSuccess) s = fail(IMPACT_ERR_CUDA, cudaGetErrorString(e));
     }
     impact_status r = release(W, st);

@@ -463,11 +463,82 @@ __device__ __forceinline__ double add_up(double a, double b) { return SOUND ? __
 template <bool SOUND>
 __device__ __forceinline__ double add_dn(double a, double b) { return SOUND ? __dadd_rd(a, b) : a + b; }
 
-// One thread per row: the interval image, the sink (the domain box, Remark
-// 4.1), then per region box the product over dimensions of either the box's
-// own factor (one relaxation per box) or the sum of the per-cell factors
-// over the box's cells (the paper's sums: sum over the cells of a product
-// of per-dimension factors equals the product of per-dimension sums).
+// Largest and smallest factor of a block of cells [first, last] of dimension d
+// over the image: the block's own (one relaxation), or the sums of its cells'
+// (the paper's sums: the sum over a box's cells of a product of per-dimension
+// factors equals the product of the per-dimension sums). first < 0: the whole
+// domain as one block.
+template <bool SOUND>
+__device__ __forceinline__ double2 block_factor(const ImpactDim &g, const double *E, int first,
+                                                int last, bool cell_sum, double mlo, double mhi)
+{
+    if (first < 0 || !cell_sum) {
+        const double c = first < 0 ? g.lo : E[first], e = first < 0 ? g.hi : E[last + 1];
+        return make_double2(f_max<SOUND>(c, e, mlo, mhi, g.inv_s),
+                            f_min<SOUND>(c, e, mlo, mhi, g.inv_s));
+    }
+    double fu = 0.0, fl = 0.0;
+    if (SOUND) {
+        for (int i = first; i <= last; ++i) {
+            fu = add_up<SOUND>(fu, f_max<SOUND>(E[i], E[i + 1], mlo, mhi, g.inv_s));
+            fl = add_dn<SOUND>(fl, f_min<SOUND>(E[i], E[i + 1], mlo, mhi, g.inv_s));
+        }
+        return make_double2(fu, fl);
+    }
+    // plain: erfc once per edge and image end, shared by the cells beside it
+    double c = E[first], x0 = (c - mlo) * g.inv_s, x1 = (c - mhi) * g.inv_s;
+    double f0 = erfc(fabs(x0)), f1 = erfc(fabs(x1));
+    for (int i = first; i <= last; ++i) {
+        const double e = E[i + 1], y0 = (e - mlo) * g.inv_s, y1 = (e - mhi) * g.inv_s;
+        const double h0 = erfc(fabs(y0)), h1 = erfc(fabs(y1));
+        const double lo = mass64(x0, f0, y0, h0), hi = mass64(x1, f1, y1, h1);
+        const double mid = 0.5 * (c + e);
+        fu += mid < mlo ? lo : mid > mhi ? hi : g64(c, e, mid, g.inv_s);
+        fl += fmin(lo, hi);
+        c = e;
+        x0 = y0;
+        x1 = y1;
+        f0 = h0;
+        f1 = h1;
+    }
+    return make_double2(fu, fl);
+}
+
+// The row's four vectors from its blocks' factors, f(b, d) for b = -1 (the
+// domain) and the boxes: the sink (Remark 4.1), then the products over the
+// dimensions summed over the boxes.
+template <bool SOUND, typename F>
+__device__ __forceinline__ void region_vectors(const RegionBoxes &B, int n, F f, int64_t row,
+                                               double *r_lo, double *r_up, double *a_lo,
+                                               double *a_up)
+{
+    double rl = 0.0, ru = 0.0, xl = 0.0, xu = 0.0;
+    for (int b = -1; b < B.count; ++b) {
+        double pu = 1.0, pl = 1.0;
+        for (int d = 0; d < n; ++d) {
+            const double2 v = f(b, d);
+            pu = mul_up<SOUND>(pu, v.x);
+            pl = mul_dn<SOUND>(pl, v.y);
+        }
+        if (b < 0) {
+            xl = SOUND ? fmax(__dsub_rd(1.0, pu), 0.0) : 1.0 - pu;
+            xu = SOUND ? fmin(__dsub_ru(1.0, pl), 1.0) : 1.0 - pl;
+        } else if (b < B.n_target) {
+            rl = add_dn<SOUND>(rl, pl);
+            ru = add_up<SOUND>(ru, pu);
+        } else {
+            xl = add_dn<SOUND>(xl, pl);
+            xu = add_up<SOUND>(xu, pu);
+        }
+    }
+    r_lo[row] = rl;
+    r_up[row] = ru;
+    a_lo[row] = xl;
+    a_up[row] = xu;
+}
+
+// Rows whose images are (nearly) all distinct: one thread per row evaluates
+// its blocks' factors.
 template <bool SOUND>
 __global__ void __launch_bounds__(128)
 region_rows(const ImpactDesc *__restrict__ Dp, int64_t rows, RegionBoxes B, bool cell_sum,
@@ -482,49 +553,67 @@ region_rows(const ImpactDesc *__restrict__ Dp, int64_t rows, RegionBoxes B, bool
         int j;
         decode_row(D, row, idx, j);
         double mlo[IMPACT_MAX_DIM], mhi[IMPACT_MAX_DIM];
-        double in_max = 1.0, in_min = 1.0;
-        for (int d = 0; d < n; ++d) {
-            image_dim<SOUND>(D, row, idx, j, d, mlo[d], mhi[d]);
+        for (int d = 0; d < n; ++d) image_dim<SOUND>(D, row, idx, j, d, mlo[d], mhi[d]);
+        auto f = [&](int b, int d) {
             const ImpactDim &g = D.dim[d];
-            in_max = mul_up<SOUND>(in_max, f_max<SOUND>(g.lo, g.hi, mlo[d], mhi[d], g.inv_s));
-            in_min = mul_dn<SOUND>(in_min, f_min<SOUND>(g.lo, g.hi, mlo[d], mhi[d], g.inv_s));
-        }
-        double rl = 0.0, ru = 0.0;
-        double xl = SOUND ? fmax(__dsub_rd(1.0, in_max), 0.0) : 1.0 - in_max;
-        double xu = SOUND ? fmin(__dsub_ru(1.0, in_min), 1.0) : 1.0 - in_min;
-        for (int b = 0; b < B.count; ++b) {
-            double pu = 1.0, pl = 1.0;
-            for (int d = 0; d < n; ++d) {
-                const ImpactDim &g = D.dim[d];
-                const double *E = D.edges + g.edge_off;
-                double fu, fl;
-                if (cell_sum) {
-                    fu = 0.0;
-                    fl = 0.0;
-                    for (int i = B.first[b][d]; i <= B.last[b][d]; ++i) {
-                        fu = add_up<SOUND>(fu, f_max<SOUND>(E[i], E[i + 1], mlo[d], mhi[d], g.inv_s));
-                        fl = add_dn<SOUND>(fl, f_min<SOUND>(E[i], E[i + 1], mlo[d], mhi[d], g.inv_s));
-                    }
-                } else {
-                    const double c = E[B.first[b][d]], e = E[B.last[b][d] + 1];
-                    fu = f_max<SOUND>(c, e, mlo[d], mhi[d], g.inv_s);
-                    fl = f_min<SOUND>(c, e, mlo[d], mhi[d], g.inv_s);
-                }
-                pu = mul_up<SOUND>(pu, fu);
-                pl = mul_dn<SOUND>(pl, fl);
-            }
-            if (b < B.n_target) {
-                rl = add_dn<SOUND>(rl, pl);
-                ru = add_up<SOUND>(ru, pu);
-            } else {
-                xl = add_dn<SOUND>(xl, pl);
-                xu = add_up<SOUND>(xu, pu);
-            }
-        }
-        r_lo[row] = rl;
-        r_up[row] = ru;
-        a_lo[row] = xl;
-        a_up[row] = xu;
+            return block_factor<SOUND>(g, D.edges + g.edge_off, b < 0 ? -1 : B.first[b][d],
+                                       b < 0 ? -1 : B.last[b][d], cell_sum, mlo[d], mhi[d]);
+        };
+        region_vectors<SOUND>(B, n, f, row, r_lo, r_up, a_lo, a_up);
+    }
+}
+
+// Factors of every distinct image (impact_desc.h) and block, one thread each:
+// tab[(first + c) * (count + 1) + 1 + b], dimension d's items from `first`.
+struct RegionItems {
+    int64_t first[IMPACT_MAX_DIM + 1];
+};
+
+template <bool SOUND>
+__global__ void __launch_bounds__(128)
+region_items(const ImpactDesc *__restrict__ Dp, RegionItems I, RegionBoxes B, bool cell_sum,
+             double2 *__restrict__ tab)
+{
+    const ImpactDesc &D = *Dp;
+    const int slots = B.count + 1;
+    const int64_t total = I.first[D.n] * slots;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t it = i / slots;
+        const int b = (int)(i - it * slots) - 1;
+        int d = 0;
+        while (it >= I.first[d + 1]) ++d;
+        int idx[IMPACT_MAX_DIM], j = 0;
+        const int64_t c = it - I.first[d];
+        if (D.kind != KIND_IMAGES) decode_item(D, d, c, idx, j);
+        double mlo, mhi;
+        image_dim<SOUND>(D, c, idx, j, d, mlo, mhi);
+        const ImpactDim &g = D.dim[d];
+        tab[i] = block_factor<SOUND>(g, D.edges + g.edge_off, b < 0 ? -1 : B.first[b][d],
+                                     b < 0 ? -1 : B.last[b][d], cell_sum, mlo, mhi);
+    }
+}
+
+// One thread per row: products of its items' factors.
+template <bool SOUND>
+__global__ void __launch_bounds__(256)
+region_products(const ImpactDesc *__restrict__ Dp, int64_t rows, RegionItems I, RegionBoxes B,
+                const double2 *__restrict__ tab, double *__restrict__ r_lo,
+                double *__restrict__ r_up, double *__restrict__ a_lo, double *__restrict__ a_up)
+{
+    const ImpactDesc &D = *Dp;
+    const int n = D.n, slots = B.count + 1;
+    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < rows;
+         row += (int64_t)gridDim.x * blockDim.x) {
+        int idx[IMPACT_MAX_DIM];
+        int j;
+        decode_row(D, row, idx, j);
+        const double2 *at[IMPACT_MAX_DIM];
+#pragma unroll
+        for (int d = 0; d < IMPACT_MAX_DIM; ++d)
+            if (d < n) at[d] = tab + (I.first[d] + item_of(D, row, idx, j, d)) * slots + 1;
+        auto f = [&](int b, int d) { return at[d][b]; };
+        region_vectors<SOUND>(B, n, f, row, r_lo, r_up, a_lo, a_up);
     }
 }
 
@@ -1012,11 +1101,43 @@ cudaError_t launch_labels(const RegionBoxes &boxes, int64_t total_cells, uint8_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_regions(const ImpactDesc *d_desc, int64_t rows, const RegionBoxes &boxes,
-                           bool cell_sum, bool sound, double *r_lo, double *r_up, double *a_lo,
-                           double *a_up, cudaStream_t stream)
+// Items only where rows share them: below two rows per item the table's
+// write and read back cost about what they save. FP64 erfc per row, dimension
+// and cell bounded the per-row kernel: the 11^5 room's cell sums (1.45M rows,
+// 22k items) took 50.7 ms and take 0.32 ms.
+int64_t region_scratch(const ImpactDesc &D, const RegionBoxes &boxes)
+{
+    int64_t items = 0;
+    for (int d = 0; d < D.n; ++d) items += D.dim[d].n_items;
+    return items <= D.rows * D.n / 2 ? items * (boxes.count + 1) * (int64_t)sizeof(double2) : 0;
+}
+
+cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_t rows,
+                           const RegionBoxes &boxes, bool cell_sum, bool sound, void *scratch,
+                           double *r_lo, double *r_up, double *a_lo, double *a_up,
+                           cudaStream_t stream)
 {
     if (rows <= 0) return cudaSuccess;
+    if (region_scratch(D, boxes) > 0) {
+        RegionItems I;
+        I.first[0] = 0;
+        for (int d = 0; d < D.n; ++d) I.first[d + 1] = I.first[d] + D.dim[d].n_items;
+        for (int d = D.n; d < IMPACT_MAX_DIM; ++d) I.first[d + 1] = I.first[d];
+        double2 *tab = (double2 *)scratch;
+        const int64_t total = I.first[D.n] * (boxes.count + 1);
+        const unsigned gi = (unsigned)std::min<int64_t>((total + 127) / 128, 152 * 64);
+        const unsigned gr = (unsigned)std::min<int64_t>((rows + 255) / 256, 152 * 64);
+        if (sound) {
+            region_items<true><<<gi, 128, 0, stream>>>(d_desc, I, boxes, cell_sum, tab);
+            region_products<true><<<gr, 256, 0, stream>>>(d_desc, rows, I, boxes, tab, r_lo, r_up,
+                                                          a_lo, a_up);
+        } else {
+            region_items<false><<<gi, 128, 0, stream>>>(d_desc, I, boxes, cell_sum, tab);
+            region_products<false><<<gr, 256, 0, stream>>>(d_desc, rows, I, boxes, tab, r_lo, r_up,
+                                                           a_lo, a_up);
+        }
+        return cudaGetLastError();
+    }
     const int64_t g = std::min<int64_t>((rows + 127) / 128, 152 * 32);
     if (sound)
         region_rows<true><<<(unsigned)g, 128, 0, stream>>>(d_desc, rows, boxes, cell_sum, r_lo,

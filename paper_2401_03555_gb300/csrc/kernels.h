@@ -75,12 +75,15 @@ cudaError_t launch_mc_rows(const ImpactDesc *d_desc, bool emit, int64_t rows,
 // Labels of every cell (0 free, 1 target, 2 avoid; avoid wins).
 cudaError_t launch_labels(const RegionBoxes &boxes, int64_t total_cells, uint8_t *labels,
                           cudaStream_t stream);
-// Region vectors of rows [0, rows) of the build described by d_desc (FP64
-// tables): cell_sum selects the paper's sums of per-cell bounds, else one
-// relaxation per box; sound selects the enclosing evaluation.
-cudaError_t launch_regions(const ImpactDesc *d_desc, int64_t rows, const RegionBoxes &boxes,
-                           bool cell_sum, bool sound, double *r_lo, double *r_up, double *a_lo,
-                           double *a_up, cudaStream_t stream);
+// Region vectors of rows [0, rows) of the build described by D (FP64 tables):
+// cell_sum selects the paper's sums of per-cell bounds, else one relaxation
+// per box; sound selects the enclosing evaluation. scratch: device memory of
+// region_scratch bytes (0: rows are evaluated one by one).
+int64_t region_scratch(const ImpactDesc &D, const RegionBoxes &boxes);
+cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_t rows,
+                           const RegionBoxes &boxes, bool cell_sum, bool sound, void *scratch,
+                           double *r_lo, double *r_up, double *a_lo, double *a_up,
+                           cudaStream_t stream);
 
 // FP32-sound path (walk_fp32.cu). The setup kernel writes one record per
 // row (record_stride bytes: per-dimension entries, then the window tables)

@@ -24,6 +24,7 @@ struct Batch {
     int rec_max = 0;                      // FP32 walk: largest record of the batch
     int work_max[2] = {0, 0};             // FP32 walk: largest work space, emit / count
     bool walks = true;                    // false: only the tables are used (no walk scratch)
+    int64_t extra = 0;                    // bytes of the call's own scratch
     int any64 = 0, warp64 = 0;            // FP64 walk: builds on it, largest warp memory
     std::vector<int64_t> item_begin;      // FP64 walk: [count * IMPACT_MAX_DIM + 1]
     Tuning tune;
@@ -43,6 +44,7 @@ struct BatchLayout {
     size_t status = 0, counter = 0, scan = 0;
     size_t lb = 0;                         // FP32: one look-back word per row
     std::vector<size_t> rec;               // per build: FP32 per-row records, FP64 items
+    size_t extra = 0;                      // the call's own scratch
     size_t total = 0;
 };
 
