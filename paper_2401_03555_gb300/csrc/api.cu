@@ -95,6 +95,8 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
     B.images.assign(count, nullptr);
     B.row_begin.assign(count + 1, 0);
     B.unit_begin.assign(count + 1, 0);
+    B.item_begin.assign((size_t)count * IMPACT_MAX_DIM + 1, 0);
+    B.leaf_begin.assign(count + 1, 0);
     B.prec = precision;
     uint64_t h = 1469598103934665603ull;
     for (int q = 0; q < count; ++q) {
@@ -113,26 +115,26 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
                                                               : B.nnz_bound + P.nnz_bound;
         if (precision == IMPACT_FP32_SOUND) {
             B.rec_max = std::max(B.rec_max, P.desc.rec_stride);
-            for (int c = 0; c < 2; ++c)
-                B.work_max[c] = std::max(B.work_max[c],
-                                         impact::walk_work_bytes(P.desc.n, P.desc.leaf_cap, c == 1));
+            for (int mode = 0; mode < 3; ++mode)
+                B.work_max[mode] =
+                    std::max(B.work_max[mode], impact::walk_work_bytes(P.desc, mode));
         }
-        if (precision == IMPACT_FP64_PLAIN) {
-            const ImpactDesc &D = P.desc;
-            if (q == 0) B.item_begin.assign((size_t)count * IMPACT_MAX_DIM + 1, 0);
-            for (int d = 0; d < IMPACT_MAX_DIM; ++d) {
-                const size_t i = (size_t)q * IMPACT_MAX_DIM + d;
-                int64_t units = 0;
-                if (D.walk64 && d < D.n) {
-                    const int ipw = 32 / D.dim[d].group;
-                    units = (D.dim[d].n_items + ipw - 1) / ipw;
-                }
-                B.item_begin[i + 1] = B.item_begin[i] + units;
+        const ImpactDesc &D = P.desc;
+        for (int d = 0; d < IMPACT_MAX_DIM; ++d) {
+            const size_t i = (size_t)q * IMPACT_MAX_DIM + d;
+            int64_t units = 0;
+            if ((D.walk64 || D.share32) && d < D.n) {
+                const int ipw = 32 / D.dim[d].group;
+                units = (D.dim[d].n_items + ipw - 1) / ipw;
             }
-            if (D.walk64) {
-                ++B.any64;
-                B.warp64 = std::max(B.warp64, (int)impact::walk64_bytes(D));
-            }
+            B.item_begin[i + 1] = B.item_begin[i] + units;
+        }
+        B.leaf_begin[q + 1] = B.leaf_begin[q] + (D.leaf_shared ? D.leaf_items : 0);
+        if (D.leaf_shared) B.leaf_smem = std::max(B.leaf_smem, impact::leaf32_bytes(D));
+        if (D.share32) ++B.shared32;
+        if (D.walk64) {
+            ++B.any64;
+            B.warp64 = std::max(B.warp64, (int)impact::walk64_bytes(D));
         }
         h = mix(h, P.hash);
     }
@@ -140,10 +142,10 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
     B.units = B.unit_begin[count];
     B.hash = h;   // launch shapes change no result: they are not part of the identity
     if (precision == IMPACT_FP32_SOUND &&
-        2 * (int64_t)B.rec_max + B.work_max[1] > IMPACT_WALK_SMEM_MAX)
+        2 * (int64_t)B.rec_max + B.work_max[WALK_FUSED] > IMPACT_WALK_SMEM_MAX)
         return fail(IMPACT_ERR_ARG,
                     "the builds of this batch together need " +
-                        std::to_string(2 * (int64_t)B.rec_max + B.work_max[1]) +
+                        std::to_string(2 * (int64_t)B.rec_max + B.work_max[WALK_FUSED]) +
                         " bytes of shared memory per warp, more than one warp has: "
                         "batch the widest windows separately");
     return IMPACT_OK;
@@ -165,7 +167,11 @@ BatchLayout batch_layout(const Batch &B)
     L.unit_begin = put((size_t)(count + 1) * 8);
     L.descs = put((size_t)count * 8);
     L.recs = put((size_t)count * 8);
+    L.items = put((size_t)count * 8);
+    L.leafs = put((size_t)count * 8);
+    L.termps = put((size_t)count * 8);
     L.item_begin = put(B.item_begin.size() * 8);
+    L.leaf_begin = put(B.leaf_begin.size() * 8);
     L.tables.resize(count);
     L.tl.resize(count);
     for (int q = 0; q < count; ++q) {
@@ -176,13 +182,18 @@ BatchLayout batch_layout(const Batch &B)
     L.status = put(64);
     L.counter = put(64);
     L.scan = put((size_t)impact::scan_scratch_elems(B.rows) * 8);
-    L.lb = put(B.prec == PREC_FP32_SOUND ? (size_t)B.rows * 8 : 0);
+    L.lb = put(B.prec == PREC_FP32_SOUND ? (size_t)B.rows * 16 : 0);
     L.rec.resize(count);
+    L.item.resize(count);
+    L.leaf.resize(count);
+    L.term.resize(count);
     for (int q = 0; q < count; ++q) {
         const Plan &P = B.plans[q];
-        L.rec[q] = put(!B.walks                    ? 0
-                       : B.prec == PREC_FP32_SOUND ? (size_t)P.rows * P.desc.rec_stride
-                                                   : (size_t)P.item_bytes);
+        const bool rec = B.walks && B.prec == PREC_FP32_SOUND;
+        L.rec[q] = put(rec ? (size_t)P.rows * P.desc.rec_stride : 0);
+        L.item[q] = put(B.walks ? (size_t)P.item_bytes : 0);
+        L.term[q] = put(rec && !P.desc.share32 ? (size_t)P.rows * P.desc.n * 16 : 0);
+        L.leaf[q] = put(B.walks ? (size_t)P.leaf_bytes : 0);
     }
     L.extra = put((size_t)B.extra);
     L.total = o;
@@ -271,18 +282,27 @@ impact_status upload(const Batch &B, Work &W, cudaStream_t st)
     bi.desc = (const ImpactDesc *const *)(W.base + L.descs);
     bi.rec = (unsigned char *const *)(W.base + L.recs);
     bi.next_row = W.counter();
-    bi.item_units = B.item_begin.empty() ? 0 : B.item_begin.back();
+    bi.items = (unsigned char *const *)(W.base + L.items);
+    bi.terms = (unsigned char *const *)(W.base + L.termps);
+    bi.leaf = (unsigned char *const *)(W.base + L.leafs);
+    bi.item_units = B.item_begin.back();
     bi.item_begin = (const int64_t *)(W.base + L.item_begin);
+    bi.leaf_total = B.leaf_begin.back();
+    bi.leaf_begin = (const int64_t *)(W.base + L.leaf_begin);
     memcpy(host.data() + L.index, &bi, sizeof(bi));
     memcpy(host.data() + L.row_begin, B.row_begin.data(), (size_t)(count + 1) * 8);
     memcpy(host.data() + L.unit_begin, B.unit_begin.data(), (size_t)(count + 1) * 8);
-    if (!B.item_begin.empty())
-        memcpy(host.data() + L.item_begin, B.item_begin.data(), B.item_begin.size() * 8);
+    memcpy(host.data() + L.item_begin, B.item_begin.data(), B.item_begin.size() * 8);
+    memcpy(host.data() + L.leaf_begin, B.leaf_begin.data(), B.leaf_begin.size() * 8);
     for (int q = 0; q < count; ++q) {
         const ImpactDesc *d = W.desc(q);
-        unsigned char *r = W.base + L.rec[q];
+        unsigned char *r = W.base + L.rec[q], *i = W.base + L.item[q], *f = W.base + L.leaf[q],
+                      *v = W.base + L.term[q];
         memcpy(host.data() + L.descs + 8 * (size_t)q, &d, 8);
         memcpy(host.data() + L.recs + 8 * (size_t)q, &r, 8);
+        memcpy(host.data() + L.items + 8 * (size_t)q, &i, 8);
+        memcpy(host.data() + L.leafs + 8 * (size_t)q, &f, 8);
+        memcpy(host.data() + L.termps + 8 * (size_t)q, &v, 8);
         impact::pack_tables(B.plans[q], host.data() + L.tables[q], W.base + L.tables[q],
                             B.images[q]);
     }
@@ -370,7 +390,7 @@ cudaError_t walk_pass(const Batch &B, const Work &W, int mode, int warps,
         if (e == cudaSuccess)
             e = impact::launch_walk_fp32(W.index(), r0, std::min(B.rows, r0 + step),
                                          B.rec_max, B.work_max, warps, mode, o,
-                                         mode == WALK_FUSED ? W.lb() : nullptr, B.tune.faults, st);
+                                         W.lb(), B.tune.faults, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -391,6 +411,13 @@ cudaError_t walk_pass64(const Batch &B, const Work &W, bool emit, const impact::
     return cudaSuccess;
 }
 
+// FP32 row records.
+cudaError_t setup_pass(const Batch &B, const Work &W, cudaStream_t st)
+{
+    return impact::launch_setup_fp32(W.index(), B.units, B.shared32 > 0, B.shared32 < B.count(),
+                                     B.item_begin.back(), W.status(), st);
+}
+
 // count pass: row_ptr (row pointers and the total), sink_lo, sink_up, trunc,
 // row_flags: per-row counts, then the scan. FP64 builds whose tables are too
 // large for the walk (ImpactDesc.walk64) are counted by the per-pair kernel.
@@ -401,9 +428,10 @@ impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cu
     impact::RowOutputs o{out->row_ptr, nullptr, nullptr, nullptr, out->sink_lo, out->sink_up,
                          out->trunc, out->row_flags, W.status(), -1, B.rows};
     if (B.prec == PREC_FP32_SOUND) {
-        CK(impact::launch_setup_fp32(W.index(), B.units, W.status(), out->sink_lo, out->sink_up,
-                                     out->trunc, st));
+        CK(setup_pass(B, W, st));
+        CK(impact::launch_leaf_fp32(W.index(), B.leaf_begin.back(), B.leaf_smem, st));
         CK(walk_pass(B, W, WALK_COUNT, B.tune.count_warps, o, W.counter(), chunk_rows, st));
+        CK(impact::launch_terms_fp32(W.index(), B.rows, W.lb(), B.tune.faults.fault_row, o, st));
         CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st));
         return IMPACT_OK;
     }
@@ -428,8 +456,7 @@ impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int
                          nullptr, W.status(), capacity, B.rows};
     if (B.prec == PREC_FP32_SOUND) {
         if (!records_ready)   // rebuild the records; the row outputs stay as counted
-            CK(impact::launch_setup_fp32(W.index(), B.units, W.status(), nullptr, nullptr,
-                                         nullptr, st));
+            CK(setup_pass(B, W, st));
         CK(walk_pass(B, W, WALK_EMIT, B.tune.emit_warps, o, W.counter() + 1, chunk_rows, st));
     } else {
         if (B.any64) {
@@ -459,12 +486,12 @@ impact_status run_fused(const Batch &B, const Work &W, const impact_csr *out, in
         return run_emit(B, W, out, capacity, true, st, chunk_rows);
     }
     CK(cudaMemsetAsync(W.status(), 0, 64, st));
-    CK(impact::launch_setup_fp32(W.index(), B.units, W.status(), out->sink_lo, out->sink_up,
-                                 out->trunc, st));
+    CK(setup_pass(B, W, st));
     if (B.rows > 0) CK(cudaMemsetAsync(W.lb(), 0, (size_t)B.rows * 8, st));
     else CK(cudaMemsetAsync(out->row_ptr, 0, 8, st));
     impact::RowOutputs o{out->row_ptr, out->col, out->lo, out->up, out->sink_lo, out->sink_up,
                          out->trunc, out->row_flags, W.status(), capacity, B.rows};
+    CK(impact::launch_terms_fp32(W.index(), B.rows, nullptr, -1, o, st));
     CK(walk_pass(B, W, WALK_FUSED, B.tune.count_warps, o, W.counter(), chunk_rows, st));
     return IMPACT_OK;
 }

@@ -37,9 +37,9 @@ struct ImpactDim {
     int64_t item_mul[IMPACT_MAX_DIM];   // 0: the image does not read dimension k
     int n_classes;        // classes of inputs
     int w64;              // FP64: targets an item's table holds (largest window)
-    int group;            // FP64: lanes that make one item (8, 16 or 32)
-    int item_stride;      // FP64: bytes of one item
-    int64_t item_off;     // FP64: bytes of the build's items before this dimension's
+    int group;            // lanes that make one item (FP64: 8, 16 or 32; FP32: 1)
+    int item_stride;      // bytes of one item
+    int64_t item_off;     // bytes of the build's items before this dimension's
 };
 
 // Kinds (match impact_kind) and precisions (match impact_precision).
@@ -81,6 +81,17 @@ struct ImpactDesc {
     const double *images;     // IMAGES: [rows][n][2], caller's device array
     int n_max;                // max N_d
     int walk64;               // FP64: built by the item tables and the tree walk
+    // FP32 sound: rows gather their windows from the items (share32), and the
+    // count pass reads one sorted leaf table per distinct image of the last two
+    // dimensions together (leaf_shared), numbered like the items
+    int share32;
+    int leaf_shared;
+    int64_t leaf_items;
+    int64_t leaf_mul[IMPACT_MAX_DIM];
+    int leaf_classes;
+    int leaf_stride;          // bytes of one leaf table
+    const int *leaf_cls;      // [n_inputs]
+    const int *leaf_rep;      // [n_inputs]
     const int *cls;           // [n][n_inputs] class of an input in dimension d
     const int *cls_rep;       // [n][n_inputs] an input of each class
 
@@ -118,8 +129,13 @@ struct BatchIndex {
     const int64_t *row_begin;           // [count + 1]
     const int64_t *unit_begin;          // [count + 1]
     const ImpactDesc *const *desc;      // [count] device descriptors
-    unsigned char *const *rec;          // [count] FP32: per-row records, FP64: items
-    int64_t item_units;                 // FP64: warps' worth of items, all builds
+    unsigned char *const *rec;          // [count] FP32 per-row records
+    unsigned char *const *items;        // [count] item tables
+    unsigned char *const *leaf;         // [count] FP32 leaf tables
+    unsigned char *const *terms;        // [count] FP32: (row, dimension) numbers of the row terms
+    int64_t item_units;                 // warps' worth of items, all builds
     const int64_t *item_begin;          // [count * IMPACT_MAX_DIM + 1] first unit per dimension
+    int64_t leaf_total;                 // leaf tables, all builds
+    const int64_t *leaf_begin;          // [count + 1] first leaf table of each build
     unsigned long long *next_row;       // [2] row counters of the count / emit walk
 };

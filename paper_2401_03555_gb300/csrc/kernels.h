@@ -85,19 +85,17 @@ cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_
                            double *r_lo, double *r_up, double *a_lo, double *a_up,
                            cudaStream_t stream);
 
-// FP32-sound path (walk_fp32.cu). The setup kernel writes one record per
-// row (record_stride bytes: per-dimension entries, then the window tables)
-// and, when the row arrays are given, the sink bounds and the mass outside
-// the window box; the walk kernels read the records. A walk launch covers
+// FP32-sound path (walk_fp32.cu). The setup kernels write one record per
+// row (record_stride bytes: per-dimension entries, then the window tables);
+// the walk kernels read the records. A walk launch covers
 // the global rows [row_begin, row_end) of a batch (the pass's row counter
 // zeroed before each launch; launches of one pass in row order on one
 // stream). A warp's shared memory holds two record buffers of `rec_max`
 // bytes (the largest record_stride of the batch: the row being walked and the
 // next one, prefetched) and work space: `work_max` = the largest
-// walk_work_bytes of the batch for the emit pass [0] and the passes that
-// count [1]; `lb`: one
-// 8-byte look-back word per row, zeroed before the first launch of a FUSED
-// pass. COUNT writes per-row counts (a scan makes them row pointers), FUSED
+// walk_work_bytes of the batch per mode; `lb`: 16 bytes per row, for FUSED
+// one 8-byte look-back word per row, zeroed before the first launch of the
+// pass, for COUNT the row's sums. COUNT writes per-row counts (a scan makes them row pointers), FUSED
 // the row pointers themselves.
 enum { WALK_COUNT = 0, WALK_EMIT = 1, WALK_FUSED = 2 };
 struct WalkFaults {
@@ -108,11 +106,23 @@ struct WalkFaults {
 };
 int64_t record_stride(int n, int tsum_cap);
 int walk_core_bytes(int n, int tsum_cap, int leaf_cap);   // both buffers and the work space
-int walk_work_bytes(int n, int leaf_cap, bool count);
-cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, uint32_t *status,
-                              double *sink_lo, double *sink_up, double *trunc, cudaStream_t stream);
+int walk_work_bytes(const ImpactDesc &D, int mode);
+// The planner calls size_items32 (item and leaf table layout, whether a build
+// uses them); `shared` / `own`: some build of the batch does / does not.
+void size_items32(ImpactDesc &D, int64_t &item_bytes, int64_t &leaf_bytes);
+cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, bool shared, bool own,
+                              int64_t item_units, uint32_t *status, cudaStream_t stream);
+// FP64 row terms of every row from its windows' numbers; acc: the sums that a
+// COUNT pass left in `lb` (null: only the sinks and the mass outside).
+cudaError_t launch_terms_fp32(const BatchIndex *d_index, int64_t rows, const void *acc,
+                              int64_t fault_row, const RowOutputs &o, cudaStream_t stream);
+// Leaf tables of the builds that share them (after the items, before a count
+// pass); leaf_smem: the largest leaf32_bytes of the batch.
+int leaf32_bytes(const ImpactDesc &D);
+cudaError_t launch_leaf_fp32(const BatchIndex *d_index, int64_t tables, int leaf_smem,
+                             cudaStream_t stream);
 cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64_t row_end,
-                             int rec_max, const int work_max[2], int warps, int mode,
+                             int rec_max, const int work_max[3], int warps, int mode,
                              const RowOutputs &o,
                              unsigned long long *lb, const WalkFaults &f, cudaStream_t stream);
 // FP64 path (walk_fp64.cu): item tables, per-row terms, the walk (launches of

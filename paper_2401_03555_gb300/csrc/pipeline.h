@@ -22,11 +22,13 @@ struct Batch {
     int64_t rows = 0, units = 0, nnz_bound = 0;
     int prec = 0;
     int rec_max = 0;                      // FP32 walk: largest record of the batch
-    int work_max[2] = {0, 0};             // FP32 walk: largest work space, emit / count
+    int work_max[3] = {0, 0, 0};          // FP32 walk: largest work space per mode
     bool walks = true;                    // false: only the tables are used (no walk scratch)
     int64_t extra = 0;                    // bytes of the call's own scratch
     int any64 = 0, warp64 = 0;            // FP64 walk: builds on it, largest warp memory
-    std::vector<int64_t> item_begin;      // FP64 walk: [count * IMPACT_MAX_DIM + 1]
+    int shared32 = 0, leaf_smem = 0;      // FP32: builds with shared windows, leaf kernel memory
+    std::vector<int64_t> item_begin;      // [count * IMPACT_MAX_DIM + 1] first item unit
+    std::vector<int64_t> leaf_begin;      // [count + 1] first leaf table
     Tuning tune;
     uint64_t hash = 0;
     int count() const { return (int)plans.size(); }
@@ -38,12 +40,15 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
 // Offsets (bytes, 256-aligned) of everything in the device workspace.
 struct BatchLayout {
     size_t index = 0, row_begin = 0, unit_begin = 0, descs = 0, recs = 0, item_begin = 0;
+    size_t items = 0, leafs = 0, termps = 0, leaf_begin = 0;
     std::vector<size_t> tables;            // per build: its descriptor and tables
     std::vector<impact::TableLayout> tl;
     size_t upload_end = 0;                 // [0, upload_end) is copied from the host
     size_t status = 0, counter = 0, scan = 0;
-    size_t lb = 0;                         // FP32: one look-back word per row
-    std::vector<size_t> rec;               // per build: FP32 per-row records, FP64 items
+    size_t lb = 0;                         // FP32: 16 bytes per row (look-back word, or sums)
+    std::vector<size_t> rec;               // per build: FP32 per-row records
+    std::vector<size_t> item, leaf;        // per build: item tables, FP32 leaf tables
+    std::vector<size_t> term;              // per build: FP32 (row, dimension) numbers
     size_t extra = 0;                      // the call's own scratch
     size_t total = 0;
 };

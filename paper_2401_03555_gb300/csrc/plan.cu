@@ -127,6 +127,33 @@ void number_items(const impact_system *sys, const impact_inputs *inputs, Plan &P
             g.n_items = D.rows;
         }
     }
+    // the last two dimensions together: what either reads, and the pairs of
+    // their input classes
+    D.leaf_items = D.rows;
+    D.leaf_classes = 1;
+    if (n < 2 || D.kind == KIND_IMAGES) return;
+    const int *cm = &P.cls[(size_t)(n - 2) * ni], *cl = &P.cls[(size_t)(n - 1) * ni];
+    std::vector<int> leaf_cls((size_t)ni), leaf_rep((size_t)ni, 0);
+    for (int j = 0; j < ni; ++j) order[j] = j;
+    std::sort(order.begin(), order.end(), [&](int a, int b) {
+        return cm[a] != cm[b] ? cm[a] < cm[b] : cl[a] != cl[b] ? cl[a] < cl[b] : a < b;
+    });
+    int classes = 0;
+    for (int i = 0; i < ni; ++i) {
+        const int a = i > 0 ? order[i - 1] : 0, b = order[i];
+        if (i == 0 || cm[a] != cm[b] || cl[a] != cl[b]) leaf_rep[classes++] = b;
+        leaf_cls[b] = classes - 1;
+    }
+    D.leaf_classes = classes;
+    int64_t c = classes;
+    for (int k = n - 1; k >= 0; --k) {
+        const bool reads = D.dim[n - 2].item_mul[k] != 0 || D.dim[n - 1].item_mul[k] != 0;
+        D.leaf_mul[k] = reads ? c : 0;
+        if (reads) c *= D.dim[k].N;
+    }
+    D.leaf_items = c;
+    P.cls.insert(P.cls.end(), leaf_cls.begin(), leaf_cls.end());
+    P.cls_rep.insert(P.cls_rep.end(), leaf_rep.begin(), leaf_rep.end());
 }
 
 uint64_t fnv(uint64_t h, const void *p, size_t bytes)
@@ -419,15 +446,15 @@ impact_status make_plan(const impact_system *sys, const impact_grid *grid,
                         "the per-row windows need " + std::to_string(tsum) +
                             " factor entries, more than one warp's shared memory holds: "
                             "raise the cutoff or use fewer cells");
-        D.tsum_cap = (int)tsum;
         D.leaf_cap = leaf_cap;
+        int ro = 0;
+        for (int d = 0; d < n; ++d) {   // tables start 16-byte aligned
+            D.dim[d].rec_off = ro;
+            ro += (D.dim[d].wcap + 1) & ~1;
+        }
+        D.tsum_cap = ro;
         D.walk_core = impact::walk_core_bytes(n, D.tsum_cap, D.leaf_cap);
         D.rec_stride = (int)impact::record_stride(n, D.tsum_cap);
-        int ro = 0;
-        for (int d = 0; d < n; ++d) {
-            D.dim[d].rec_off = ro;
-            ro += D.dim[d].wcap;
-        }
         // tables in erf units (x / (sigma sqrt2)) as FP32 pairs, and in cells
         for (int d = 0; d < n; ++d) {
             const ImpactDim &g = D.dim[d];
@@ -476,6 +503,7 @@ impact_status make_plan(const impact_system *sys, const impact_grid *grid,
         }
     }
     number_items(sys, inputs, P);
+    if (precision == IMPACT_FP32_SOUND) impact::size_items32(D, P.item_bytes, P.leaf_bytes);
     if (precision == IMPACT_FP64_PLAIN) P.item_bytes = impact::size_items64(D, P.nnz_bound);
     // identity of the arguments, for reusing a caller's workspace
     uint64_t h = 1469598103934665603ull;
@@ -529,6 +557,8 @@ void pack_tables(const Plan &P, unsigned char *host, unsigned char *dev_base,
     D.omm = (const float *)dp(L.omm, P.omm.size());
     D.cls = (const int *)dp(L.cls, P.cls.size());
     D.cls_rep = (const int *)dp(L.cls_rep, P.cls_rep.size());
+    D.leaf_cls = D.cls + (size_t)D.n * D.n_inputs;
+    D.leaf_rep = D.cls_rep + (size_t)D.n * D.n_inputs;
     D.images = dev_images;
     memcpy(host + L.desc, &D, sizeof(D));
     auto put = [&](size_t off, const void *src, size_t bytes) {

@@ -34,7 +34,8 @@ struct Plan {
     std::vector<float> mu_lo, mu_hi, mo, um, omm;
     // distinct images (impact_desc.h): input classes per dimension
     std::vector<int> cls, cls_rep;
-    int64_t item_bytes = 0;   // FP64: the build's item tables
+    int64_t item_bytes = 0;   // the build's item tables
+    int64_t leaf_bytes = 0;   // FP32: its leaf tables
     int64_t rows = 0;
     int64_t nnz_bound = 0;
     int table_need = 0;   // upper bound of the staged entries per row (-1: unknown)

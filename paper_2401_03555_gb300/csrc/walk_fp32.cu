@@ -1,19 +1,23 @@
 // walk_fp32.cu -- FP32-sound construction (Def. 3.1 with outward rounding,
-// Sec. 4.4 cutoff, Remark 4.1 sink) in two steps.
+// Sec. 4.4 cutoff, Remark 4.1 sink).
 //
-//   setup_fp32  one lane per (row, dimension), the 32/n rows of a warp
-//               aligned to it (Alg. 2: rows are independent). From the
-//               interval image of the source cell the lane finds the window
-//               of target cells that can pass the cutoff, evaluates erf/erfc
-//               once per window edge at the image's lower and upper end, and
-//               writes the window's factor table to the row's record: U[t] >=
-//               the largest Gaussian mass of target t over the image (T_max of
-//               Def. 3.1 relaxed to the image box) and L[t] <= the smallest
-//               (T_min), trimmed to the targets that pass on their own. The
-//               lanes of a row then exchange their window maxima and sums by
-//               shuffles: each finishes its dimension's pruning threshold, and
-//               the lane of dimension 0 writes the row's sink bounds and the
-//               mass of the targets outside the window box (FP64, outward).
+//   setup       From the interval image of the source cell: the window of
+//               target cells that can pass the cutoff, erf/erfc once per window
+//               edge at the image's lower and upper end, and the window's factor
+//               table: U[t] >= the largest Gaussian mass of target t over the
+//               image (T_max of Def. 3.1 relaxed to the image box) and L[t] <= the
+//               smallest (T_min), trimmed to the targets that pass on their own.
+//               Rows that read the same coordinates and input offset share an
+//               image (impact_desc.h): items_fp32 makes each window once and
+//               rows_fp32 gathers a row's into its record; systems whose images
+//               are distinct make them per row (setup_fp32, one lane per row and
+//               dimension). The lanes of a row exchange their window maxima and
+//               sums by shuffles for the pruning thresholds.
+//   leaf_fp32   the sorted leaf tables (below) of the distinct images of the
+//               last two dimensions, for the count pass.
+//   terms_fp32  after the count pass, one thread per row: sink bounds, mass of
+//               the targets outside the window box, truncated mass and row
+//               checks (FP64, outward).
 //   walk_fp32   one warp per row, persistent (rows from an atomic counter in
 //               ascending order). It walks the prefix tree of target cells
 //               level by level in C order over the first n - 2 dimensions: a
@@ -29,7 +33,8 @@
 //               RD product of the lower factors), so a pair's bound is one more
 //               product RU(P B[a, b]). The count pass finds how many entries of
 //               B pass under each parent by a binary search in B sorted by
-//               value, with prefix sums for the row sums; the emit pass tests
+//               value, with prefix sums for the row sums (B from the row's shared
+//               leaf table, else sorted by the warp); the emit pass tests
 //               every entry of B under each parent, one lane each, and stores
 //               the kept pairs warp-contiguously.
 //
@@ -53,17 +58,16 @@
 #include "../../include/impact.h"
 #include "impact_desc.h"
 #include "kernels.h"
+#include "rowmath.cuh"
 #include "sound_fp32.cuh"
 
 namespace {
 
+using rowmath::fastdiv;
+using rowmath::find_problem;
+
 constexpr float kTwoM44 = 5.6843419e-14f;       // 2^-44
 constexpr float kGrow18 = 1.0000038147f;        // 1 + 2^-18
-
-__device__ __forceinline__ uint32_t fastdiv(uint32_t x, uint32_t m, int s)
-{
-    return (__umulhi(x, m) + x) >> s;   // exact for x < 2^31 (host-built m, s)
-}
 
 __device__ __forceinline__ unsigned lanemask_lt()
 {
@@ -102,18 +106,6 @@ __device__ __forceinline__ float threshold(float c, float r)
 {
     if (!(r > 0.0f)) return INFINITY;
     return fsucc(__fdiv_rd(fpred(c), r));
-}
-
-// Problem of a batch that owns global row x: begin[q] <= x < begin[q + 1].
-__device__ __forceinline__ int find_problem(const int64_t *__restrict__ begin, int count,
-                                            int64_t x)
-{
-    int lo = 0, hi = count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (begin[mid] <= x) lo = mid; else hi = mid - 1;
-    }
-    return lo;
 }
 
 // Edge point: alpha = (E - m)/(sigma sqrt2) at one image end, its half-width
@@ -157,32 +149,9 @@ __device__ __forceinline__ EdgePt edge_at(const Win &h, int k, bool hi_end)
 // outside lies more than delta beyond the image), and rho = (E_a - m) /
 // (sigma sqrt2) at both image ends as FP32 pairs. False if the window
 // exceeds the planner's bound wcap.
-__device__ bool dim_window(const ImpactDesc &D, int64_t row, int d, Win &h)
+__device__ bool dim_window(const ImpactDesc &D, int64_t row, const int *idx, int j, int d, Win &h)
 {
     const int n = D.n;
-    int64_t cell;
-    int j;
-    if (row < ((int64_t)1 << 31)) {
-        uint32_t c = fastdiv((uint32_t)row, D.inp_div_m, D.inp_div_s);
-        cell = c;
-        j = (int)((uint32_t)row - c * (uint32_t)D.n_inputs);
-    } else {
-        cell = row / D.n_inputs;
-        j = (int)(row - cell * D.n_inputs);
-    }
-    int idx[IMPACT_MAX_DIM];
-    {
-        uint32_t c = (uint32_t)cell;
-#pragma unroll
-        for (int k = IMPACT_MAX_DIM - 1; k >= 0; --k) {
-            idx[k] = 0;
-            if (k < n) {
-                uint32_t q = fastdiv(c, D.dim[k].div_m, D.dim[k].div_s);
-                idx[k] = (int)(c - q * (uint32_t)D.dim[k].N);
-                c = q;
-            }
-        }
-    }
     int my_idx = 0, idx2 = idx[2 < IMPACT_MAX_DIM ? 2 : 0];
 #pragma unroll
     for (int k = 0; k < IMPACT_MAX_DIM; ++k)
@@ -276,8 +245,8 @@ __device__ bool dim_window(const ImpactDesc &D, int64_t row, int d, Win &h)
 // setup: one record per row
 // ---------------------------------------------------------------------------
 
-// Per (row, dimension) entry of a row record. The record is RecDim[n], then
-// the window tables, (U, L) pairs, dimension d's at entry rec_off[d].
+// Per (row, dimension) entry of a row record. The record is RecDim[n], RecRow,
+// then the window tables, (U, L) pairs, dimension d's at entry rec_off[d].
 struct RecDim {
     int tw;          // trimmed width: targets first..last that pass on their own
     int tb;          // table entry of the first trimmed target
@@ -292,6 +261,32 @@ struct RecDim {
 };
 static_assert(sizeof(RecDim) == 32, "RecDim layout");
 
+// Per-row entry of the record, between the dimensions' entries and the tables.
+struct RecRow {
+    int64_t leaf;    // the row's leaf table (builds that share them)
+    int64_t pad;
+};
+
+__device__ __forceinline__ RecRow *rec_row(unsigned char *rec, int n)
+{
+    return reinterpret_cast<RecRow *>(rec + sizeof(RecDim) * n);
+}
+__device__ __forceinline__ float2 *rec_table(unsigned char *rec, int n)
+{
+    return reinterpret_cast<float2 *>(rec + sizeof(RecDim) * n + sizeof(RecRow));
+}
+
+// Leaf table of the last two dimensions that a row with these digits shares.
+__device__ __forceinline__ int64_t leaf_of_row(const ImpactDesc &D, const int *idx, int j)
+{
+    if (!D.leaf_shared) return 0;
+    int64_t c = D.leaf_cls[j];
+#pragma unroll
+    for (int k = 0; k < IMPACT_MAX_DIM; ++k)
+        if (k < D.n) c += (int64_t)idx[k] * D.leaf_mul[k];
+    return c;
+}
+
 // Everything of one (row, dimension) that needs no other dimension.
 struct DimOut {
     int tw = 0, f0 = 0, a = 0;
@@ -300,16 +295,18 @@ struct DimOut {
     float O = 0.0f;     // mass outside the trimmed window (rounded up)
     float qlo = 0.0f, qhi = 0.0f;   // out-of-domain mass bounds
 };
+static_assert(sizeof(DimOut) == 32, "DimOut layout");
 
 // The window of dimension d of a row and its factor table, written to `ul`
 // (the record's entries of dimension d): U[k], L[k] for target a + k from the
 // tails of its two edges at both image ends (neighbouring targets share an
 // edge), then the trimmed window, its sums and the out-of-domain bounds.
-__device__ DimOut setup_dim(const ImpactDesc &D, int64_t row, int d, float2 *ul, uint32_t *status)
+__device__ DimOut setup_dim(const ImpactDesc &D, int64_t row, const int *idx, int j, int d,
+                            float2 *ul, uint32_t *status)
 {
     DimOut o;
     Win h;
-    if (!dim_window(D, row, d, h)) {
+    if (!dim_window(D, row, idx, j, d, h)) {
         atomicOr(status, IMPACT_STATUS_TABLE_OVERFLOW);
         return o;
     }
@@ -381,19 +378,122 @@ __device__ DimOut setup_dim(const ImpactDesc &D, int64_t row, int d, float2 *ul,
     return o;
 }
 
-// setup_fp32: one warp per 32/n rows of one build, one lane per (row,
-// dimension). Each lane builds its dimension's table; the lanes of a row then
-// exchange their maxima and sums by shuffles and each finishes its entry of
-// the record: the pruning threshold (a child t of a node with product P
-// survives iff RU(RU(P U[t]) R') >= cutoff, R' the product of the later
-// dimensions' largest factors grown by 2^-18 to cover the rounding of the
-// rest of the chain; cp is the least such child product). The lane of
-// dimension 0 also writes the row's sink bounds and the mass of the targets
-// outside the window box (FP64, outward rounding), unless the row outputs
-// are null (records rebuilt for an emit pass).
+// What one lane of a row's dimensions finishes with the row's others (the
+// lanes of a row are `base` .. `base + n - 1`): its record entry with the
+// pruning threshold (a child t of a node with product P survives iff
+// RU(RU(P U[t]) R') >= cutoff, R' the product of the later dimensions' largest
+// factors grown by 2^-18 to cover the rounding of the rest of the chain; cp is
+// the least such child product).
+__device__ __forceinline__ void finish_dim(const ImpactDesc &D, const DimOut &o, int d, int base,
+                                           bool act, unsigned char *rr)
+{
+    const int n = D.n;
+    float R = 1.0f, SR = 1.0f;
+#pragma unroll
+    for (int k = 0; k < IMPACT_MAX_DIM; ++k) {
+        if (k < n) {   // n is the same for the whole warp
+            const int src = (base + k) & 31;
+            const float Mk = __shfl_sync(0xffffffffu, o.M, src);
+            const float SWk = __shfl_sync(0xffffffffu, o.SW, src);
+            if (k > d) {
+                R = __fmul_ru(R, Mk);
+                SR = __fmul_ru(SR, SWk);
+            }
+        }
+    }
+    if (!act) return;
+    const float cut = D.cutoff32;
+    RecDim rd;
+    rd.tw = o.tw;
+    rd.tb = D.dim[d].rec_off + o.f0;
+    rd.cb = (o.a + o.f0) * D.dim[d].stride;
+    rd.magic = o.tw > 1 ? 0xffffffffu / (unsigned)o.tw + 1u : 0u;   // ceil(2^32 / tw)
+    rd.cp = 0.0f;
+    if (cut > 0.0f) rd.cp = (d == n - 1) ? cut : threshold(cut, __fmul_ru(R, kGrow18));
+    rd.SR = SR;
+    rd.stride = D.dim[d].stride;
+    rd.lay = (o.tw >= 1 && o.tw <= 32)
+                 ? ((32 / o.tw) | (((IMPACT_WALK_CAP / o.tw) * o.tw) << 16)) : 0;
+    reinterpret_cast<RecDim *>(rr)[d] = rd;
+}
+
+// The numbers of one (row, dimension) that the row terms need.
+__device__ __forceinline__ float4 term_of(const DimOut &o)
+{
+    return make_float4(o.SW, o.O, o.qlo, o.qhi);
+}
+
+// terms_fp32: the FP64 row terms, one thread per row: sink bounds and the mass
+// of the targets outside the window box, with outward rounding, and after a
+// count pass (acc: its FP32 sums per row: dropped mass, upper and lower bounds
+// of the kept pairs) the truncated mass and the row checks of Def. 3.1.
+// FP64 issues two lanes per clock and SM here, whatever share of a warp's
+// lanes is active: in the setup (n lanes per row) and at the end of a row's
+// walk (one lane) the same operations took 1.1 ms of the 11^5 room's 12.
+__global__ void __launch_bounds__(256)
+terms_fp32(const BatchIndex *__restrict__ B, const float4 *__restrict__ acc, int64_t fault_row,
+           double *__restrict__ sink_lo, double *__restrict__ sink_up, double *__restrict__ trunc,
+           uint32_t *__restrict__ flags, uint32_t *__restrict__ status)
+{
+    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < B->rows;
+         row += (int64_t)gridDim.x * blockDim.x) {
+        const int q = find_problem(B->row_begin, B->count, row);
+        const ImpactDesc &D = *B->desc[q];
+        const int n = D.n;
+        const int64_t rl = row - B->row_begin[q];
+        int idx[IMPACT_MAX_DIM], j = 0;
+        if (D.share32) rowmath::decode_row(D, rl, idx, j);
+        const float4 *own = reinterpret_cast<const float4 *>(B->terms[q]) + rl * n;
+        double pin_up = 1.0, pin_dn = 1.0, out = 0.0, pre = 1.0;
+#pragma unroll
+        for (int k = 0; k < IMPACT_MAX_DIM; ++k) {
+            if (k < n) {
+                float4 v;
+                if (D.share32) {
+                    const ImpactDim &g = D.dim[k];
+                    v = term_of(*reinterpret_cast<const DimOut *>(
+                        B->items[q] + g.item_off +
+                        rowmath::item_of(D, rl, idx, j, k) * g.item_stride));
+                } else {
+                    v = own[k];
+                }
+                const double SWk = (double)v.x, Ok = (double)v.y;
+                // sink: 1 - prod_k (1 - Q_k)
+                pin_up = __dmul_ru(pin_up, __dsub_ru(1.0, (double)v.z));
+                pin_dn = __dmul_rd(pin_dn, __dsub_rd(1.0, (double)v.w));
+                // mass outside the window box, partitioned by the first
+                // dimension that leaves its window:
+                // sum_k prod_{i<k} SW_i * O_k * prod_{i>k} (SW_i + O_i)
+                out = __dadd_ru(__dmul_ru(out, __dadd_ru(SWk, Ok)), __dmul_ru(pre, Ok));
+                pre = __dmul_ru(pre, SWk);
+            }
+        }
+        const double sl = fmax(__dsub_rd(1.0, pin_up), 0.0), su = fmin(__dsub_ru(1.0, pin_dn), 1.0);
+        double tr = out;
+        if (acc) {
+            const float4 a = acc[row];
+            tr = __dadd_ru(out, (double)a.x);
+            if (flags) {
+                const double lo_sum = row == fault_row ? 2.0 : (double)a.z;
+                uint32_t f = 0;
+                if (__dadd_rd(lo_sum, sl) > 1.0) f |= IMPACT_ROW_LO_SUM_ABOVE_ONE;
+                if (__dadd_ru(__dadd_ru((double)a.y, su), tr) < 1.0) f |= IMPACT_ROW_UP_SUM_BELOW_ONE;
+                flags[row] = f;
+                if (f) atomicOr(status, IMPACT_STATUS_UNSOUND);
+            }
+        }
+        sink_lo[row] = sl;
+        sink_up[row] = su;
+        trunc[row] = tr;
+    }
+}
+
+// setup_fp32 (builds whose images are nearly all distinct): one warp per 32/n
+// rows of one build, one lane per (row, dimension). Each lane builds its
+// dimension's table; the lanes of a row then exchange their maxima and sums
+// by shuffles (finish_dim).
 __global__ void __launch_bounds__(256, 3)
-setup_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status,
-           double *__restrict__ sink_lo, double *__restrict__ sink_up, double *__restrict__ trunc)
+setup_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -401,6 +501,7 @@ setup_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status,
     for (int64_t u = warp0; u < B->units; u += nwarps) {
         const int q = find_problem(B->unit_begin, B->count, u);
         const ImpactDesc &D = *B->desc[q];
+        if (D.share32) continue;
         const int n = D.n;
         const int rpw = 32 / n;
         const int slot = lane / n, d = lane - slot * n;
@@ -410,56 +511,89 @@ setup_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status,
         unsigned char *rr = act ? B->rec[q] + rl * (int64_t)D.rec_stride : nullptr;
         DimOut o;
         if (act) {
-            float2 *ul = reinterpret_cast<float2 *>(rr + 32 * n) + D.dim[d].rec_off;
-            o = setup_dim(D, rl, d, ul, status);
+            int idx[IMPACT_MAX_DIM], j;
+            rowmath::decode_row(D, rl, idx, j);
+            o = setup_dim(D, rl, idx, j, d, rec_table(rr, n) + D.dim[d].rec_off, status);
+            reinterpret_cast<float4 *>(B->terms[q])[rl * n + d] = term_of(o);
         }
-        // the row's other dimensions, in order k = 0..n-1 (lanes base + k)
-        const int base = slot * n;
-        float R = 1.0f, SR = 1.0f;
-        double pin_up = 1.0, pin_dn = 1.0, acc = 0.0, pre = 1.0;
+        finish_dim(D, o, d, slot * n, act, rr);
+    }
+}
+
+// items_fp32: the window and factor table of every distinct image
+// (impact_desc.h), one lane each: DimOut, then the window's (U, L) pairs.
+__device__ __forceinline__ float2 *item_table(unsigned char *it)
+{
+    return reinterpret_cast<float2 *>(it + sizeof(DimOut));
+}
+
+__global__ void __launch_bounds__(128)
+items_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
+{
+    const int64_t total = B->item_units * 32;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int seg = find_problem(B->item_begin, B->count * IMPACT_MAX_DIM, i >> 5);
+        const int q = seg / IMPACT_MAX_DIM, d = seg % IMPACT_MAX_DIM;
+        const ImpactDesc &D = *B->desc[q];
+        const ImpactDim &g = D.dim[d];
+        const int64_t c = i - B->item_begin[seg] * 32;
+        if (c >= g.n_items) continue;
+        int idx[IMPACT_MAX_DIM], j;
+        rowmath::decode_item(D, d, c, idx, j);
+        unsigned char *it = B->items[q] + g.item_off + c * g.item_stride;
+        *reinterpret_cast<DimOut *>(it) = setup_dim(D, c, idx, j, d, item_table(it), status);
+    }
+}
+
+// rows_fp32 (builds that share windows): the lanes of setup_fp32 load their
+// dimension's item instead of making it, and the warp then copies the trimmed
+// tables into the records, eight lanes per table in 16-byte pieces (items and
+// record tables start 16-byte aligned). Bound by the records it writes.
+__global__ void __launch_bounds__(256)
+rows_fp32(const BatchIndex *__restrict__ B)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t u = warp0; u < B->units; u += nwarps) {
+        const int q = find_problem(B->unit_begin, B->count, u);
+        const ImpactDesc &D = *B->desc[q];
+        if (!D.share32) continue;
+        const int n = D.n;
+        const int rpw = 32 / n;
+        const int slot = lane / n, d = lane - slot * n;
+        const int64_t rows_q = B->row_begin[q + 1] - B->row_begin[q];
+        const int64_t rl = (u - B->unit_begin[q]) * rpw + slot;
+        const bool act = slot < rpw && rl < rows_q;
+        unsigned char *rr = act ? B->rec[q] + rl * (int64_t)D.rec_stride : nullptr;
+        DimOut o;
+        const float4 *src = nullptr;
+        float4 *dst = nullptr;
+        int pieces = 0;
+        if (act) {
+            int idx[IMPACT_MAX_DIM], j;
+            rowmath::decode_row(D, rl, idx, j);
+            const ImpactDim &g = D.dim[d];
+            unsigned char *it = B->items[q] + g.item_off +
+                                rowmath::item_of(D, rl, idx, j, d) * g.item_stride;
+            o = *reinterpret_cast<const DimOut *>(it);
+            const int p0 = o.f0 >> 1;
+            pieces = ((o.f0 + o.tw + 1) >> 1) - p0;
+            src = reinterpret_cast<const float4 *>(item_table(it)) + p0;
+            dst = reinterpret_cast<float4 *>(rec_table(rr, n) + g.rec_off) + p0;
+            if (d == 0) rec_row(rr, n)->leaf = leaf_of_row(D, idx, j);
+        }
+        finish_dim(D, o, d, slot * n, act, rr);
 #pragma unroll
-        for (int k = 0; k < IMPACT_MAX_DIM; ++k) {
-            if (k < n) {   // n is the same for the whole warp
-                const int src = (base + k) & 31;
-                const float Mk = __shfl_sync(0xffffffffu, o.M, src);
-                const float SWk = __shfl_sync(0xffffffffu, o.SW, src);
-                const float Ok = __shfl_sync(0xffffffffu, o.O, src);
-                const float qlk = __shfl_sync(0xffffffffu, o.qlo, src);
-                const float qhk = __shfl_sync(0xffffffffu, o.qhi, src);
-                if (k > d) {
-                    R = __fmul_ru(R, Mk);
-                    SR = __fmul_ru(SR, SWk);
-                }
-                // sink: 1 - prod_k (1 - Q_k)
-                pin_up = __dmul_ru(pin_up, __dsub_ru(1.0, (double)qlk));
-                pin_dn = __dmul_rd(pin_dn, __dsub_rd(1.0, (double)qhk));
-                // mass outside the window box, partitioned by the first
-                // dimension that leaves its window:
-                // sum_k prod_{i<k} SW_i * O_k * prod_{i>k} (SW_i + O_i)
-                acc = __dadd_ru(__dmul_ru(acc, __dadd_ru((double)SWk, (double)Ok)),
-                                __dmul_ru(pre, (double)Ok));
-                pre = __dmul_ru(pre, (double)SWk);
-            }
-        }
-        if (!act) continue;
-        const float cut = D.cutoff32;
-        RecDim rd;
-        rd.tw = o.tw;
-        rd.tb = D.dim[d].rec_off + o.f0;
-        rd.cb = (o.a + o.f0) * D.dim[d].stride;
-        rd.magic = o.tw > 1 ? (uint32_t)((0x100000000ull + (unsigned)o.tw - 1) / (unsigned)o.tw) : 0u;
-        rd.cp = 0.0f;
-        if (cut > 0.0f) rd.cp = (d == n - 1) ? cut : threshold(cut, __fmul_ru(R, kGrow18));
-        rd.SR = SR;
-        rd.stride = D.dim[d].stride;
-        rd.lay = (o.tw >= 1 && o.tw <= 32)
-                     ? ((32 / o.tw) | (((IMPACT_WALK_CAP / o.tw) * o.tw) << 16)) : 0;
-        reinterpret_cast<RecDim *>(rr)[d] = rd;
-        if (d == 0 && trunc) {
-            const int64_t row = B->row_begin[q] + rl;   // global row
-            sink_lo[row] = fmax(__dsub_rd(1.0, pin_up), 0.0);
-            sink_up[row] = fmin(__dsub_ru(1.0, pin_dn), 1.0);
-            trunc[row] = acc;
+        for (int p0 = 0; p0 < 32; p0 += 4) {
+            const int p = p0 + (lane >> 3);
+            const float4 *s = reinterpret_cast<const float4 *>(
+                __shfl_sync(0xffffffffu, (unsigned long long)src, p));
+            float4 *t = reinterpret_cast<float4 *>(
+                __shfl_sync(0xffffffffu, (unsigned long long)dst, p));
+            const int k = __shfl_sync(0xffffffffu, pieces, p);
+            for (int i = lane & 7; i < k; i += 8) t[i] = s[i];
         }
     }
 }
@@ -499,7 +633,7 @@ __device__ __forceinline__ WarpMem carve(unsigned char *work, unsigned char *rec
 {
     WarpMem m;
     m.h = reinterpret_cast<RecDim *>(rec);
-    m.ul = reinterpret_cast<float2 *>(rec + 32 * D.n);
+    m.ul = rec_table(rec, D.n);
     m.work = work;
     m.leaf = reinterpret_cast<float *>(m.work + list_bytes(D.n));
     m.leaf_cap = D.leaf_cap;
@@ -557,6 +691,7 @@ struct Leaf {
     uint32_t magic_l;
     bool staged;
     bool sorted;          // count pass: su, sl, pu, pl, sf are built
+    const float4 *shared;    // count pass: the row's shared sorted table, or null
     uint32_t magic_nb;    // ceil(2^32 / nb) when 1 < nb <= 4096, for the emit's flat layout
     float *bu, *bl, *su, *sl, *pu, *pl, *sf;
     int *bc;
@@ -571,6 +706,7 @@ __device__ __forceinline__ Leaf leaf_of(const WarpMem &S, int n)
     f.nb = n >= 2 ? S.h[n - 2].tw * hl.tw : hl.tw;
     f.staged = f.nb <= S.leaf_cap;
     f.sorted = false;
+    f.shared = nullptr;
     f.magic_nb = (f.nb > 1 && f.nb <= 4096)
                      ? (uint32_t)((0x100000000ull + (unsigned)f.nb - 1) / (unsigned)f.nb) : 0u;
     const int c = S.leaf_cap + 1;
@@ -760,6 +896,83 @@ __device__ void leaf_build(const WarpMem &S, int n, Leaf &f, int lane, float cut
     __syncwarp();
 }
 
+// leaf_fp32: the sorted leaf table of every distinct image of the last two
+// dimensions together, one warp each, from their items: {nb, ..} in 16 bytes,
+// then (su, sf, pu, pl) per entry k = 0..nb, su[nb] unused. Tables of more than
+// leaf_cap entries stay empty (their rows test the entries directly).
+struct LeafHead {
+    int nb, pad[3];
+};
+
+__global__ void __launch_bounds__(128)
+leaf_fp32(const BatchIndex *__restrict__ B, int warp_smem)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31;
+    unsigned char *const mine = smem_raw + (size_t)(threadIdx.x >> 5) * warp_smem;
+    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t u = warp0; u < B->leaf_total; u += nwarps) {
+        const int q = find_problem(B->leaf_begin, B->count, u);
+        const ImpactDesc &D = *B->desc[q];
+        const int n = D.n;
+        const int64_t c0 = u - B->leaf_begin[q];
+        int idx[IMPACT_MAX_DIM], j;
+        {
+            int64_t c = c0;
+            j = D.leaf_rep[(int)(c % D.leaf_classes)];
+            c /= D.leaf_classes;
+#pragma unroll
+            for (int k = IMPACT_MAX_DIM - 1; k >= 0; --k) {
+                idx[k] = 0;
+                if (k < n && D.leaf_mul[k] != 0) {
+                    idx[k] = (int)(c % D.dim[k].N);
+                    c /= D.dim[k].N;
+                }
+            }
+        }
+        // the entries of the last two dimensions of a record, in place
+        WarpMem S;
+        S.h = reinterpret_cast<RecDim *>(mine) - (n - 2);
+        S.ul = reinterpret_cast<float2 *>(mine + 2 * sizeof(RecDim));
+        const int wm = (D.dim[n - 2].wcap + 1) & ~1, wl = (D.dim[n - 1].wcap + 1) & ~1;
+        S.work = nullptr;
+        S.leaf = reinterpret_cast<float *>(S.ul + wm + wl);
+        S.leaf_cap = D.leaf_cap;
+        for (int e = 0; e < 2; ++e) {
+            const int d = n - 2 + e;
+            const ImpactDim &g = D.dim[d];
+            unsigned char *it = B->items[q] + g.item_off +
+                                rowmath::item_of(D, 0, idx, j, d) * g.item_stride;
+            const DimOut o = *reinterpret_cast<const DimOut *>(it);
+            if (lane == 0) {
+                RecDim rd;
+                rd.tw = o.tw;
+                rd.tb = e * wm;
+                rd.cb = 0;
+                rd.magic = o.tw > 1
+                               ? (uint32_t)((0x100000000ull + (unsigned)o.tw - 1) / (unsigned)o.tw) : 0u;
+                rd.cp = rd.SR = 0.0f;
+                rd.stride = 0;
+                rd.lay = 0;
+                S.h[d] = rd;
+            }
+            for (int k = lane; k < o.tw; k += 32) S.ul[e * wm + k] = item_table(it)[o.f0 + k];
+        }
+        __syncwarp();
+        unsigned char *out = B->leaf[q] + c0 * D.leaf_stride;
+        Leaf f = leaf_of(S, n);
+        if (f.nb > 0 && f.staged) leaf_build<true>(S, n, f, lane, D.cutoff32);
+        if (lane == 0) reinterpret_cast<LeafHead *>(out)->nb = f.sorted ? f.nb : -1;
+        if (f.sorted) {
+            float4 *to = reinterpret_cast<float4 *>(out + sizeof(LeafHead));
+            for (int k = lane; k <= f.nb; k += 32)
+                to[k] = make_float4(k < f.nb ? f.su[k] : 0.0f, f.sf[k], f.pu[k], f.pl[k]);
+        }
+        __syncwarp();
+    }
+}
+
 // Node of a level list, or the root (P = Pl = 1, column 0).
 struct Node {
     float P, Pl;
@@ -928,6 +1141,28 @@ __device__ void leaf_count(const WarpMem &S, int n, const Leaf &f, const NodeLis
     }
 }
 
+// The same from the row's shared leaf table (in L2; the searches of a step's
+// parents overlap).
+__device__ __forceinline__ void leaf_count_shared(const float4 *__restrict__ tab, int nb,
+                                                  const NodeList &Lp, int npar, int lane,
+                                                  CountAcc &acc, float cut)
+{
+    for (int pi = lane; pi < npar; pi += 32) {
+        const float P = Lp.P[pi], Pl = Lp.Pl[pi];
+        int lo = 0, hi = nb;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (__fmul_ru(P, __ldg(&tab[mid].x)) >= cut) lo = mid + 1;
+            else hi = mid;
+        }
+        const float4 e = __ldg(tab + lo);
+        acc.cnt += lo;
+        acc.sup = __fadd_ru(acc.sup, up_sum(P, e.z, lo));
+        acc.slo = __fadd_rd(acc.slo, lo_sum(Pl, e.w, lo));
+        acc.drop = __fadd_ru(acc.drop, __fmul_ru(P, e.y));
+    }
+}
+
 // Stores that the predicate guards, without a branch around them.
 __device__ __forceinline__ void st_if(bool p, int32_t *a, int32_t v)
 {
@@ -1064,6 +1299,7 @@ __device__ bool walk_row(const WarpMem &S, int n, const Leaf &f, int lane, Count
             if (f.staged) leaf_emit<false, true>(S, n, f, Lp, npar, lane, out, written, cut);
             else leaf_emit<false, false>(S, n, f, Lp, npar, lane, out, written, cut);
         }
+        else if (f.shared) leaf_count_shared(f.shared, f.nb, Lp, npar, lane, acc, cut);
         else leaf_count(S, n, f, Lp, false, npar, lane, acc, cut);
     };
     const int last = n - 3;   // deepest list level
@@ -1212,7 +1448,8 @@ struct WalkArgs {
     int64_t *row_ptr;        // COUNT: per-row counts; FUSED: row pointers; EMIT: read
     int32_t *col;
     float *lo, *up;
-    double *trunc;           // COUNT / FUSED: outside-window mass in, full truncated mass out
+    float4 *acc;             // COUNT: the row's FP32 sums, for terms_fp32
+    double *trunc;           // FUSED: outside-window mass in, full truncated mass out
     double *sink_lo, *sink_up;
     uint32_t *flags;
     uint32_t *status;        // [0] status bits, [1] look-back abort flag
@@ -1317,7 +1554,13 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32) walk_fp32(const Wa
         bool empty = false;
         for (int k = 0; k < n; ++k) empty |= (S.h[k].tw == 0);
         Leaf f = leaf_of(S, n);
-        if (!empty) leaf_build<kCount>(S, n, f, lane, cut);
+        if (MODE == MODE_COUNT && D.leaf_shared && !empty) {
+            const unsigned char *tab =
+                B->leaf[q] + rec_row(wbase + b * A.rec_max, n)->leaf * D.leaf_stride;
+            if (reinterpret_cast<const LeafHead *>(tab)->nb > 0)
+                f.shared = reinterpret_cast<const float4 *>(tab + sizeof(LeafHead));
+        }
+        if (!empty && !f.shared) leaf_build<kCount>(S, n, f, lane, cut);
         bool walked = true;
         int64_t base = 0, len = 0;
         if (kCount) {
@@ -1345,7 +1588,9 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32) walk_fp32(const Wa
             }
             base = prefix;
             len = c;
-            if (lane == 0) {
+            if (MODE == MODE_COUNT) {   // terms_fp32 finishes the row
+                if (lane == 0) A.acc[row] = make_float4(drop, sup, slo, 0.0f);
+            } else if (lane == 0) {
                 // FP64 row terms: the dropped in-window mass joins the mass
                 // outside the window box; then the row checks of Def. 3.1
                 const double tr = __dadd_ru(A.trunc[row], (double)drop);
@@ -1415,31 +1660,98 @@ namespace impact {
 
 int64_t record_stride(int n, int tsum_cap)
 {
-    return ((int64_t)32 * n + (int64_t)8 * tsum_cap + 15) / 16 * 16;
+    return ((int64_t)32 * n + 16 + (int64_t)8 * tsum_cap + 15) / 16 * 16;
 }
 
-int walk_work_bytes(int n, int leaf_cap, bool count)
+int walk_work_bytes(const ImpactDesc &D, int mode)
 {
-    return list_bytes(n) + align16((count ? 32 : 24) * (leaf_cap + 1));
+    // rows with a shared leaf table stage none of their own to count
+    if (mode == MODE_COUNT && D.leaf_shared) return list_bytes(D.n);
+    return list_bytes(D.n) + align16((mode == MODE_EMIT ? 24 : 32) * (D.leaf_cap + 1));
 }
 
 int walk_core_bytes(int n, int tsum_cap, int leaf_cap)
 {
-    const int64_t b = 2 * record_stride(n, tsum_cap) + walk_work_bytes(n, leaf_cap, true);
+    const int64_t b = 2 * record_stride(n, tsum_cap) + list_bytes(n) + align16(32 * (leaf_cap + 1));
     return (int)std::min<int64_t>(b, INT32_MAX / 2);
 }
 
-cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, uint32_t *status,
-                              double *sink_lo, double *sink_up, double *trunc, cudaStream_t stream)
+// Shared windows pay when a window serves three rows or more (below that the
+// items' write and read back cost about what they save): the 11^5 room's 20k
+// windows take 0.014 ms and the gather of 1.45M records 0.37 ms, one setup per
+// row 1.39 ms; building 6^7 0.44 against 1.79 ms. Leaf tables pay when one
+// serves four rows or more and all of them take less than the records: the
+// unicycle 51x51x25 (26k tables of about 200 entries for 1.3M rows) sorted them
+// per row in 11.7 ms of count pass, and takes 0.28 ms for the tables and 1.1 ms
+// for the pass.
+void size_items32(ImpactDesc &D, int64_t &item_bytes, int64_t &leaf_bytes)
+{
+    const int n = D.n;
+    int64_t bytes = 0, items = 0;
+    for (int d = 0; d < n; ++d) {
+        ImpactDim &g = D.dim[d];
+        g.group = 1;
+        g.item_stride = (int)sizeof(DimOut) + 8 * ((g.wcap + 1) & ~1);
+        g.item_off = bytes;
+        bytes += g.n_items * (int64_t)g.item_stride;
+        items += g.n_items;
+    }
+    D.share32 = D.kind != KIND_IMAGES && items * 3 <= D.rows * n;
+    item_bytes = D.share32 ? bytes : 0;
+    D.leaf_stride = (int)sizeof(LeafHead) + 16 * (D.leaf_cap + 1);
+    D.leaf_shared = D.share32 && n >= 3 && D.cutoff32 > 0.0f && D.leaf_items * 4 <= D.rows &&
+                    D.leaf_items * D.leaf_stride <= D.rows * (int64_t)D.rec_stride;
+    leaf_bytes = D.leaf_shared ? D.leaf_items * D.leaf_stride : 0;
+}
+
+int leaf32_bytes(const ImpactDesc &D)
+{
+    const int w = ((D.dim[D.n - 2].wcap + 1) & ~1) + ((D.dim[D.n - 1].wcap + 1) & ~1);
+    return 2 * (int)sizeof(RecDim) + 8 * w + align16(32 * (D.leaf_cap + 1));
+}
+
+cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, bool shared, bool own,
+                              int64_t item_units, uint32_t *status, cudaStream_t stream)
 {
     if (units <= 0) return cudaSuccess;
-    const int g = occupancy_grid((const void *)setup_fp32, 256, 0, units, 256 / 32);
-    setup_fp32<<<g, 256, 0, stream>>>(d_index, status, sink_lo, sink_up, trunc);
+    if (own) {
+        const int g = occupancy_grid((const void *)setup_fp32, 256, 0, units, 256 / 32);
+        setup_fp32<<<g, 256, 0, stream>>>(d_index, status);
+    }
+    if (shared) {
+        const int gi = occupancy_grid((const void *)items_fp32, 128, 0, item_units, 128 / 32);
+        items_fp32<<<gi, 128, 0, stream>>>(d_index, status);
+        const int gr = occupancy_grid((const void *)rows_fp32, 256, 0, units, 256 / 32);
+        rows_fp32<<<gr, 256, 0, stream>>>(d_index);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_terms_fp32(const BatchIndex *d_index, int64_t rows, const void *acc,
+                              int64_t fault_row, const RowOutputs &o, cudaStream_t stream)
+{
+    if (rows <= 0) return cudaSuccess;
+    const int g = occupancy_grid((const void *)terms_fp32, 256, 0, rows, 256);
+    terms_fp32<<<g, 256, 0, stream>>>(d_index, (const float4 *)acc, fault_row, o.sink_lo,
+                                      o.sink_up, o.trunc, o.flags, o.status);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_leaf_fp32(const BatchIndex *d_index, int64_t tables, int leaf_smem,
+                             cudaStream_t stream)
+{
+    if (tables <= 0) return cudaSuccess;
+    const size_t smem = (size_t)leaf_smem * 4;
+    cudaError_t e = cudaFuncSetAttribute((const void *)leaf_fp32,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int g = occupancy_grid((const void *)leaf_fp32, 128, smem, tables, 4);
+    leaf_fp32<<<g, 128, smem, stream>>>(d_index, leaf_smem);
     return cudaGetLastError();
 }
 
 cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64_t row_end,
-                             int rec_max, const int work_max[2], int warps, int mode,
+                             int rec_max, const int work_max[3], int warps, int mode,
                              const RowOutputs &o,
                              unsigned long long *lb, const WalkFaults &f, cudaStream_t stream)
 {
@@ -1448,7 +1760,7 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
     // record buffers and warp blocks start 16-byte aligned (record strides are
     // multiples of 16)
     rec_max = (rec_max + 15) & ~15;
-    const int work = work_max[mode == MODE_EMIT ? 0 : 1];
+    const int work = work_max[mode];
     const int warp_smem = (mode == MODE_EMIT ? 1 : 2) * rec_max + ((work + 15) & ~15) + kClaimBytes;
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
@@ -1469,6 +1781,7 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
     A.col = o.col;
     A.lo = (float *)o.lo;
     A.up = (float *)o.up;
+    A.acc = (float4 *)lb;
     A.trunc = o.trunc;
     A.sink_lo = o.sink_lo;
     A.sink_up = o.sink_up;

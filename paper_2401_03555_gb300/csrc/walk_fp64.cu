@@ -112,7 +112,7 @@ items_fp64(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
         const int64_t c = (u - B->item_begin[seg]) * (32 / G) + lane / G;
         const bool act = c < g.n_items;
         const int64_t cc = act ? c : 0;   // idle groups repeat item 0 and store nothing
-        unsigned char *it = B->rec[q] + g.item_off + cc * g.item_stride;
+        unsigned char *it = B->items[q] + g.item_off + cc * g.item_stride;
         double2 *ul = item_table(it);
         const double *E = D.edges + g.edge_off;
         double mlo, mhi;
@@ -264,7 +264,7 @@ terms_fp64(const BatchIndex *__restrict__ B, double *__restrict__ sink_lo,
         for (int d = 0; d < D.n; ++d) {
             const ImpactDim &g = D.dim[d];
             const Item64 *h = reinterpret_cast<const Item64 *>(
-                B->rec[q] + g.item_off + item_of(D, r, idx, j, d) * g.item_stride);
+                B->items[q] + g.item_off + item_of(D, r, idx, j, d) * g.item_stride);
             pmax *= h->gmax;
             pmin *= h->gmin;
             acc = acc * (h->SW + h->O) + pre * h->O;
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
             decode_row(D, r, idx, j);
             if (lane < n) {
                 const ImpactDim &g = D.dim[lane];
-                it = B->rec[q] + g.item_off + item_of(D, r, idx, j, lane) * g.item_stride;
+                it = B->items[q] + g.item_off + item_of(D, r, idx, j, lane) * g.item_stride;
                 h = *reinterpret_cast<const Item64 *>(it);
             }
         }
