@@ -22,7 +22,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libimpact.so")
 SOURCES = ["api.cu", "alloc.cu", "plan.cu", "kernels.cu", "static_scan.cu", "walk_fp32.cu", "walk_fp64.cu",
            "server.cu",
-           "synth.cu", "mc.cu"]
+           "synth.cu", "mc.cu", "mc_masks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

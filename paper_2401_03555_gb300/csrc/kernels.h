@@ -72,6 +72,25 @@ cudaError_t launch_mc_rows(const ImpactDesc *d_desc, bool emit, int64_t rows,
                            const double *val, const float *val_dn, const float *val_up,
                            unsigned kmin, const RowOutputs &o, cudaStream_t stream);
 
+// Sampled noise by draw masks (mc_masks.cu): layout of the masks per distinct
+// image, and their bytes (0: the per-row histogram is used).
+struct McMasks {
+    int nw;                             // words of 32 draws per lane
+    int cap[IMPACT_MAX_DIM];            // window cells an item holds
+    int stride[IMPACT_MAX_DIM];         // bytes of one item
+    int64_t first[IMPACT_MAX_DIM + 1];  // items before each dimension's
+    int64_t off[IMPACT_MAX_DIM];        // bytes before each dimension's
+    int64_t bytes;
+};
+McMasks mc_masks(const ImpactDesc &D, int64_t S, double cutoff);
+cudaError_t launch_mc_items(const ImpactDesc *d_desc, int n, const McMasks &K,
+                            const long long *keys, int64_t S, const double *range,
+                            unsigned char *items, cudaStream_t stream);
+cudaError_t launch_mc_walk(const ImpactDesc *d_desc, bool emit, int64_t rows, const McMasks &K,
+                           unsigned char *items, int64_t S, const double *val,
+                           const float *val_dn, const float *val_up, unsigned kmin,
+                           const RowOutputs &o, cudaStream_t stream);
+
 // Labels of every cell (0 free, 1 target, 2 avoid; avoid wins).
 cudaError_t launch_labels(const RegionBoxes &boxes, int64_t total_cells, uint8_t *labels,
                           cudaStream_t stream);

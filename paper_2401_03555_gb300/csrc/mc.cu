@@ -2,7 +2,7 @@
 // a noise given by draws (Sec. 4.1: a full covariance Gaussian or a custom
 // distribution, integrated by Monte-Carlo sampling instead of the closed-form
 // Gaussian factors). Same image, grid, rows and output layout as impact_build;
-// the per-row histogram kernels are in kernels.cu (mc_rows).
+// the per-row kernels are in mc_masks.cu (draw masks) and kernels.cu (histograms).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -70,6 +70,8 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     impact_status s = make_batch(&req, 1, IMPACT_FP64_PLAIN, nullptr, B);
     if (s != IMPACT_OK) return s;
     B.walks = false;
+    const McMasks masks = mc_masks(B.plans[0].desc, n_samples, cutoff);
+    B.extra = masks.bytes;
     B.plans[0].desc.cutoff = cutoff;
     B.plans[0].desc.prec = precision;
     configure_pool_once();
@@ -140,9 +142,16 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     cudaError_t e = cudaMemsetAsync(bad, 0, 4, st);
     if (e == cudaSuccess)
         e = launch_mc_prep(samples, n, S, keys, val, val_dn, val_up, bad, range, st);
-    if (e == cudaSuccess)
-        e = launch_mc_rows(desc, false, B.rows, keys, S, range, val, val_dn, val_up,
-                           (unsigned)kmin, o, st);
+    unsigned char *mask = W.base + W.L.extra;
+    auto rows_pass = [&](bool emit) {
+        return masks.bytes > 0 ? launch_mc_walk(desc, emit, B.rows, masks, mask, S, val, val_dn,
+                                                val_up, (unsigned)kmin, o, st)
+                               : launch_mc_rows(desc, emit, B.rows, keys, S, range, val, val_dn,
+                                                val_up, (unsigned)kmin, o, st);
+    };
+    if (e == cudaSuccess && masks.bytes > 0)
+        e = launch_mc_items(desc, n, masks, keys, S, range, mask, st);
+    if (e == cudaSuccess) e = rows_pass(false);
     if (e == cudaSuccess) e = launch_scan(out->row_ptr, B.rows, W.scan(), st);
     if (e != cudaSuccess) return done(fail(IMPACT_ERR_CUDA, cudaGetErrorString(e)));
     int64_t nnz = 0;
@@ -178,8 +187,7 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     o.lo = view.lo;
     o.up = view.up;
     o.capacity = capacity;
-    e = launch_mc_rows(desc, true, B.rows, keys, S, range, val, val_dn, val_up, (unsigned)kmin,
-                       o, st);
+    e = rows_pass(true);
     if (e != cudaSuccess) return done(fail(IMPACT_ERR_CUDA, cudaGetErrorString(e)));
     if (cudaMemcpyAsync(&status, W.status(), 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
