@@ -457,7 +457,7 @@ typedef enum {
  * (DEVICE int32[cells], input index; 0 on labelled cells), and the iterations
  * of each phase to iterations[2] (host, may be NULL). A phase that reaches
  * max_iters stops there (its interval is then wider than eps). Synchronizes
- * `stream` once per iteration. Same as impact_synthesize_ex with a
+ * `stream` as it goes (the stopping test itself runs on the device). Same as impact_synthesize_ex with a
  * pessimistic policy, no horizon, one disturbance point and no region
  * vectors. Errors: IMPACT_ERR_ARG, IMPACT_ERR_OOM, IMPACT_ERR_CUDA.
  */
@@ -598,7 +598,7 @@ typedef struct {
  * P_max = 1 - V0 of the min-LP phase. The policy is phase 1's choice on the
  * vector whose end phase 1 reports (ties: the lowest input index).
  * rows of imdp must equal cells * n_inputs * n_disturb. Synchronizes
- * `stream` once per iteration (once per phase with a horizon). Errors:
+ * `stream` as it goes and at the end. Errors:
  * IMPACT_ERR_ARG, IMPACT_ERR_OOM, IMPACT_ERR_CUDA.
  */
 impact_status impact_synthesize_ex(const impact_csr *imdp, impact_precision precision,
