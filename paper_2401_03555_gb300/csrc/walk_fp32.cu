@@ -603,18 +603,19 @@ rows_fp32(const BatchIndex *__restrict__ B)
 // ---------------------------------------------------------------------------
 
 constexpr int kCap = IMPACT_WALK_CAP;      // nodes per level list (one chunk)
-constexpr int kClaimBytes = 32;            // per warp: the claimed row range, rows per claim
+constexpr int kSlots = kCap + 1;           // and a spare slot
+constexpr int kClaimBytes = 16;            // per warp: the claimed row range
 constexpr int kTrimMin = 512;              // emit: candidates of a chunk worth trimming its table for
 
 // Warp shared memory: two record buffers of the batch's largest record (the
 // row being walked and the next one, copied in meanwhile), then the work
 // space (offsets fixed per problem by leaf_cap):
 //   h      RecDim[n]                 the row record's per-dimension entries
-//   ul     (U, L) x tsum_cap         the record's window tables, right after
-//   work   (n - 2) x (kCap + 1) x 12 B  node lists of levels 0..n-3
-//   leaf   3 x (leaf_cap + 1) words  the staged leaf table (see Leaf), and
-//          5 x (leaf_cap + 1) words  the count pass's sorted form and sums, or
-//                                    the emit pass's table trimmed per chunk
+//   ul     (U, L) x tsum_cap         the record's window tables
+//   work   (n - 2) x kSlots x 12 B   node lists of levels 0..n-3
+//   leaf   count: 8 x (leaf_cap + 1) words, the leaf table (see Leaf) with its
+//          sorted form and sums; emit: twice 3 words per entry, the staged
+//          table and its copy trimmed per chunk
 struct WarpMem {
     RecDim *h;
     float2 *ul;
@@ -627,16 +628,19 @@ __host__ __device__ constexpr int align16(int x) { return (x + 15) & ~15; }
 
 // Node lists of levels 0..n-3, padded to 16 bytes: the warp blocks are laid
 // end to end and each starts with 16-byte record copies.
-__host__ __device__ inline int list_bytes(int n) { return align16((n > 2 ? n - 2 : 0) * (kCap + 1) * 12); }
+__host__ __device__ inline int list_bytes(int n) { return align16((n > 2 ? n - 2 : 0) * kSlots * 12); }
 
-__device__ __forceinline__ WarpMem carve(unsigned char *work, unsigned char *rec, const ImpactDesc &D)
+// Entries of an emit leaf table, even: the tables are 8-byte aligned.
+__host__ __device__ constexpr int emit_cap(int leaf_cap) { return (leaf_cap + 1) & ~1; }
+
+__device__ __forceinline__ WarpMem carve(unsigned char *work, unsigned char *rec, int n, int leaf_cap)
 {
     WarpMem m;
     m.h = reinterpret_cast<RecDim *>(rec);
-    m.ul = rec_table(rec, D.n);
+    m.ul = rec_table(rec, n);
     m.work = work;
-    m.leaf = reinterpret_cast<float *>(m.work + list_bytes(D.n));
-    m.leaf_cap = D.leaf_cap;
+    m.leaf = reinterpret_cast<float *>(m.work + list_bytes(n));
+    m.leaf_cap = leaf_cap;
     return m;
 }
 
@@ -652,10 +656,10 @@ __device__ __forceinline__ NodeList node_list(unsigned char *work, int k)
     NodeList L;
     // kCap nodes and one spare slot that takes the stores of the lanes
     // whose candidate was not kept (stores without a branch)
-    unsigned char *b = work + (size_t)k * (kCap + 1) * 12;
+    unsigned char *b = work + k * (kSlots * 12);
     L.P = reinterpret_cast<float *>(b);
-    L.Pl = reinterpret_cast<float *>(b + (kCap + 1) * 4);
-    L.col = reinterpret_cast<int *>(b + (kCap + 1) * 8);
+    L.Pl = L.P + kSlots;
+    L.col = reinterpret_cast<int *>(L.Pl + kSlots);
     return L;
 }
 
@@ -707,8 +711,8 @@ __device__ __forceinline__ Leaf leaf_of(const WarpMem &S, int n)
     f.staged = f.nb <= S.leaf_cap;
     f.sorted = false;
     f.shared = nullptr;
-    f.magic_nb = (f.nb > 1 && f.nb <= 4096)
-                     ? (uint32_t)((0x100000000ull + (unsigned)f.nb - 1) / (unsigned)f.nb) : 0u;
+    f.magic_nb = (f.nb > 1 && f.nb <= 4096)   // ceil(2^32 / nb)
+                     ? 0xffffffffu / (unsigned)f.nb + 1u : 0u;
     const int c = S.leaf_cap + 1;
     f.bu = S.leaf;
     f.bl = f.bu + c;
@@ -748,13 +752,6 @@ __device__ __forceinline__ LeafEntry leaf_eval(const WarpMem &S, int n, const Le
     return e;
 }
 
-template <bool STAGED>
-__device__ __forceinline__ LeafEntry leaf_at(const WarpMem &S, int n, const Leaf &f, int j)
-{
-    if (!STAGED) return leaf_eval(S, n, f, j);
-    return LeafEntry{f.bu[j], f.bl[j], f.bc[j]};
-}
-
 // Inclusive warp scans of a lane's value with directed rounding (a fixed
 // association: the same bits whatever ran before).
 __device__ __forceinline__ float scan_ru(float x, int lane)
@@ -776,11 +773,13 @@ __device__ __forceinline__ float scan_rd(float x, int lane)
     return x;
 }
 
-// Stages the leaf table of a row (and, for the count pass, its sorted form
-// and sums) when it fits.
-template <bool COUNT>
+// Count pass: stages the leaf table of a row with its sorted form and sums when
+// it fits (dense rows: only the totals). A row of at most two dimensions has
+// one parent (the root): testing its entries directly costs less than sorting
+// them.
 __device__ void leaf_build(const WarpMem &S, int n, Leaf &f, int lane, float cut)
 {
+    if (n <= 2 && cut > 0.0f) return;
     float su_l = 0.0f, sl_l = 0.0f;   // this lane's part of the totals
     for (int j = lane; j < f.nb; j += 32) {
         const LeafEntry e = leaf_eval(S, n, f, j);
@@ -793,7 +792,6 @@ __device__ void leaf_build(const WarpMem &S, int n, Leaf &f, int lane, float cut
         sl_l = __fadd_rd(sl_l, e.l);
     }
     __syncwarp();
-    if (!COUNT) return;
     if (!(cut > 0.0f)) {   // the totals serve the dense count only
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -803,9 +801,7 @@ __device__ void leaf_build(const WarpMem &S, int n, Leaf &f, int lane, float cut
         f.tot_u = __shfl_sync(0xffffffffu, su_l, 0);
         f.tot_l = __shfl_sync(0xffffffffu, sl_l, 0);
     }
-    // a row of at most two dimensions has one parent (the root): testing
-    // its entries directly costs less than sorting them
-    if (!f.staged || !(cut > 0.0f) || n <= 2) return;
+    if (!f.staged || !(cut > 0.0f)) return;
     f.sorted = true;
     if (f.nb <= 32) {
         // one entry per lane: a bitonic sorting network over the warp puts
@@ -962,7 +958,7 @@ leaf_fp32(const BatchIndex *__restrict__ B, int warp_smem)
         __syncwarp();
         unsigned char *out = B->leaf[q] + c0 * D.leaf_stride;
         Leaf f = leaf_of(S, n);
-        if (f.nb > 0 && f.staged) leaf_build<true>(S, n, f, lane, D.cutoff32);
+        if (f.nb > 0 && f.staged) leaf_build(S, n, f, lane, D.cutoff32);
         if (lane == 0) reinterpret_cast<LeafHead *>(out)->nb = f.sorted ? f.nb : -1;
         if (f.sorted) {
             float4 *to = reinterpret_cast<float4 *>(out + sizeof(LeafHead));
@@ -981,13 +977,8 @@ struct Node {
 
 __device__ __forceinline__ Node node_at(const NodeList &L, bool root, int i)
 {
-    Node x{1.0f, 1.0f, 0};
-    if (!root) {
-        x.P = L.P[i];
-        x.Pl = L.Pl[i];
-        x.c = L.col[i];
-    }
-    return x;
+    if (root) return Node{1.0f, 1.0f, 0};
+    return Node{L.P[i], L.Pl[i], L.col[i]};
 }
 
 // A narrow window (tw <= 32) is walked with each lane fixed on one target t
@@ -1023,22 +1014,23 @@ __device__ __forceinline__ int chunk_of(const RecDim &h)
 // Children of candidates [c0, c1) of the level k - 1 list (the root when
 // k = 0) in dimension k, kept ones compacted into the level k list in order.
 // A candidate e is (parent e / tw, target t = e mod tw of the trimmed window).
-__device__ __forceinline__ int expand(const WarpMem &S, int k, int c0, int c1, int lane,
-                                      CountAcc &acc, bool count)
+template <bool COUNT>
+__device__ __forceinline__ int expand(const WarpMem &S, int k, bool root, int c0, int c1, int lane,
+                                      CountAcc &acc)
 {
     const RecDim &h = S.h[k];
     const int tw = h.tw, tb = h.tb, cb = h.cb, st = h.stride;
     const uint32_t magic = h.magic;
-    const float cp = h.cp, SR = h.SR;
+    const float cp = h.cp, SR = COUNT ? h.SR : 0.0f;
     const NodeList Lc = node_list(S.work, k);
-    const NodeList Lp = node_list(S.work, k > 0 ? k - 1 : 0);
-    const bool root = k == 0;
+    const NodeList Lp = node_list(S.work, root ? 0 : k - 1);
     const Lanes z = lanes_of(h, lane);
     int nout = 0;
+    __syncwarp();   // the list's readers are done
     auto offer = [&](bool act, const Node &par, float2 ul, int t) {
         const float Pc = __fmul_ru(par.P, ul.x);
         const bool keep = act && Pc >= cp;
-        if (count) {
+        if (COUNT) {
             const float d = __fadd_ru(acc.drop, __fmul_ru(Pc, SR));
             acc.drop = (act && !keep) ? d : acc.drop;
         }
@@ -1163,159 +1155,212 @@ __device__ __forceinline__ void leaf_count_shared(const float4 *__restrict__ tab
     }
 }
 
-// Stores that the predicate guards, without a branch around them.
-__device__ __forceinline__ void st_if(bool p, int32_t *a, int32_t v)
+// Stores of one pair that the predicate guards, without a branch around them.
+__device__ __forceinline__ void st_pair(bool p, int32_t *c, float *l, float *u, int32_t col, float lo,
+                                        float up)
 {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q st.global.b32 [%1], %2;\n\t}"
-                 :: "r"((int)p), "l"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void st_if(bool p, float *a, float v)
-{
-    st_if(p, reinterpret_cast<int32_t *>(a), __float_as_int(v));
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t"
+                 "@q st.global.b32 [%1], %4;\n\t@q st.global.b32 [%2], %5;\n\t"
+                 "@q st.global.b32 [%3], %6;\n\t}"
+                 :: "r"((int)p), "l"(c), "l"(l), "l"(u), "r"(col), "r"(__float_as_int(lo)),
+                    "r"(__float_as_int(up)) : "memory");
 }
 
 // One candidate per lane: the kept ones are compacted in lane order after the
 // pairs already written and stored (predicated, no divergence).
-__device__ __forceinline__ void offer_pair(bool act, const Node &par, const LeafEntry &e, float cut,
-                                           const EmitOut &out, int &written)
+__device__ __forceinline__ void offer_pair(bool act, float P, float Pl, int c, float u, float l,
+                                           float cut, const EmitOut &out, int &written)
 {
-    const float Pc = __fmul_ru(par.P, e.u);
+    const float Pc = __fmul_ru(P, u);
     const bool keep = act && Pc >= cut;
     const unsigned bal = __ballot_sync(0xffffffffu, keep);
     const int pos = written + __popc(bal & lanemask_lt());
-    const bool st = keep && pos < out.len;
-    st_if(st, out.col + pos, par.c + e.c);
-    st_if(st, out.lo + pos, __fmul_rd(par.Pl, e.l));
-    st_if(st, out.up + pos, Pc);
+    st_pair(keep && pos < out.len, out.col + pos, out.lo + pos, out.up + pos, c, __fmul_rd(Pl, l), Pc);
     written += __popc(bal);
 }
 
-// Emit pass over the leaves of npar parents: each entry of the table under
-// each parent one lane (flat: candidate e = parent * nb + entry, so no lane
-// idles but in the last step); kept pairs are compacted in C order and stored
-// warp-contiguously. A layout that keeps the table in registers and steps
-// over parents measured slower: its lanes idle when 32 is not a multiple of
-// nb, and its registers cost occupancy.
-template <bool ROOT, bool STAGED>
-__device__ void leaf_emit(const WarpMem &S, int n, const Leaf &f, const NodeList &Lp, int npar,
-                          int lane, const EmitOut &out, int &written, float cut)
+// The leaf table as the emit pass walks it: the products of upper and of lower
+// factors and the columns, `cap` words apart (32-bit arrays: the lanes of a step
+// wrap from a parent's last entry to the next one's first, which pairs of
+// words in one array turn into bank conflicts).
+struct EmitLeaf {
+    float *u;
+    int cap;
+    int nb;
+    uint32_t magic;    // ceil(2^32 / nb)
+    bool staged;
+};
+
+__device__ __forceinline__ EmitLeaf emit_leaf(const WarpMem &S, const Leaf &f)
 {
+    EmitLeaf e;
+    e.u = S.leaf;
+    e.cap = emit_cap(S.leaf_cap);
+    e.nb = f.nb;
+    e.magic = f.magic_nb;
+    e.staged = f.staged;
+    return e;
+}
+
+// Emit pass over the leaves of npar parents from the staged table: each entry
+// under each parent one lane (flat: candidate e = parent * nb + entry, so no
+// lane idles but in the last step); kept pairs are compacted in C order and
+// stored warp-contiguously. A layout that keeps the table in registers and
+// steps over parents measured slower: its lanes idle when 32 is not a multiple
+// of nb, and its registers cost occupancy.
+__device__ __forceinline__ void leaf_emit(const WarpMem &S, const EmitLeaf &f, const NodeList &Lp,
+                                          int npar, int lane, const EmitOut &out, int &written,
+                                          float cut)
+{
+    const float *tu = f.u;
+    const int cs = f.cap;
     int nb = f.nb;
-    uint32_t magic = f.magic_nb;
-    // the table walked: upper, lower and column columns leaf_cap + 1 words
-    // apart (the staged table, or its trimmed copy in the count pass's space)
-    const float *tu = f.bu;
-    const int cs = S.leaf_cap + 1;
-    if (STAGED && !ROOT && cut > 0.0f && npar * nb >= kTrimMin) {
+    uint32_t magic = f.magic;
+    if (cut > 0.0f && npar * nb >= kTrimMin) {
         // entries that no parent of these can keep: RU(P x) is monotone in P,
         // so an entry below the cutoff under the largest P is below it under
         // every P. The rest, in C order, form the table walked below; the
         // pairs are the same. (A pass over the table and a division: worth it
         // only when the parents and the table are large.)
         float pm = 0.0f;
-        for (int pi = lane; pi < npar; pi += 32) pm = fmaxf(pm, node_at(Lp, ROOT, pi).P);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
-        float *const su = f.su;
+        for (int pi = lane; pi < npar; pi += 32) pm = fmaxf(pm, Lp.P[pi]);
+        pm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(pm)));   // pm >= 0
+        float *const su = f.u + 3 * cs;
         int nt = 0;
-        for (int j0 = 0; j0 < f.nb; j0 += 32) {
-            const int j = j0 + lane;
-            const float u = j < f.nb ? f.bu[j] : 0.0f;
-            const bool k = j < f.nb && __fmul_ru(pm, u) >= cut;
+        for (int j0 = 0; j0 < nb; j0 += 32) {
+            const int j = min(j0 + lane, nb - 1);
+            const float v = tu[j];
+            const bool k = j0 + lane < nb && __fmul_ru(pm, v) >= cut;
             const unsigned bal = __ballot_sync(0xffffffffu, k);
             if (k) {
                 const int o = nt + __popc(bal & lanemask_lt());
-                su[o] = u;
-                su[o + cs] = f.bl[j];
-                su[o + 2 * cs] = f.bu[j + 2 * cs];   // the column's bits
+                su[o] = v;
+                su[o + cs] = tu[j + cs];
+                su[o + 2 * cs] = tu[j + 2 * cs];   // the column's bits
             }
             nt += __popc(bal);
         }
         __syncwarp();
         if (nt == 0) return;
-        nb = nt;
-        magic = nt > 1 ? 0xffffffffu / (unsigned)nt + 1u : 0u;   // ceil(2^32 / nt)
-        tu = su;
-    }
-    auto entry = [&](int j) -> LeafEntry {
-        if (!STAGED) return leaf_eval(S, n, f, j);
-        return LeafEntry{tu[j], tu[j + cs], __float_as_int(tu[j + 2 * cs])};
-    };
-    // every lane computes, the kept ones store (predicated, no divergence)
-    auto offer = [&](bool act, const Node &par, const LeafEntry &e) {
-        offer_pair(act, par, e, cut, out, written);
-    };
-    if (ROOT || nb <= 4096) {
-        // the division is exact for e < 64 nb, nb <= 4096; lanes past the end
-        // read the last candidate and store nothing
-        const int total = npar * nb;
-        int e0 = 0;
-        // two candidates per lane and step, both loaded before either ballot
-        for (; e0 + 32 < total; e0 += 64) {
-            const int ea = e0 + lane, eb = min(e0 + 32 + lane, total - 1);
-            const int pa = (ROOT || nb == 1) ? (ROOT ? 0 : ea) : (int)__umulhi((uint32_t)ea, magic);
-            const int pb = (ROOT || nb == 1) ? (ROOT ? 0 : eb) : (int)__umulhi((uint32_t)eb, magic);
-            const Node node_a = node_at(Lp, ROOT, pa), node_b = node_at(Lp, ROOT, pb);
-            const LeafEntry leaf_a = entry(ea - pa * nb);
-            const LeafEntry leaf_b = entry(eb - pb * nb);
-            offer(true, node_a, leaf_a);
-            offer(e0 + 32 + lane < total, node_b, leaf_b);
+        if (nt < nb) {
+            nb = nt;
+            magic = nt > 1 ? 0xffffffffu / (unsigned)nt + 1u : 0u;   // ceil(2^32 / nt)
+            tu = su;
         }
-        for (; e0 < total; e0 += 32) {
-            const int e = min(e0 + lane, total - 1);
-            const int pi = (ROOT || nb == 1) ? (ROOT ? 0 : e) : (int)__umulhi((uint32_t)e, magic);
-            const int j = e - pi * nb;
-            offer(e0 + lane < total, node_at(Lp, ROOT, pi), entry(j));
-        }
-        return;
     }
+    // the division is exact for e < 64 nb, nb <= 4096; lanes past the end read
+    // the last candidate and store nothing
+    const int total = npar * nb;
+    auto offer = [&](bool act, const Node &par, int j) {
+        offer_pair(act, par.P, par.Pl, par.c + __float_as_int(tu[j + 2 * cs]), tu[j], tu[j + cs],
+                   cut, out, written);
+    };
+    int e0 = 0;
+    for (; e0 + 32 < total; e0 += 64) {   // two candidates per lane and step
+        const int ea = e0 + lane, eb = min(e0 + 32 + lane, total - 1);
+        const int pa = nb == 1 ? ea : (int)__umulhi((uint32_t)ea, magic);
+        const int pb = nb == 1 ? eb : (int)__umulhi((uint32_t)eb, magic);
+        const int ja = ea - pa * nb, jb = eb - pb * nb;
+        const Node na = node_at(Lp, false, pa), nc = node_at(Lp, false, pb);
+        const float ua = tu[ja], la = tu[ja + cs], ub = tu[jb], lb = tu[jb + cs];
+        const int ca = __float_as_int(tu[ja + 2 * cs]), cb = __float_as_int(tu[jb + 2 * cs]);
+        offer_pair(true, na.P, na.Pl, na.c + ca, ua, la, cut, out, written);
+        offer_pair(e0 + 32 + lane < total, nc.P, nc.Pl, nc.c + cb, ub, lb, cut, out, written);
+    }
+    for (; e0 < total; e0 += 32) {
+        const int e = min(e0 + lane, total - 1);
+        const int pi = nb == 1 ? e : (int)__umulhi((uint32_t)e, magic);
+        offer(e0 + lane < total, node_at(Lp, false, pi), e - pi * nb);
+    }
+}
+
+// The same for a table too wide to stage, and for the root (rows of at most two
+// dimensions): entries evaluated where they are read.
+__device__ __forceinline__ void leaf_emit_wide(const WarpMem &S, int n, const Leaf &f,
+                                               const NodeList &Lp, bool root, int npar, int lane,
+                                               const EmitOut &out, int &written, float cut)
+{
     for (int pi = 0; pi < npar; ++pi) {
-        const Node par = node_at(Lp, ROOT, pi);
-        for (int j0 = 0; j0 < nb; j0 += 32) {
-            const int j = min(j0 + lane, nb - 1);
-            offer(j0 + lane < nb, par, entry(j));
+        const Node par = node_at(Lp, root, pi);
+        for (int j0 = 0; j0 < f.nb; j0 += 32) {
+            const LeafEntry e = leaf_eval(S, n, f, min(j0 + lane, f.nb - 1));
+            offer_pair(j0 + lane < f.nb, par.P, par.Pl, par.c + e.c, e.u, e.l, cut, out, written);
         }
     }
 }
 
-// Walks one row whose record is in S: levels 0..n-3 as node lists, depth
-// first over chunks, the leaf table under every chunk of the deepest list.
-// Returns false if the step guard ran out (a broken invariant, reported as
-// an error).
-template <bool EMIT>
-__device__ bool walk_row(const WarpMem &S, int n, const Leaf &f, int lane, CountAcc &acc,
-                         const EmitOut &out, int &written, float cut)
+// Count walk: levels 0..n-3 of one row as node lists, depth first over chunks,
+// the leaves under every chunk of the deepest list. LEFT lists are still to
+// come; the recursion is unrolled at compile time (a loop with the level as a
+// variable spends more on finding its place than on the nodes: the 8^5 room's
+// count pass took 1251 instructions a row, and takes 861), and every loop runs
+// over a list's candidates once, so it ends.
+template <int LEFT, bool ROOT>
+__device__ __forceinline__ void count_levels(const WarpMem &S, int n, const Leaf &f, int npar,
+                                             int lane, CountAcc &acc, float cut)
+{
+    const int k = n - 2 - LEFT;
+    const int total = npar * S.h[k].tw, chunk = chunk_of(S.h[k]);
+#pragma unroll 1
+    for (int c0 = 0; c0 < total; c0 += chunk) {
+        const int nout = expand<true>(S, k, ROOT, c0, min(c0 + chunk, total), lane, acc);
+        if constexpr (LEFT > 1) {
+            count_levels<LEFT - 1, false>(S, n, f, nout, lane, acc, cut);
+        } else {
+            const NodeList L = node_list(S.work, k);
+            if (f.shared) leaf_count_shared(f.shared, f.nb, L, nout, lane, acc, cut);
+            else leaf_count(S, n, f, L, false, nout, lane, acc, cut);
+        }
+    }
+}
+
+// Counts one row whose record is in S (its leaf table built or shared).
+__device__ __forceinline__ void count_row(const WarpMem &S, int n, const Leaf &f, int lane,
+                                          CountAcc &acc, float cut)
+{
+    switch (n) {
+    case 1:
+    case 2: leaf_count(S, n, f, NodeList{}, true, 1, lane, acc, cut); break;
+    case 3: count_levels<1, true>(S, n, f, 1, lane, acc, cut); break;
+    case 4: count_levels<2, true>(S, n, f, 1, lane, acc, cut); break;
+    case 5: count_levels<3, true>(S, n, f, 1, lane, acc, cut); break;
+    case 6: count_levels<4, true>(S, n, f, 1, lane, acc, cut); break;
+    case 7: count_levels<5, true>(S, n, f, 1, lane, acc, cut); break;
+    default: count_levels<6, true>(S, n, f, 1, lane, acc, cut); break;
+    }
+}
+
+// Writes the pairs of one row whose record is in S: the same lists, with the
+// level as a variable (the unrolled recursion keeps every level's loop state
+// live, and the emit's inner loop needs the registers: 64 let 8 warps per
+// scheduler hide its shared-memory latency; unrolled, the 11^5 room's emit
+// pass took 7.8 ms against 7.45). Every step fills a list, runs the leaves of one
+// or leaves one whose candidates are used up, so the loop ends.
+__device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f, int lane,
+                                         const EmitOut &out, int &written, float cut)
 {
     if (n <= 2) {
-        if (EMIT) {
-            if (f.staged) leaf_emit<true, true>(S, n, f, node_list(S.work, 0), 1, lane, out, written, cut);
-            else leaf_emit<true, false>(S, n, f, node_list(S.work, 0), 1, lane, out, written, cut);
-        }
-        else leaf_count(S, n, f, node_list(S.work, 0), true, 1, lane, acc, cut);
-        return true;
+        leaf_emit_wide(S, n, f, NodeList{}, true, 1, lane, out, written, cut);
+        return;
     }
-    auto leaves = [&](const NodeList &Lp, int npar) {
-        if (EMIT) {
-            if (f.staged) leaf_emit<false, true>(S, n, f, Lp, npar, lane, out, written, cut);
-            else leaf_emit<false, false>(S, n, f, Lp, npar, lane, out, written, cut);
+    const EmitLeaf g = emit_leaf(S, f);
+    if (g.staged)
+        for (int j = lane; j < f.nb; j += 32) {
+            const LeafEntry e = leaf_eval(S, n, f, j);
+            g.u[j] = e.u;
+            g.u[j + g.cap] = e.l;
+            g.u[j + 2 * g.cap] = __int_as_float(e.c);
         }
-        else if (f.shared) leaf_count_shared(f.shared, f.nb, Lp, npar, lane, acc, cut);
-        else leaf_count(S, n, f, Lp, false, npar, lane, acc, cut);
-    };
-    const int last = n - 3;   // deepest list level
-    // every step fills a list, leaves one or runs the leaves of one: bound
-    // them by the candidates of every level (loose, overflow-safe)
-    int64_t guard = 16, prod = 1;
-    for (int k = 0; k <= last; ++k) {
-        prod = min(prod * (int64_t)S.h[k].tw, (int64_t)1 << 40);
-        guard += 8 * (int64_t)(k + 1) * (1 + prod / kCap);
-    }
+    const int last = n - 3;      // deepest list level
     int my_cur = 0, my_sz = 0;   // lane k: next candidate of level k, size of list k
+    CountAcc none;
     int k = 0;
     while (true) {
-        if (--guard < 0) return false;
         if (k == last + 1) {
-            leaves(node_list(S.work, last), __shfl_sync(0xffffffffu, my_sz, last));
+            const NodeList L = node_list(S.work, last);
+            const int npar = __shfl_sync(0xffffffffu, my_sz, last);
+            if (g.staged) leaf_emit(S, g, L, npar, lane, out, written, cut);
+            else leaf_emit_wide(S, n, f, L, false, npar, lane, out, written, cut);
             k = last;
             continue;
         }
@@ -1328,7 +1373,7 @@ __device__ bool walk_row(const WarpMem &S, int n, const Leaf &f, int lane, Count
             continue;
         }
         const int end = min(cur + chunk_of(S.h[k]), total);
-        const int nout = expand(S, k, cur, end, lane, acc, !EMIT);
+        const int nout = expand<false>(S, k, k == 0, cur, end, lane, none);
         if (lane == k) {
             my_cur = end;
             my_sz = nout;
@@ -1336,8 +1381,8 @@ __device__ bool walk_row(const WarpMem &S, int n, const Leaf &f, int lane, Count
         if (lane == k + 1) my_cur = 0;
         ++k;
     }
-    return true;
 }
+
 // ---------------------------------------------------------------------------
 // row offsets by decoupled look-back, and the FP64 row terms
 // ---------------------------------------------------------------------------
@@ -1465,7 +1510,7 @@ struct WalkArgs {
 };
 
 template <int MODE>
-__global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32) walk_fp32(const WalkArgs A)
+__global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const WalkArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr bool kCount = MODE != MODE_EMIT;
@@ -1478,133 +1523,132 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32) walk_fp32(const Wa
         return;
     }
     unsigned long long *const next_row = B->next_row + (MODE == MODE_EMIT ? 1 : 0);
-    bool lb_ok = true;
 
     // persistent: each warp takes rows from the batch's row counter,
     // A.row_block consecutive rows per atomic (one counter serves every warp
     // of the grid: claiming short rows one by one queues the atomics), in
-    // ascending order. The passes that count take them two ahead: while a
-    // warp walks a row, the index of the row after the next is known and the
-    // next row's record is copied (cp.async) into the warp's other record
-    // buffer. The emit pass (more registers live in its walk) copies each
-    // record when it starts it.
+    // ascending order. The passes that count take
+    // rows one ahead: while a warp walks a row, the next row's record is copied
+    // (cp.async) into the warp's other record buffer. The emit pass (more
+    // registers live in its walk) copies each record when it starts it.
     constexpr bool kAhead = MODE != MODE_EMIT;
-    const unsigned long long nrows = (unsigned long long)(A.row_end - A.row_begin);
+    const int64_t row_end = A.row_end;
     unsigned char *const work = wbase + (kAhead ? 2 : 1) * A.rec_max;
-    // the warp's claimed rows [claim[0], claim[1]) and the rows per claim
-    // (claim[2]), in the last bytes of its block (not registers: the walk
-    // needs all of them)
+    // the claimed rows [claim[0], claim[1]) stand in the last bytes of the
+    // warp's block (not in registers: the walk needs all of them)
     unsigned long long *const claim =
         reinterpret_cast<unsigned long long *>(wbase + A.warp_smem - kClaimBytes);
-    if (lane == 0) {
-        claim[0] = claim[1] = 0;
-        claim[2] = (unsigned long long)A.row_block;
-    }
+    if (lane == 0) claim[0] = claim[1] = 0;
     __syncwarp();
-    auto take = [&]() -> unsigned long long {
+    auto take = [&]() -> int64_t {
         unsigned long long t = claim[0];
         if (t == claim[1]) {   // warp-uniform: every lane reads the same words
             unsigned long long c = 0;
-            if (lane == 0) c = atomicAdd(next_row, claim[2]);
+            if (lane == 0) c = atomicAdd(next_row, (unsigned long long)A.row_block);
             t = __shfl_sync(0xffffffffu, c, 0);
-            if (lane == 0) claim[1] = t + claim[2];
+            if (lane == 0) claim[1] = t + A.row_block;
         }
         __syncwarp();
         if (lane == 0) claim[0] = t + 1;
         __syncwarp();
-        return t;
+        return A.row_begin + (int64_t)t;
     };
-    auto fetch = [&](unsigned long long t, int &q, unsigned char *dst) {
-        if (t >= nrows) return;
-        const int64_t row = A.row_begin + (int64_t)t;
+    auto fetch = [&](int64_t row, int &q, unsigned char *dst) {
+        if (row >= row_end) return;
         q = next_problem(B->row_begin, B->count, q, row);
-        const int stride = B->desc[q]->rec_stride;
+        const ImpactDesc &D = *B->desc[q];
+        const int stride = D.rec_stride;
         const unsigned char *src = B->rec[q] + (row - B->row_begin[q]) * (int64_t)stride;
-        for (int i = lane; i < (stride >> 4); i += 32) cp_async16(dst + 16 * i, src + 16 * i);
+        // a count with a shared leaf table reads no table of the last two
+        // dimensions
+        const int bytes = MODE == MODE_COUNT && D.leaf_shared
+                              ? (int)(sizeof(RecDim) * D.n + sizeof(RecRow)) + 8 * D.dim[D.n - 2].rec_off
+                              : stride;
+        for (int i = lane; i < (bytes >> 4); i += 32) cp_async16(dst + 16 * i, src + 16 * i);
     };
-    unsigned long long t_cur = take();
-    unsigned long long t_nxt = 0;
-    int q_cur = 0, b = 0;
+    int64_t row = take();
+    int q = 0, b = 0;
     if (kAhead) {
-        t_nxt = take();
-        fetch(t_cur, q_cur, wbase);
+        fetch(row, q, wbase);
         cp_async_commit();
     }
-    while (t_cur < nrows) {
-        unsigned long long t_after = 0;
-        int q_nxt = q_cur;
+    while (row < row_end) {
+        int64_t nxt = 0;
+        int q_nxt = q;
         if (kAhead) {
-            t_after = take();
-            fetch(t_nxt, q_nxt, wbase + (b ^ 1) * A.rec_max);
+            nxt = take();
+            fetch(nxt, q_nxt, wbase + (b ^ 1) * A.rec_max);
             cp_async_commit();
             cp_async_wait_prior();   // this row's record has landed
         } else {
-            fetch(t_cur, q_cur, wbase);
+            fetch(row, q, wbase);
             cp_async_commit();
             cp_async_wait_all();
         }
         __syncwarp();
-        const int64_t row = A.row_begin + (int64_t)t_cur;   // global row of the batch
-        const int q = q_cur;
         const ImpactDesc &D = *B->desc[q];
         const int n = D.n;
         const float cut = D.cutoff32;
-        const WarpMem S = carve(work, wbase + b * A.rec_max, D);
-        __syncwarp();
-        bool empty = false;
-        for (int k = 0; k < n; ++k) empty |= (S.h[k].tw == 0);
+        unsigned char *const rec = wbase + b * A.rec_max;
+        const WarpMem S = carve(work, rec, n, D.leaf_cap);
+        const bool empty = __any_sync(0xffffffffu, lane < n && S.h[lane].tw == 0);
         Leaf f = leaf_of(S, n);
-        if (MODE == MODE_COUNT && D.leaf_shared && !empty) {
-            const unsigned char *tab =
-                B->leaf[q] + rec_row(wbase + b * A.rec_max, n)->leaf * D.leaf_stride;
-            if (reinterpret_cast<const LeafHead *>(tab)->nb > 0)
-                f.shared = reinterpret_cast<const float4 *>(tab + sizeof(LeafHead));
-        }
-        if (!empty && !f.shared) leaf_build<kCount>(S, n, f, lane, cut);
-        bool walked = true;
+        bool walked = row != A.guard_row;   // fault injection: a broken walk
+        bool lb_ok = true;
         int64_t base = 0, len = 0;
         if (kCount) {
             CountAcc acc;
-            const EmitOut none{nullptr, nullptr, nullptr, 0};
-            int w0 = 0;
-            if (row == A.guard_row) walked = false;
-            else if (!empty) walked = walk_row<false>(S, n, f, lane, acc, none, w0, cut);
-            int c = walked ? acc.cnt : 0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-            const float drop = warp_sum_ru(walked ? acc.drop : 0.0f);
-            const float sup = warp_sum_ru(walked ? acc.sup : 0.0f);
-            const float slo = warp_sum_rd(walked ? acc.slo : 0.0f);
-            int64_t prefix = 0;
+            if (!empty && walked) {
+                if (MODE == MODE_COUNT && D.leaf_shared) {
+                    const unsigned char *tab = B->leaf[q] + rec_row(rec, n)->leaf * D.leaf_stride;
+                    if (reinterpret_cast<const LeafHead *>(tab)->nb > 0) {
+                        f.shared = reinterpret_cast<const float4 *>(tab + sizeof(LeafHead));
+                    } else {   // too wide for a table: the last two windows after all
+                        const unsigned char *src = B->rec[q] + (row - B->row_begin[q]) * (int64_t)D.rec_stride;
+                        const int from = (int)(sizeof(RecDim) * n + sizeof(RecRow)) + 8 * D.dim[n - 2].rec_off;
+                        for (int i = (from >> 4) + lane; i < (D.rec_stride >> 4); i += 32)
+                            cp_async16(rec + 16 * i, src + 16 * i);
+                        cp_async_commit();
+                        cp_async_wait_all();
+                        __syncwarp();
+                    }
+                }
+                if (!f.shared) leaf_build(S, n, f, lane, cut);
+                count_row(S, n, f, lane, acc, cut);
+            }
+            const int c = __reduce_add_sync(0xffffffffu, acc.cnt);
+            const float drop = warp_sum_ru(acc.drop);
+            const float sup = warp_sum_ru(acc.sup);
+            const float slo = warp_sum_rd(acc.slo);
             if (MODE == MODE_FUSED) {
+                int64_t prefix = 0;
                 lb_ok = lookback(A.lb, row, c, lane, A.status + 1, A.status, A.spin_limit,
                                  row == A.stall_row, prefix);
                 if (lane == 0 && lb_ok) {
                     A.row_ptr[row] = prefix;
                     if (row == B->rows - 1) A.row_ptr[B->rows] = prefix + c;
                 }
+                base = prefix;
+                len = c;
+                if (lane == 0) {
+                    // FP64 row terms: the dropped in-window mass joins the mass
+                    // outside the window box; then the row checks of Def. 3.1
+                    const double tr = __dadd_ru(A.trunc[row], (double)drop);
+                    A.trunc[row] = tr;
+                    if (A.flags) {
+                        const double slv = A.sink_lo[row], suv = A.sink_up[row];
+                        const double lo_sum = row == A.fault_row ? 2.0 : (double)slo;
+                        uint32_t fl = 0;
+                        if (__dadd_rd(lo_sum, slv) > 1.0) fl |= IMPACT_ROW_LO_SUM_ABOVE_ONE;
+                        if (__dadd_ru(__dadd_ru((double)sup, suv), tr) < 1.0)
+                            fl |= IMPACT_ROW_UP_SUM_BELOW_ONE;
+                        A.flags[row] = fl;
+                        if (fl) atomicOr(A.status, IMPACT_STATUS_UNSOUND);
+                    }
+                }
             } else if (lane == 0) {
                 A.row_ptr[row] = c;   // counts; the scan turns them into row pointers
-            }
-            base = prefix;
-            len = c;
-            if (MODE == MODE_COUNT) {   // terms_fp32 finishes the row
-                if (lane == 0) A.acc[row] = make_float4(drop, sup, slo, 0.0f);
-            } else if (lane == 0) {
-                // FP64 row terms: the dropped in-window mass joins the mass
-                // outside the window box; then the row checks of Def. 3.1
-                const double tr = __dadd_ru(A.trunc[row], (double)drop);
-                A.trunc[row] = tr;
-                if (A.flags) {
-                    const double slv = A.sink_lo[row], suv = A.sink_up[row];
-                    const double lo_sum = row == A.fault_row ? 2.0 : (double)slo;
-                    uint32_t fl = 0;
-                    if (__dadd_rd(lo_sum, slv) > 1.0) fl |= IMPACT_ROW_LO_SUM_ABOVE_ONE;
-                    if (__dadd_ru(__dadd_ru((double)sup, suv), tr) < 1.0)
-                        fl |= IMPACT_ROW_UP_SUM_BELOW_ONE;
-                    A.flags[row] = fl;
-                    if (fl) atomicOr(A.status, IMPACT_STATUS_UNSOUND);
-                }
+                A.acc[row] = make_float4(drop, sup, slo, 0.0f);   // terms_fp32 finishes the row
             }
         } else {
             base = A.row_ptr[row];
@@ -1617,25 +1661,21 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32) walk_fp32(const Wa
                                                           : IMPACT_STATUS_EMIT_MISMATCH);
             } else {
                 const EmitOut out{A.col + base, A.lo + base, A.up + base, (int)len};
-                CountAcc none;
                 int written = 0;
-                bool wok = true;
-                if (row == A.guard_row) wok = false;
-                else if (!empty) wok = walk_row<true>(S, n, f, lane, none, out, written, cut);
-                if (lane == 0 && (!wok || written != len))
-                    atomicOr(A.status, wok ? IMPACT_STATUS_EMIT_MISMATCH : IMPACT_STATUS_INTERNAL);
+                __syncwarp();   // FUSED: the count's leaf table makes room
+                if (!empty) emit_row(S, n, f, lane, out, written, cut);
+                if (lane == 0 && written != len) atomicOr(A.status, IMPACT_STATUS_EMIT_MISMATCH);
             }
         }
         if (lane == 0 && !walked) atomicOr(A.status, IMPACT_STATUS_INTERNAL);
         if (!lb_ok) break;   // the rows after this one cannot find their offsets
         __syncwarp();        // every lane is done with the buffer before it is refilled
         if (kAhead) {
-            t_cur = t_nxt;
-            q_cur = q_nxt;
-            t_nxt = t_after;
+            row = nxt;
+            q = q_nxt;
             b ^= 1;
         } else {
-            t_cur = take();
+            row = take();
         }
     }
     cp_async_wait_all();
@@ -1665,9 +1705,13 @@ int64_t record_stride(int n, int tsum_cap)
 
 int walk_work_bytes(const ImpactDesc &D, int mode)
 {
-    // rows with a shared leaf table stage none of their own to count
-    if (mode == MODE_COUNT && D.leaf_shared) return list_bytes(D.n);
-    return list_bytes(D.n) + align16((mode == MODE_EMIT ? 24 : 32) * (D.leaf_cap + 1));
+    // rows with a shared leaf table stage none of their own to count, and
+    // rows of at most two dimensions none at all
+    const int emit = D.n > 2 ? 24 * emit_cap(D.leaf_cap) : 0;
+    const int count = D.n > 2 || !(D.cutoff32 > 0.0f) ? 32 * (D.leaf_cap + 1) : 0;
+    if (mode == MODE_EMIT) return list_bytes(D.n) + align16(emit);
+    if (mode == MODE_COUNT) return list_bytes(D.n) + align16(D.leaf_shared ? 0 : count);
+    return list_bytes(D.n) + align16(emit > count ? emit : count);
 }
 
 int walk_core_bytes(int n, int tsum_cap, int leaf_cap)
