@@ -180,9 +180,10 @@ BatchLayout batch_layout(const Batch &B)
     }
     L.upload_end = o;
     L.status = put(64);
-    L.counter = put(64);
     L.scan = put((size_t)impact::scan_scratch_elems(B.rows) * 8);
-    L.lb = put(B.prec == PREC_FP32_SOUND ? (size_t)B.rows * 16 : 0);
+    L.lb = put(!B.walks                    ? 0
+               : B.prec == PREC_FP32_SOUND ? (size_t)B.rows * 16
+                                           : (B.any64 ? (size_t)B.rows * 24 : 0));
     L.rec.resize(count);
     L.item.resize(count);
     L.leaf.resize(count);
@@ -308,7 +309,6 @@ impact_status upload(const Batch &B, Work &W, cudaStream_t st)
     }
     // pageable source: returns once the bytes are staged, so `host` may go
     CK(cudaMemcpyAsync(W.base, host.data(), host.size(), cudaMemcpyHostToDevice, st));
-    CK(cudaMemsetAsync(W.status(), 0, 64, st));
     return IMPACT_OK;
 }
 
@@ -379,14 +379,14 @@ impact::RowOutputs shifted(const impact::RowOutputs &o, int64_t rb, int64_t rows
 
 // FP32 walk launches of one pass over the batch's rows, in chunks of
 // `chunk_rows` rows (0: one launch) in row order on `st`; `counter` is the
-// pass's row counter, reset before each launch.
+// pass's row counter (zero at the first launch, reset before the others).
 cudaError_t walk_pass(const Batch &B, const Work &W, int mode, int warps,
                       const impact::RowOutputs &o, unsigned long long *counter,
                       int64_t chunk_rows, cudaStream_t st)
 {
     const int64_t step = chunk_rows > 0 ? chunk_rows : std::max<int64_t>(B.rows, 1);
     for (int64_t r0 = 0; r0 < B.rows; r0 += step) {
-        cudaError_t e = cudaMemsetAsync(counter, 0, 8, st);
+        cudaError_t e = r0 > 0 ? cudaMemsetAsync(counter, 0, 8, st) : cudaSuccess;
         if (e == cudaSuccess)
             e = impact::launch_walk_fp32(W.index(), r0, std::min(B.rows, r0 + step),
                                          B.rec_max, B.work_max, warps, mode, o,
@@ -402,10 +402,10 @@ cudaError_t walk_pass64(const Batch &B, const Work &W, bool emit, const impact::
 {
     const int64_t step = chunk_rows > 0 ? chunk_rows : std::max<int64_t>(B.rows, 1);
     for (int64_t r0 = 0; r0 < B.rows; r0 += step) {
-        cudaError_t e = cudaMemsetAsync(counter, 0, 8, st);
+        cudaError_t e = r0 > 0 ? cudaMemsetAsync(counter, 0, 8, st) : cudaSuccess;
         if (e == cudaSuccess)
             e = impact::launch_walk64(W.index(), r0, std::min(B.rows, r0 + step), B.warp64, emit, o,
-                                      counter, st);
+                                      (double *)W.lb(), B.rows, counter, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -432,26 +432,27 @@ impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cu
         CK(impact::launch_leaf_fp32(W.index(), B.leaf_begin.back(), B.leaf_smem, st));
         CK(walk_pass(B, W, WALK_COUNT, B.tune.count_warps, o, W.counter(), chunk_rows, st));
         CK(impact::launch_terms_fp32(W.index(), B.rows, W.lb(), B.tune.faults.fault_row, o, st));
-        CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st));
+        CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st, W.total()));
         return IMPACT_OK;
     }
     if (B.any64) {
         CK(impact::launch_items64(W.index(), B.item_begin.back(), W.status(), st));
-        CK(impact::launch_terms64(W.index(), B.rows, out->sink_lo, out->sink_up, out->trunc, st));
         CK(walk_pass64(B, W, false, o, W.counter(), chunk_rows, st));
+        CK(impact::launch_terms64(W.index(), B.rows, (const double *)W.lb(), o, st));
     }
     for (int q = 0; q < B.count(); ++q)
         if (!B.plans[q].desc.walk64)
             CK(impact::launch_rows(W.desc(q), B.prec, false, 0, B.plans[q].rows,
                                    shifted(o, B.row_begin[q], B.rows), st));
-    CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st));
+    CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st, W.total()));
     return IMPACT_OK;
 }
 
 // emit pass at the row pointers in out->row_ptr
 impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
-                       bool records_ready, cudaStream_t st, int64_t chunk_rows)
+                       bool records_ready, cudaStream_t st, int64_t chunk_rows, bool fresh)
 {
+    if (!fresh) CK(cudaMemsetAsync(W.status(), 0, 64, st));
     impact::RowOutputs o{out->row_ptr, out->col, out->lo, out->up, nullptr, nullptr, nullptr,
                          nullptr, W.status(), capacity, B.rows};
     if (B.prec == PREC_FP32_SOUND) {
@@ -524,6 +525,12 @@ impact_status pair_view(const impact_csr *out, impact_csr &v)
 // the three phases behind the entry points
 // ---------------------------------------------------------------------------
 
+// The head of the status block (Work::status), read back in one copy.
+struct Outcome {
+    uint32_t status = 0, abort = 0;
+    int64_t nnz = 0;
+};
+
 impact_status do_count(const Batch &B, impact_csr *out, cudaStream_t st)
 {
     impact_status s;
@@ -535,15 +542,13 @@ impact_status do_count(const Batch &B, impact_csr *out, cudaStream_t st)
     if (!W.owned) ws_tag(W.base, 0);
     if ((s = upload(B, W, st)) != IMPACT_OK) return s;
     if ((s = run_count(B, W, out, st)) != IMPACT_OK) return s;
-    int64_t nnz = 0;
-    uint32_t status = 0;
-    CK(cudaMemcpyAsync(&nnz, out->row_ptr + B.rows, 8, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&status, W.status(), 4, cudaMemcpyDeviceToHost, st));
+    Outcome r;
+    CK(cudaMemcpyAsync(&r, W.status(), sizeof(r), cudaMemcpyDeviceToHost, st));
     if ((s = release(W, st)) != IMPACT_OK) return s;
     CK(cudaStreamSynchronize(st));
     out->rows = B.rows;
-    out->nnz = nnz;
-    s = status_result(status);
+    out->nnz = r.nnz;
+    s = status_result(r.status);
     if (!W.owned && (s == IMPACT_OK || s == IMPACT_ERR_UNSOUND)) ws_tag(out->workspace, B.hash);
     return s;
 }
@@ -566,12 +571,8 @@ impact_status do_emit(const Batch &B, impact_csr *out, cudaStream_t st)
     Work W;
     if ((s = get_work(B, out, st, W)) != IMPACT_OK) return s;
     WorkHold hold{W, st};
-    if (!ready) {
-        if ((s = upload(B, W, st)) != IMPACT_OK) return s;
-    } else {
-        CK(cudaMemsetAsync(W.status(), 0, 64, st));
-    }
-    if ((s = run_emit(B, W, &view, out->nnz, ready, st)) != IMPACT_OK) return s;
+    if (!ready && (s = upload(B, W, st)) != IMPACT_OK) return s;
+    if ((s = run_emit(B, W, &view, out->nnz, ready, st, 0, false)) != IMPACT_OK) return s;
     uint32_t status = 0;
     CK(cudaMemcpyAsync(&status, W.status(), 4, cudaMemcpyDeviceToHost, st));
     if ((s = release(W, st)) != IMPACT_OK) return s;
@@ -602,7 +603,7 @@ impact_status build_into(const Batch &B, impact_csr *out, bool lib_owned, cudaSt
     if (lib_owned) {   // the output size is known after the count pass
         if ((s = run_count(B, W, out, st)) != IMPACT_OK) return s;
         int64_t nnz = 0;
-        CK(cudaMemcpyAsync(&nnz, out->row_ptr + B.rows, 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(&nnz, W.total(), 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         size_t k = (size_t)std::max<int64_t>(nnz, 1);
         CK(dev_malloc_async(&out->col, k * 4, st));
@@ -617,18 +618,16 @@ impact_status build_into(const Batch &B, impact_csr *out, bool lib_owned, cudaSt
         if ((s = pair_view(out, view)) != IMPACT_OK) return s;
         if ((s = run_fused(B, W, &view, capacity, st)) != IMPACT_OK) return s;
     }
-    int64_t nnz = 0;
-    uint32_t status = 0;
-    CK(cudaMemcpyAsync(&nnz, out->row_ptr + B.rows, 8, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&status, W.status(), 4, cudaMemcpyDeviceToHost, st));
+    Outcome r;
+    CK(cudaMemcpyAsync(&r, W.status(), sizeof(r), cudaMemcpyDeviceToHost, st));
     if ((s = release(W, st)) != IMPACT_OK) return s;
     CK(cudaStreamSynchronize(st));
     out->rows = B.rows;
-    out->nnz = nnz;
-    if (status & IMPACT_STATUS_CAPACITY)
+    out->nnz = r.nnz;
+    if (r.status & IMPACT_STATUS_CAPACITY)
         return fail(IMPACT_ERR_CAPACITY, "output capacity " + std::to_string(capacity) +
-                                             " < needed pairs " + std::to_string(nnz));
-    return status_result(status);
+                                             " < needed pairs " + std::to_string(r.nnz));
+    return status_result(r.status);
 }
 
 impact_status do_build(const Batch &B, impact_csr *out, cudaStream_t st)
@@ -758,7 +757,7 @@ using namespace impact;
 struct impact_graph {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    int64_t *h_result = nullptr;   // pinned: [0] nnz, [1] status
+    impact::Outcome *h_result = nullptr;   // pinned
     unsigned char *own_ws = nullptr;
     int64_t rows = 0, capacity = 0;
 };
@@ -926,7 +925,7 @@ impact_status impact_graph_create(const impact_request *reqs, int count,
         if (e != cudaSuccess) return cleanup(fail(IMPACT_ERR_OOM, cudaGetErrorString(e)));
         W.base = g->own_ws;
     }
-    if (host_malloc(&g->h_result, 16) != cudaSuccess)
+    if (host_malloc(&g->h_result, sizeof(Outcome)) != cudaSuccess)
         return cleanup(fail(IMPACT_ERR_OOM, "pinned result word"));
     if ((s = upload(B, W, st)) != IMPACT_OK) return cleanup(s);
     if (cudaStreamSynchronize(st) != cudaSuccess)
@@ -940,8 +939,7 @@ impact_status impact_graph_create(const impact_request *reqs, int count,
     if (e == cudaSuccess) {
         s = run_fused(B, W, &o, g->capacity, cs);
         if (s == IMPACT_OK) {
-            cudaMemcpyAsync(g->h_result, o.row_ptr + B.rows, 8, cudaMemcpyDeviceToHost, cs);
-            cudaMemcpyAsync(g->h_result + 1, W.status(), 4, cudaMemcpyDeviceToHost, cs);
+            cudaMemcpyAsync(g->h_result, W.status(), sizeof(Outcome), cudaMemcpyDeviceToHost, cs);
         }
         cudaError_t e2 = cudaStreamEndCapture(cs, &g->graph);
         if (s == IMPACT_OK && e2 != cudaSuccess) s = fail(IMPACT_ERR_CUDA, cudaGetErrorString(e2));
@@ -959,8 +957,8 @@ impact_status impact_graph_create(const impact_request *reqs, int count,
 impact_status impact_graph_launch(impact_graph *graph, void *stream)
 {
     if (!graph || !graph->exec) return fail(IMPACT_ERR_ARG, "null graph");
-    graph->h_result[0] = -1;
-    graph->h_result[1] = 0;
+    graph->h_result->nnz = -1;
+    graph->h_result->status = 0;
     CK(cudaGraphLaunch(graph->exec, (cudaStream_t)stream));
     return IMPACT_OK;
 }
@@ -968,8 +966,8 @@ impact_status impact_graph_launch(impact_graph *graph, void *stream)
 impact_status impact_graph_result(impact_graph *graph, int64_t *nnz)
 {
     if (!graph) return fail(IMPACT_ERR_ARG, "null graph");
-    const int64_t got = graph->h_result[0];
-    const uint32_t status = (uint32_t)graph->h_result[1];
+    const int64_t got = graph->h_result->nnz;
+    const uint32_t status = graph->h_result->status;
     if (nnz) *nnz = got;
     if (got < 0) return fail(IMPACT_ERR_ARG, "no finished launch: synchronize the stream first");
     if (status & IMPACT_STATUS_CAPACITY)
@@ -1025,7 +1023,7 @@ impact_status impact_batch_tune(const impact_request *reqs, int count,
         for (int i = 0; i < reps; ++i) {
             CK(cudaEventRecord(e0, st));
             impact_status r = pass == 0 ? run_count(B, W, out, st)
-                                        : run_emit(B, W, out, out->nnz, true, st);
+                                        : run_emit(B, W, out, out->nnz, true, st, 0, false);
             if (r != IMPACT_OK) return r;
             CK(cudaEventRecord(e1, st));
             CK(cudaEventSynchronize(e1));

@@ -291,12 +291,15 @@ rows_fp64(const ImpactDesc *__restrict__ Dp, int64_t row_begin, int64_t row_end,
 }
 
 // ---------------------------------------------------------------------------
-// Exclusive scan of the per-row counts (in place in row_ptr), 3 passes.
+// Exclusive scan of the per-row counts (in place in row_ptr): tile sums, then
+// every tile adds up the sums before it and applies its own scan. One tile
+// needs no sums; beyond kScanSelf tiles a pass over the sums comes between.
 // ---------------------------------------------------------------------------
 
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;
+constexpr int64_t kScanSelf = 4 * kScanThreads;   // tile sums a block adds up itself
 
 __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t *sh, int64_t &total)
 {
@@ -339,8 +342,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles(const int64_t *__rest
     if (threadIdx.x == 0) tsum[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_sums(int64_t *__restrict__ tsum, int64_t nt,
-                                                          int64_t *__restrict__ grand)
+__global__ void __launch_bounds__(kScanThreads) scan_sums(int64_t *__restrict__ tsum, int64_t nt)
 {
     __shared__ int64_t sh[32];
     int64_t carry = 0;
@@ -352,13 +354,25 @@ __global__ void __launch_bounds__(kScanThreads) scan_sums(int64_t *__restrict__ 
         if (i < nt) tsum[i] = carry + ex;
         carry += total;
     }
-    if (threadIdx.x == 0) *grand = carry;
 }
 
+// SELF: toff holds the tiles' sums (unused by the first tile), else their
+// offsets. The last block also stores the total, in *total and *also.
+template <bool SELF>
 __global__ void __launch_bounds__(kScanThreads) scan_apply(int64_t *__restrict__ v, int64_t n,
-                                                           const int64_t *__restrict__ toff)
+                                                           const int64_t *__restrict__ toff,
+                                                           int64_t *__restrict__ total,
+                                                           int64_t *__restrict__ also)
 {
     __shared__ int64_t sh[32];
+    int64_t before = 0;
+    if (SELF) {
+        int64_t s = 0;
+        for (int i = threadIdx.x; i < blockIdx.x; i += kScanThreads) s += toff[i];
+        if (blockIdx.x > 0) block_excl_scan(s, sh, before);
+    } else {
+        before = toff[blockIdx.x];
+    }
     int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
     int64_t loc[kScanItems];
     int64_t s = 0;
@@ -367,12 +381,16 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply(int64_t *__restrict__
         loc[k] = (base + k < n) ? v[base + k] : 0;
         s += loc[k];
     }
-    int64_t total;
-    int64_t ex = block_excl_scan(s, sh, total) + toff[blockIdx.x];
+    int64_t sum;
+    int64_t ex = block_excl_scan(s, sh, sum) + before;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         if (base + k < n) v[base + k] = ex;
         ex += loc[k];
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        *total = before + sum;
+        if (also) *also = before + sum;
     }
 }
 
@@ -1117,13 +1135,20 @@ int64_t scan_scratch_elems(int64_t n)
     return (n + kScanTile - 1) / kScanTile + 1;
 }
 
-cudaError_t launch_scan(int64_t *row_ptr, int64_t n, int64_t *scratch, cudaStream_t stream)
+cudaError_t launch_scan(int64_t *row_ptr, int64_t n, int64_t *scratch, cudaStream_t stream,
+                        int64_t *also)
 {
     int64_t nt = (n + kScanTile - 1) / kScanTile;
     if (nt < 1) nt = 1;
-    scan_tiles<<<(unsigned)nt, kScanThreads, 0, stream>>>(row_ptr, n, scratch);
-    scan_sums<<<1, kScanThreads, 0, stream>>>(scratch, nt, row_ptr + n);
-    scan_apply<<<(unsigned)nt, kScanThreads, 0, stream>>>(row_ptr, n, scratch);
+    if (nt > 1) scan_tiles<<<(unsigned)nt, kScanThreads, 0, stream>>>(row_ptr, n, scratch);
+    if (nt <= kScanSelf) {
+        scan_apply<true><<<(unsigned)nt, kScanThreads, 0, stream>>>(row_ptr, n, scratch,
+                                                                    row_ptr + n, also);
+    } else {
+        scan_sums<<<1, kScanThreads, 0, stream>>>(scratch, nt);
+        scan_apply<false><<<(unsigned)nt, kScanThreads, 0, stream>>>(row_ptr, n, scratch,
+                                                                     row_ptr + n, also);
+    }
     return cudaGetLastError();
 }
 

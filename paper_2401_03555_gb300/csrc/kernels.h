@@ -144,19 +144,23 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
                              int rec_max, const int work_max[3], int warps, int mode,
                              const RowOutputs &o,
                              unsigned long long *lb, const WalkFaults &f, cudaStream_t stream);
-// FP64 path (walk_fp64.cu): item tables, per-row terms, the walk (launches of
-// one pass cover row ranges in order; *counter zeroed before each). The
+// FP64 path (walk_fp64.cu): item tables, the walk (launches of one pass cover
+// row ranges in order; *counter zeroed before each; a count leaves 3 doubles
+// per row in `acc`, [3][rows of the batch]), then the per-row terms. The
 // planner calls size_items64 (item layout and whether the build takes this
 // path: ImpactDesc.walk64; returns the bytes of the build's items).
 int64_t size_items64(ImpactDesc &D, int64_t nnz_bound);
 int64_t walk64_bytes(const ImpactDesc &D);   // shared memory of one warp
 cudaError_t launch_items64(const BatchIndex *d_index, int64_t units, uint32_t *status,
                            cudaStream_t stream);
-cudaError_t launch_terms64(const BatchIndex *d_index, int64_t rows, double *sink_lo,
-                           double *sink_up, double *trunc, cudaStream_t stream);
+cudaError_t launch_terms64(const BatchIndex *d_index, int64_t rows, const double *acc,
+                           const RowOutputs &o, cudaStream_t stream);
 cudaError_t launch_walk64(const BatchIndex *d_index, int64_t row_begin, int64_t row_end,
-                          int warp_smem, bool emit, const RowOutputs &o,
-                          unsigned long long *counter, cudaStream_t stream);
-cudaError_t launch_scan(int64_t *row_ptr, int64_t n, int64_t *scratch, cudaStream_t stream);
+                          int warp_smem, bool emit, const RowOutputs &o, double *acc,
+                          int64_t rows, unsigned long long *counter, cudaStream_t stream);
+// Row pointers from per-row counts, in place; the total goes to row_ptr[n] and
+// to *also (may be null).
+cudaError_t launch_scan(int64_t *row_ptr, int64_t n, int64_t *scratch, cudaStream_t stream,
+                        int64_t *also = nullptr);
 
 }  // namespace impact

@@ -140,6 +140,7 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     o.total_at = B.rows;
     const ImpactDesc *desc = W.desc(0);
     cudaError_t e = cudaMemsetAsync(bad, 0, 4, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(W.status(), 0, 64, st);
     if (e == cudaSuccess)
         e = launch_mc_prep(samples, n, S, keys, val, val_dn, val_up, bad, range, st);
     unsigned char *mask = W.base + W.L.extra;

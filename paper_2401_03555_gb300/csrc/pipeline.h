@@ -44,8 +44,9 @@ struct BatchLayout {
     std::vector<size_t> tables;            // per build: its descriptor and tables
     std::vector<impact::TableLayout> tl;
     size_t upload_end = 0;                 // [0, upload_end) is copied from the host
-    size_t status = 0, counter = 0, scan = 0;
-    size_t lb = 0;                         // FP32: 16 bytes per row (look-back word, or sums)
+    size_t status = 0, scan = 0;
+    size_t lb = 0;                         // per row: 16 bytes (FP32 look-back word, or the
+                                           // count's sums), 24 (FP64 sums)
     std::vector<size_t> rec;               // per build: FP32 per-row records
     std::vector<size_t> item, leaf;        // per build: item tables, FP32 leaf tables
     std::vector<size_t> term;              // per build: FP32 (row, dimension) numbers
@@ -61,8 +62,11 @@ struct Work {
     BatchLayout L;
     bool owned = false;
     const BatchIndex *index() const { return (const BatchIndex *)(base + L.index); }
+    // 64 bytes: the status word and the look-back abort flag, the pair total,
+    // the row counters of the count and the emit walk
     uint32_t *status() const { return (uint32_t *)(base + L.status); }
-    unsigned long long *counter() const { return (unsigned long long *)(base + L.counter); }
+    int64_t *total() const { return (int64_t *)(base + L.status) + 1; }
+    unsigned long long *counter() const { return (unsigned long long *)(base + L.status) + 2; }
     int64_t *scan() const { return (int64_t *)(base + L.scan); }
     unsigned long long *lb() const { return (unsigned long long *)(base + L.lb); }
     const ImpactDesc *desc(int q) const
@@ -80,9 +84,11 @@ impact_status upload(const Batch &B, Work &W, cudaStream_t st);
 impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cudaStream_t st,
                         int64_t chunk_rows = 0);
 // emit pass into out's pair arrays at the row pointers of a count pass
-// (`records_ready`: W holds the FP32 row records of that count pass).
+// (`records_ready`: W holds the records or items of that count pass; `fresh`:
+// W's status block is as a count left it, or zeroed).
 impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
-                       bool records_ready, cudaStream_t st, int64_t chunk_rows = 0);
+                       bool records_ready, cudaStream_t st, int64_t chunk_rows = 0,
+                       bool fresh = true);
 // FP32: count and emit in one pass (capacity known); FP64: count, scan, emit.
 impact_status run_fused(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
                         cudaStream_t st, int64_t chunk_rows = 0);

@@ -214,6 +214,7 @@ double normal_quantile_upper(double p)
     double lo = 0.0, hi = 40.0;
     for (int it = 0; it < 200; ++it) {
         double mid = 0.5 * (lo + hi);
+        if (mid == lo || mid == hi) break;   // neighbouring doubles
         if (0.5 * erfc(mid * M_SQRT1_2) <= p) hi = mid; else lo = mid;
     }
     return hi;

@@ -1626,7 +1626,10 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
                                  row == A.stall_row, prefix);
                 if (lane == 0 && lb_ok) {
                     A.row_ptr[row] = prefix;
-                    if (row == B->rows - 1) A.row_ptr[B->rows] = prefix + c;
+                    if (row == B->rows - 1) {   // the total, also beside the status
+                        A.row_ptr[B->rows] = prefix + c;
+                        reinterpret_cast<int64_t *>(A.status)[1] = prefix + c;
+                    }
                 }
                 base = prefix;
                 len = c;

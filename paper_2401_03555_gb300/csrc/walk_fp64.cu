@@ -9,8 +9,6 @@
 //               of the cells between from neighbouring lanes; then the trimmed
 //               window, its sums and, for the last dimension, the targets
 //               sorted by upper factor with prefix sums.
-//   terms_fp64  one thread per row: sink bounds and the mass outside the
-//               window box, products of per-item numbers.
 //   walk_fp64   one warp per row: the prefix tree of target cells level by
 //               level in C order over the dimensions but the last, as in the
 //               FP32 walk; a node is dropped when even the largest later
@@ -18,6 +16,8 @@
 //               many targets of the last dimension pass under each parent by a
 //               search in the sorted table (RN(P u) is monotone in u), the
 //               emit pass tests every target under every parent, one lane each.
+//   terms_fp64  after the count, one thread per row: sink bounds, truncated mass
+//               and row checks.
 //
 // What bounds it: FP64 issue (2 lanes per clock and SM on this part, so a
 // warp-wide multiply holds the pipe 16 clocks) and the 20 bytes a pair writes.
@@ -245,9 +245,12 @@ items_fp64(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
     }
 }
 
+// Row terms after the count walk (acc: its dropped mass, upper and lower sums
+// per row).
 __global__ void __launch_bounds__(256)
-terms_fp64(const BatchIndex *__restrict__ B, double *__restrict__ sink_lo,
-           double *__restrict__ sink_up, double *__restrict__ trunc)
+terms_fp64(const BatchIndex *__restrict__ B, const double *__restrict__ acc,
+           double *__restrict__ sink_lo, double *__restrict__ sink_up, double *__restrict__ trunc,
+           uint32_t *__restrict__ flags, uint32_t *__restrict__ status)
 {
     for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < B->rows;
          row += (int64_t)gridDim.x * blockDim.x) {
@@ -260,19 +263,30 @@ terms_fp64(const BatchIndex *__restrict__ B, double *__restrict__ sink_lo,
         // sink: 1 - prod of the in-domain masses. Outside the window box,
         // partitioned by the first dimension that leaves its window:
         // sum_k prod_{i<k} SW_i * O_k * prod_{i>k} (SW_i + O_i)
-        double pmax = 1.0, pmin = 1.0, acc = 0.0, pre = 1.0;
-        for (int d = 0; d < D.n; ++d) {
-            const ImpactDim &g = D.dim[d];
-            const Item64 *h = reinterpret_cast<const Item64 *>(
-                B->items[q] + g.item_off + item_of(D, r, idx, j, d) * g.item_stride);
-            pmax *= h->gmax;
-            pmin *= h->gmin;
-            acc = acc * (h->SW + h->O) + pre * h->O;
-            pre *= h->SW;
+        double pmax = 1.0, pmin = 1.0, out = 0.0, pre = 1.0;
+#pragma unroll
+        for (int d = 0; d < IMPACT_MAX_DIM; ++d) {
+            if (d < D.n) {
+                const ImpactDim &g = D.dim[d];
+                const Item64 *h = reinterpret_cast<const Item64 *>(
+                    B->items[q] + g.item_off + item_of(D, r, idx, j, d) * g.item_stride);
+                pmax *= h->gmax;
+                pmin *= h->gmin;
+                out = out * (h->SW + h->O) + pre * h->O;
+                pre *= h->SW;
+            }
         }
-        sink_lo[row] = 1.0 - pmax;
-        sink_up[row] = 1.0 - pmin;
-        trunc[row] = acc;
+        const double sl = 1.0 - pmax, su = 1.0 - pmin, tr = out + acc[row];
+        sink_lo[row] = sl;
+        sink_up[row] = su;
+        trunc[row] = tr;
+        if (flags) {
+            uint32_t f = 0;
+            if (acc[2 * B->rows + row] + sl > 1.0 + 1e-12) f |= 0x1u;
+            if (acc[B->rows + row] + su + tr < 1.0 - 1e-12) f |= 0x2u;
+            flags[row] = f;
+            if (f) atomicOr(status, IMPACT_STATUS_UNSOUND);
+        }
     }
 }
 
@@ -324,8 +338,27 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
+// Sums of three values over the warp; lane k (k < 3) gets the k-th in x[0]. The
+// lanes share the work (7 FP64 adds a lane and not 15: the pipe is busy 16
+// clocks with each, whatever share of the lanes is active).
+__device__ __forceinline__ void warp_sums(double (&x)[3], int lane)
+{
+    const unsigned m = 0xffffffffu;
+    // halves keep (x0, x1) or (x2, -), quarters one of them each
+    double a = lane & 16 ? x[2] : x[0], b = lane & 16 ? 0.0 : x[1];
+    const double ga = lane & 16 ? x[0] : x[2], gb = lane & 16 ? x[1] : 0.0;
+    a += __shfl_xor_sync(m, ga, 16);
+    b += __shfl_xor_sync(m, gb, 16);
+    double v = lane & 8 ? b : a;
+    v += __shfl_xor_sync(m, lane & 8 ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(m, v, o);
+    // lanes 0, 8, 16 hold x0, x1, x2
+    x[0] = __shfl_sync(m, v, (lane & 3) * 8);
+}
+
 struct Sums64 {
-    long long cnt = 0;
+    int cnt = 0;
     double drop = 0.0, sup = 0.0, slo = 0.0;
 };
 
@@ -508,9 +541,8 @@ struct Walk64Args {
     int64_t *row_ptr;          // COUNT: per-row counts; EMIT: row pointers
     int32_t *col;
     double *lo, *up;
-    double *trunc;             // COUNT: outside mass in, full truncated mass out
-    const double *sink_lo, *sink_up;
-    uint32_t *flags;
+    double *acc;               // COUNT: [3][rows] dropped mass, upper and lower sums
+    int64_t rows;
     uint32_t *status;
     int64_t capacity, total_at;
     int64_t row_begin, row_end;
@@ -655,28 +687,12 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
             int64_t w0 = 0;
             bool ok = true;
             if (!empty) ok = walk_row64<false>(S, n, lane, acc, none, w0, cut, cutb, sorted);
-            long long cnt = acc.cnt;
-            double drop = acc.drop, sup = acc.sup, slo = acc.slo;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-                drop += __shfl_xor_sync(0xffffffffu, drop, o);
-                sup += __shfl_xor_sync(0xffffffffu, sup, o);
-                slo += __shfl_xor_sync(0xffffffffu, slo, o);
-            }
-            if (lane == 0) {
-                A.row_ptr[row] = ok ? cnt : 0;
-                const double tr = A.trunc[row] + drop;
-                A.trunc[row] = tr;
-                if (!ok) atomicOr(A.status, IMPACT_STATUS_INTERNAL);
-                if (A.flags) {
-                    uint32_t f = 0;
-                    if (slo + A.sink_lo[row] > 1.0 + 1e-12) f |= 0x1u;
-                    if (sup + A.sink_up[row] + tr < 1.0 - 1e-12) f |= 0x2u;
-                    A.flags[row] = f;
-                    if (f) atomicOr(A.status, IMPACT_STATUS_UNSOUND);
-                }
-            }
+            const int cnt = __reduce_add_sync(0xffffffffu, acc.cnt);
+            double sum[3] = {acc.drop, acc.sup, acc.slo};
+            warp_sums(sum, lane);
+            if (lane == 0) A.row_ptr[row] = ok ? cnt : 0;
+            if (lane < 3) A.acc[lane * A.rows + row] = sum[0];
+            if (lane == 0 && !ok) atomicOr(A.status, IMPACT_STATUS_INTERNAL);
         }
         __syncwarp();   // every lane is done with the row's tables
     }
@@ -736,21 +752,22 @@ cudaError_t launch_items64(const BatchIndex *d_index, int64_t units, uint32_t *s
     return cudaGetLastError();
 }
 
-cudaError_t launch_terms64(const BatchIndex *d_index, int64_t rows, double *sink_lo,
-                           double *sink_up, double *trunc, cudaStream_t stream)
+cudaError_t launch_terms64(const BatchIndex *d_index, int64_t rows, const double *acc,
+                           const RowOutputs &o, cudaStream_t stream)
 {
     if (rows <= 0) return cudaSuccess;
     const int g = blocks_for((const void *)terms_fp64, 256, 0, rows, 256);
-    terms_fp64<<<g, 256, 0, stream>>>(d_index, sink_lo, sink_up, trunc);
+    terms_fp64<<<g, 256, 0, stream>>>(d_index, acc, o.sink_lo, o.sink_up, o.trunc, o.flags,
+                                      o.status);
     return cudaGetLastError();
 }
 
 cudaError_t launch_walk64(const BatchIndex *d_index, int64_t row_begin, int64_t row_end,
-                          int warp_smem, bool emit, const RowOutputs &o,
-                          unsigned long long *counter, cudaStream_t stream)
+                          int warp_smem, bool emit, const RowOutputs &o, double *acc,
+                          int64_t rows, unsigned long long *counter, cudaStream_t stream)
 {
-    const int64_t rows = row_end - row_begin;
-    if (rows <= 0) return cudaSuccess;
+    const int64_t span = row_end - row_begin;
+    if (span <= 0) return cudaSuccess;
     const int warps = std::max(1, std::min(kWarps, 200 * 1024 / std::max(warp_smem, 1)));
     const size_t smem = (size_t)warp_smem * warps;
     const void *k = emit ? (const void *)walk_fp64<true> : (const void *)walk_fp64<false>;
@@ -763,18 +780,16 @@ cudaError_t launch_walk64(const BatchIndex *d_index, int64_t row_begin, int64_t 
     A.col = o.col;
     A.lo = (double *)o.lo;
     A.up = (double *)o.up;
-    A.trunc = o.trunc;
-    A.sink_lo = o.sink_lo;
-    A.sink_up = o.sink_up;
-    A.flags = o.flags;
+    A.acc = acc;
+    A.rows = rows;
     A.status = o.status;
     A.capacity = o.capacity;
     A.total_at = o.total_at;
     A.row_begin = row_begin;
     A.row_end = row_end;
     A.next_row = counter;
-    const int g = blocks_for(k, warps * 32, smem, rows, warps);
-    A.row_block = (int)std::max<int64_t>(1, std::min<int64_t>(4, rows / ((int64_t)g * warps * 64)));
+    const int g = blocks_for(k, warps * 32, smem, span, warps);
+    A.row_block = (int)std::max<int64_t>(1, std::min<int64_t>(4, span / ((int64_t)g * warps * 64)));
     if (emit) walk_fp64<true><<<g, warps * 32, smem, stream>>>(A);
     else walk_fp64<false><<<g, warps * 32, smem, stream>>>(A);
     return cudaGetLastError();
