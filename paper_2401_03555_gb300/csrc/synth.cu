@@ -71,6 +71,38 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// Sums of a value per vector over the warp: the lower half-warp gets V0's sum,
+// the upper V1's, each the bits of warp_sum (the same tree of additions). Five
+// adds and not ten: the FP64 pipe is busy as long with one active lane as with
+// 32, so the halves work side by side.
+__device__ __forceinline__ double half_sum(double v0, double v1, int lane)
+{
+    const unsigned m = 0xffffffffu;
+    double x = lane & 16 ? v1 : v0;
+    x += __shfl_xor_sync(m, lane & 16 ? v0 : v1, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(m, x, o);
+    return x;
+}
+
+// The same for two values per vector (a, b): six adds and not twenty.
+__device__ __forceinline__ void half_sums(const double (&a)[2], const double (&b)[2], int lane,
+                                          double &sa, double &sb)
+{
+    const unsigned m = 0xffffffffu;
+    const bool up = lane & 16, right = lane & 8;
+    double x = up ? a[1] : a[0], y = up ? b[1] : b[0];
+    x += __shfl_xor_sync(m, up ? a[0] : a[1], 16);
+    y += __shfl_xor_sync(m, up ? b[0] : b[1], 16);
+    double s = right ? y : x;
+    s += __shfl_xor_sync(m, right ? x : y, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(m, s, o);
+    const double other = __shfl_xor_sync(m, s, 8);
+    sa = right ? other : s;
+    sb = right ? s : other;
+}
+
 // Order-preserving integer key of a finite double (-0 and +0 share key 0):
 // x <= y exactly when okey(x) <= okey(y).
 __device__ __forceinline__ long long okey(double x)
@@ -113,11 +145,18 @@ struct Step {
 
 struct RowRef {
     int64_t a, b;           // successor range in col/lo/up
-    // three further successors: the sink and an empty one, or the two
-    // regions; then the truncated mass. Widths and values (before the max LP's
-    // mapping v -> 1 - v, and 0 or 1); the lower bounds are in `rest`
-    double xlo[3], xw[3], xv[3];
+    // three further successors: the sink and an empty one, or the two regions;
+    // then the truncated mass. Bounds, widths, and whether the min LP sees them
+    // with value 1 (else 0)
+    double xlo[3], xw[3];
+    bool one[3];
     double rest;            // 1 - sum of all lower bounds
+};
+
+// Mass the lower bounds of a row leave and widths of its further successors,
+// in 2^-52 units.
+struct RowFix {
+    long long rest, xw[3];
 };
 
 // Sum over the warp of 64-bit integers: three 32-bit warp sums of 27-bit pieces.
@@ -131,21 +170,22 @@ __device__ __forceinline__ long long warp_sum_ll(long long x)
 }
 
 // Greedy (sorting-method) optimum of one row for both value vectors at once:
-// res[0] for V0 (the remaining mass valued low), res[1] for V1 (valued high).
+// for V0 (the remaining mass valued low) in the lower half-warp, for V1 (valued
+// high) in the upper.
 // `excl`: when not null, successors t with excl[t] != 0 are left out (their
 // mass is in the region successors). Short rows (SHORT: at most 512) load their
 // successors in unrolled, independent steps and keep ranks and widths in
 // registers for the whole bisection; long rows read them again in every pass.
 template <typename VT, bool PACKED, bool SHORT>
-__device__ __forceinline__ void row_lp(const RowRef &R, const int32_t *__restrict__ col,
-                                       const VT *__restrict__ lo, const VT *__restrict__ up,
-                                       const long long *__restrict__ wfix,
-                                       const uint8_t *__restrict__ excl, const Seen &Q,
-                                       bool maximize, double *res)
+__device__ __forceinline__ double row_lp(const RowRef &R, const RowFix &F,
+                                         const int32_t *__restrict__ col,
+                                         const VT *__restrict__ lo, const VT *__restrict__ up,
+                                         const long long *__restrict__ wfix,
+                                         const uint8_t *__restrict__ excl, const Seen &Q,
+                                         bool maximize)
 {
     constexpr int kKeep = SHORT ? kCache : 1;
     const int lane = threadIdx.x & 31;
-    auto val = [&](double v) { return maximize ? 1.0 - v : v; };
     auto out = [&](int32_t t) { return excl != nullptr && excl[t] != 0; };
     const int len = (int)min(R.b - R.a, (int64_t)INT_MAX);
     double slov[2] = {0.0, 0.0};
@@ -184,31 +224,23 @@ __device__ __forceinline__ void row_lp(const RowRef &R, const int32_t *__restric
             if (!out(t)) lower((double)lo[i], Q.val[t]);
         }
     }
+    double sum = half_sum(slov[0], slov[1], lane);
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        slov[v] = warp_sum(slov[v]);
-#pragma unroll
-        for (int x = 0; x < 3; ++x) slov[v] += R.xlo[x] * val(R.xv[x]);
-    }
-    if (R.rest <= 0.0) {
-        res[0] = maximize ? 1.0 - slov[0] : slov[0];
-        res[1] = maximize ? 1.0 - slov[1] : slov[1];
-        return;
-    }
+    for (int x = 0; x < 3; ++x)
+        if (R.one[x]) sum += R.xlo[x];
+    if (R.rest <= 0.0) return maximize ? 1.0 - sum : sum;
     // G over ranks: mass (2^-52 units) of the successors of rank <= m
-    const long long rest_f = __double2ll_rn(R.rest * 0x1p52);
     long long base = 0, top = 0;   // the further successors of value 0 and 1
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const long long x = __double2ll_rn(R.xw[k] * 0x1p52);
-        if (val(R.xv[k]) > 0.0) top += x; else base += x;
+        if (R.one[k]) top += F.xw[k]; else base += F.xw[k];
     }
     int l[2] = {-1, -1}, h[2] = {Q.one[0], Q.one[1]};
     const int one[2] = {h[0], h[1]};
     auto narrow = [&](int v, int m, long long g) {
         if (h[v] - l[v] <= 1) return;
         g += base + (m >= one[v] ? top : 0);
-        if (g >= rest_f) h[v] = m; else l[v] = m;
+        if (g >= F.rest) h[v] = m; else l[v] = m;
     };
     while (h[0] - l[0] > 1 || h[1] - l[1] > 1) {
         const int m0 = l[0] + ((h[0] - l[0]) >> 1), m1 = l[1] + ((h[1] - l[1]) >> 1);
@@ -235,7 +267,7 @@ __device__ __forceinline__ void row_lp(const RowRef &R, const int32_t *__restric
     }
     // the mass below tau and its weighted value, in FP64 (nothing is below
     // when no mass is left to place)
-    const int cut0 = rest_f > 0 ? h[0] : 0, cut1 = rest_f > 0 ? h[1] : 0;
+    const int cut0 = F.rest > 0 ? h[0] : 0, cut1 = F.rest > 0 ? h[1] : 0;
     double g[2] = {0.0, 0.0}, gv[2] = {0.0, 0.0};
     auto below = [&](int64_t i, bool b0, bool b1) {
         if (!(b0 || b1)) return;
@@ -266,25 +298,18 @@ __device__ __forceinline__ void row_lp(const RowRef &R, const int32_t *__restric
             below(i, r.x < cut0, r.y < cut1);
         }
     }
+    double below_w, below_v;
+    half_sums(g, gv, lane, below_w, below_v);
+    // tau and the double before it; the further successors of value 0 lie
+    // below it when it is positive (those of value 1 never do)
+    const bool high = lane & 16;
+    const long long kh = F.rest > 0 ? (high ? Q.key[1][h[1]] : Q.key[0][h[0]]) : okey(-1.0) + 1;
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        g[v] = warp_sum(g[v]);
-        gv[v] = warp_sum(gv[v]);
-        // tau and the double before it
-        const long long kh = rest_f > 0 ? Q.key[v][h[v]] : okey(-1.0) + 1;
-        const double xl = from_okey(kh - 1), xh = from_okey(kh);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double y = val(R.xv[k]);
-            if (y <= xl) {
-                g[v] += R.xw[k];
-                gv[v] += R.xw[k] * y;
-            }
-        }
-        const double x = (maximize == (v == 1)) ? xl : xh;
-        const double y = slov[v] + gv[v] + (R.rest - g[v]) * fmax(x, 0.0);
-        res[v] = maximize ? 1.0 - y : y;
-    }
+    for (int k = 0; k < 3; ++k)
+        if (!R.one[k] && kh > 0) below_w += R.xw[k];
+    const double x = from_okey(maximize == high ? kh - 1 : kh);
+    const double y = sum + below_v + (R.rest - below_w) * fmax(x, 0.0);
+    return maximize ? 1.0 - y : y;
 }
 
 struct Phase {
@@ -308,26 +333,29 @@ __device__ __forceinline__ void further(const Phase &ph, const Regions &rg, int6
                                         const double *__restrict__ trunc, RowRef &R)
 {
     const bool reach = ph.spec == IMPACT_REACH_AVOID;
+    bool one[3];   // the successor's value, before the max LP's v -> 1 - v
     if (rg.r_lo) {
         // the target region (reach: value 1) and the avoid region with the
         // sink (safety: value 1)
         R.xlo[0] = rg.r_lo[r];
         R.xw[0] = rg.r_up[r] - rg.r_lo[r];
-        R.xv[0] = reach ? 1.0 : 0.0;
+        one[0] = reach;
         R.xlo[1] = rg.a_lo[r];
         R.xw[1] = rg.a_up[r] - rg.a_lo[r];
-        R.xv[1] = reach ? 0.0 : 1.0;
+        one[1] = !reach;
     } else {
         R.xlo[0] = sink_lo[r];
         R.xw[0] = sink_up[r] - sink_lo[r];
-        R.xv[0] = reach ? 0.0 : 1.0;
+        one[0] = !reach;
         R.xlo[1] = 0.0;
         R.xw[1] = 0.0;
-        R.xv[1] = 0.0;
+        one[1] = false;
     }
     R.xlo[2] = 0.0;
     R.xw[2] = trunc[r];
-    R.xv[2] = ph.maximize ? 1.0 : 0.0;
+    one[2] = ph.maximize;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) R.one[k] = one[k] != ph.maximize;
 }
 
 // What no iteration changes: per pair the width up - lo in 2^-52 units (the
@@ -338,7 +366,7 @@ row_prep(Phase ph, int64_t rows, int64_t per_cell, const uint8_t *__restrict__ l
          const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
          const VT *__restrict__ lo, const VT *__restrict__ up, const double *__restrict__ sink_lo,
          const double *__restrict__ sink_up, const double *__restrict__ trunc, Regions rg,
-         long long *__restrict__ wfix, double *__restrict__ rest)
+         long long *__restrict__ wfix, double *__restrict__ rest, RowFix *__restrict__ fix)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -356,7 +384,15 @@ row_prep(Phase ph, int64_t rows, int64_t per_cell, const uint8_t *__restrict__ l
         slo = warp_sum(slo);
 #pragma unroll
         for (int x = 0; x < 3; ++x) slo += R.xlo[x];
-        if (lane == 0) rest[r] = 1.0 - slo;
+        if (lane == 0) {
+            const double left = 1.0 - slo;
+            rest[r] = left;
+            RowFix f;
+            f.rest = __double2ll_rn(left * 0x1p52);
+#pragma unroll
+            for (int x = 0; x < 3; ++x) f.xw[x] = __double2ll_rn(R.xw[x] * 0x1p52);
+            fix[r] = f;
+        }
     }
 }
 
@@ -370,7 +406,7 @@ row_values(Phase ph, const Step *__restrict__ step, int64_t rows, int n_inputs,
            const int32_t *__restrict__ col, const VT *__restrict__ lo, const VT *__restrict__ up,
            const double *__restrict__ sink_lo, const double *__restrict__ sink_up,
            const double *__restrict__ trunc, const long long *__restrict__ wfix,
-           const double *__restrict__ rest, Regions rg, Seen Q,
+           const double *__restrict__ rest, const RowFix *__restrict__ fix, Regions rg, Seen Q,
            const int32_t *__restrict__ policy, double *__restrict__ R0, double *__restrict__ R1)
 {
     if (step->done) return;
@@ -388,15 +424,13 @@ row_values(Phase ph, const Step *__restrict__ step, int64_t rows, int n_inputs,
         R.b = row_ptr[r + 1];
         R.rest = rest[r];
         further(ph, rg, r, sink_lo, sink_up, trunc, R);
-        double res[2];
-        if (R.b - R.a <= 32 * kCache)
-            row_lp<VT, PACKED, true>(R, col, lo, up, wfix, excl, Q, ph.maximize, res);
-        else
-            row_lp<VT, PACKED, false>(R, col, lo, up, wfix, excl, Q, ph.maximize, res);
-        if (lane == 0) {
-            R0[r] = res[0];
-            R1[r] = res[1];
-        }
+        const RowFix F = fix[r];
+        const double res =
+            R.b - R.a <= 32 * kCache
+                ? row_lp<VT, PACKED, true>(R, F, col, lo, up, wfix, excl, Q, ph.maximize)
+                : row_lp<VT, PACKED, false>(R, F, col, lo, up, wfix, excl, Q, ph.maximize);
+        if (lane == 0) R0[r] = res;
+        if (lane == 16) R1[r] = res;
     }
 }
 
@@ -428,6 +462,7 @@ __device__ __forceinline__ void cell_next(const Phase &ph, int64_t c, int n_inpu
     } else if (ph.choose) {
         double b0 = 0.0, b1 = 0.0;
         int arg0 = 0, arg1 = 0;
+#pragma unroll 4
         for (int j = 0; j < n_inputs; ++j) {
             const double a = worst(R0 + (c * n_inputs + j) * W, W, reach);
             const double b = worst(R1 + (c * n_inputs + j) * W, W, reach);
@@ -774,7 +809,8 @@ extern "C" impact_status impact_synthesize_ex(const impact_csr *imdp, impact_pre
             e = impact::dev_malloc_async(
                 &wfix, (size_t)std::max<int64_t>(nnz, 1) * sizeof(long long), st);
         if (e == cudaSuccess)
-            e = impact::dev_malloc_async(&rbuf, (size_t)rows * 3 * sizeof(double), st);
+            e = impact::dev_malloc_async(&rbuf, (size_t)rows * (3 * sizeof(double) + sizeof(RowFix)),
+                                         st);
         if (e == cudaSuccess) e = impact::dev_malloc_async(&d_step, sizeof(Step), st);
         if (e == cudaSuccess) e = impact::host_malloc(&h_step, 2 * sizeof(Step));
         for (cudaEvent_t &x : seen)
@@ -798,7 +834,8 @@ extern "C" impact_status impact_synthesize_ex(const impact_csr *imdp, impact_pre
     const int g_lp = grid_of(rows, kRowThreads / 32);
     impact_status status = IMPACT_OK;
     int its[2] = {0, 0};
-    double *R0 = rbuf, *R1 = rbuf + rows, *rest = rbuf + 2 * rows;
+    RowFix *fix = (RowFix *)rbuf;
+    double *R0 = (double *)(fix + rows), *R1 = R0 + rows, *rest = R1 + rows;
     const float *lo32 = (const float *)imdp->lo, *up32 = (const float *)imdp->up;
     const double *lo64 = (const double *)imdp->lo, *up64 = (const double *)imdp->up;
     const bool f32 = precision == IMPACT_FP32_SOUND;
@@ -816,11 +853,11 @@ extern "C" impact_status impact_synthesize_ex(const impact_csr *imdp, impact_pre
             if (f32)
                 row_prep<float><<<g_rows, kThreads, 0, st>>>(
                     ph, rows, per_cell, labels, imdp->row_ptr, imdp->col, lo32, up32,
-                    imdp->sink_lo, imdp->sink_up, imdp->trunc, rg, wfix, rest);
+                    imdp->sink_lo, imdp->sink_up, imdp->trunc, rg, wfix, rest, fix);
             else
                 row_prep<double><<<g_rows, kThreads, 0, st>>>(
                     ph, rows, per_cell, labels, imdp->row_ptr, imdp->col, lo64, up64,
-                    imdp->sink_lo, imdp->sink_up, imdp->trunc, rg, wfix, rest);
+                    imdp->sink_lo, imdp->sink_up, imdp->trunc, rg, wfix, rest, fix);
         }
         // the values of step i are in half i & 1; the rest is of the latest
         auto cells_of = [&](int i) {
@@ -865,7 +902,7 @@ extern "C" impact_status impact_synthesize_ex(const impact_csr *imdp, impact_pre
         auto rows_step = [&](auto kernel, auto *lo, auto *up) {
             kernel<<<g_lp, kRowThreads, 0, st>>>(ph, d_step, rows, n_inputs, labels, imdp->row_ptr,
                                                  imdp->col, lo, up, imdp->sink_lo, imdp->sink_up,
-                                                 imdp->trunc, wfix, rest, rg, Q, policy, R0, R1);
+                                                 imdp->trunc, wfix, rest, fix, rg, Q, policy, R0, R1);
         };
         auto iterate = [&](int i) {   // values of step i -> those of step i + 1
             if (f32 && packed) rows_step(row_values<float, true>, lo32, up32);
