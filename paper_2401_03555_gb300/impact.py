@@ -370,7 +370,11 @@ def build(prob, precision="fp32", stream=None, check_unsound: bool = True) -> CS
     prec = _PREC[precision]
     rows = prob.rows
     rb = alloc_rows(rows)
-    ws = alloc_workspace(prob, precision)
+    wb = ctypes.c_int64()
+    _check(lib.impact_workspace_bytes(ctypes.byref(a.sys), ctypes.byref(a.grid),
+                                      ctypes.byref(a.inp), a.sigma_ptr, a.cutoff, prec,
+                                      ctypes.byref(wb)))
+    ws = torch.empty(max(wb.value, 256), dtype=torch.uint8, device="cuda")
     c = _csr_struct(rb, workspace=ws)
     st = _stream_handle(stream)
     status = lib.impact_count(ctypes.byref(a.sys), ctypes.byref(a.grid), ctypes.byref(a.inp),
