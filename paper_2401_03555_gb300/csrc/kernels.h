@@ -83,13 +83,22 @@ struct McMasks {
     int64_t bytes;
 };
 McMasks mc_masks(const ImpactDesc &D, int64_t S, double cutoff);
+// What the count pass keeps for the emit pass: targets and counts of a row
+// from entries[seg[row]] (seg < 0: not kept); *used zeroed before the count.
+struct McKeep {
+    uint2 *entries;
+    int64_t cap;
+    unsigned long long *used;
+    int64_t *seg;                       // [rows]
+};
+int64_t mc_keep_entries(int64_t rows);
 cudaError_t launch_mc_items(const ImpactDesc *d_desc, int n, const McMasks &K,
                             const long long *keys, int64_t S, const double *range,
                             unsigned char *items, cudaStream_t stream);
 cudaError_t launch_mc_walk(const ImpactDesc *d_desc, bool emit, int64_t rows, const McMasks &K,
                            unsigned char *items, int64_t S, const double *val,
                            const float *val_dn, const float *val_up, unsigned kmin,
-                           const RowOutputs &o, cudaStream_t stream);
+                           const McKeep &keep, const RowOutputs &o, cudaStream_t stream);
 
 // Labels of every cell (0 free, 1 target, 2 avoid; avoid wins).
 cudaError_t launch_labels(const RegionBoxes &boxes, int64_t total_cells, uint8_t *labels,

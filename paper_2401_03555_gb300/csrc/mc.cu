@@ -71,7 +71,10 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     if (s != IMPACT_OK) return s;
     B.walks = false;
     const McMasks masks = mc_masks(B.plans[0].desc, n_samples, cutoff);
-    B.extra = masks.bytes;
+    // the masks, the entries a count keeps for the emit, a segment per row
+    const int64_t keep_cap = masks.bytes > 0 ? mc_keep_entries(B.rows) : 0;
+    const int64_t mask_end = (masks.bytes + 255) / 256 * 256;
+    if (masks.bytes > 0) B.extra = mask_end + 8 * keep_cap + 8 * B.rows;
     B.plans[0].desc.cutoff = cutoff;
     B.plans[0].desc.prec = precision;
     configure_pool_once();
@@ -144,9 +147,11 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     if (e == cudaSuccess)
         e = launch_mc_prep(samples, n, S, keys, val, val_dn, val_up, bad, range, st);
     unsigned char *mask = W.base + W.L.extra;
+    const McKeep keep{(uint2 *)(mask + mask_end), keep_cap, W.counter(),
+                      (int64_t *)(mask + mask_end + 8 * keep_cap)};
     auto rows_pass = [&](bool emit) {
         return masks.bytes > 0 ? launch_mc_walk(desc, emit, B.rows, masks, mask, S, val, val_dn,
-                                                val_up, (unsigned)kmin, o, st)
+                                                val_up, (unsigned)kmin, keep, o, st)
                                : launch_mc_rows(desc, emit, B.rows, keys, S, range, val, val_dn,
                                                 val_up, (unsigned)kmin, o, st);
     };
