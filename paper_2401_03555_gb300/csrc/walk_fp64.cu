@@ -23,9 +23,11 @@
 // warp-wide multiply holds the pipe 16 clocks) and the 20 bytes a pair writes.
 // erfc costs about a hundred FP64 instructions: evaluated per pair and
 // dimension it was the whole run time, per image and edge it is little. Whole
-// builds, per-pair kernel -> this one: unicycle 21x19x13 (25.6M pairs) 392 ->
-// 0.88 ms (items 0.07, count 0.35, emit 0.35), room 5x6x5x6x5 304 -> 0.52 ms,
-// dense robot 21x21 14.0 -> 0.35 ms.
+// builds, per-pair kernel -> this one: unicycle 21x19x13 (25.6M pairs) 395 ->
+// 0.56 ms (items 0.05, count 0.22, emit 0.22), room 5x6x5x6x5 303 -> 0.37 ms,
+// dense robot 21x21 14.0 -> 0.27 ms (host-bound). Both walks keep the FP64 pipe
+// 80% busy, so what is not a product stays off it: compares on bits, FP32
+// searches, no conversions.
 #include <cuda_runtime.h>
 #include <float.h>
 #include <limits.h>
@@ -64,9 +66,9 @@ struct Item64 {
 static_assert(sizeof(Item64) == 56, "Item64 layout");
 constexpr int kItemHead = 64;
 
-__host__ __device__ inline bool is_sorted_dim(double cutoff, int w64)
+__host__ __device__ inline bool is_sorted_dim(float cutoff32, int w64)
 {
-    return cutoff > 0.0 && w64 <= kSortMax;
+    return cutoff32 > 0.0f && w64 <= kSortMax;
 }
 
 __device__ __forceinline__ double2 *item_table(unsigned char *it)
@@ -131,21 +133,80 @@ items_fp64(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
         }
         const double cut = D.cutoff, inv_s = g.inv_s;
         // targets k0 .. k0 + G - 2 per step: lane `sub` takes edge k0 + sub,
-        // and the last lane only lends its edge to the one before it
+        // and the last lane only lends its edge to the one before it. The
+        // arguments that no edge gives (the domain's edges at both image ends,
+        // slots 0-3, and at its clamped midpoint, 4-5; targets whose midpoint
+        // lies in the image, two each) share a round of erfc of their own,
+        // one per lane: a warp-wide erfc costs the same for one lane as for 32
         int first = INT_MAX, last = -1;
+        const int shift = lane - sub;
+        const unsigned gmask = G == 32 ? kAll : (1u << G) - 1u;
+        double tx = 0.0, tf = 0.0;             // slots 0-5, in lanes 0-5
+        double ax = 0.0, af = 0.0;             // edge a at m_lo, in lane 0
+        double wx = 0.0, wf = 0.0;             // edge a + W at m_hi, in lane wlane
+        int wlane = 0;
         for (int k0 = 0; k0 < g.w64; k0 += G - 1) {
             const int k = k0 + sub;
             const double c0 = E[min(a + k, g.N)];
             const double x0 = (c0 - mlo) * inv_s, x1 = (c0 - mhi) * inv_s;
             const double f0 = erfc(fabs(x0)), f1 = erfc(fabs(x1));
+            if (k0 == 0) {
+                ax = x0;
+                af = f0;
+            }
+            const unsigned at_w = (__ballot_sync(kAll, k == W) >> shift) & gmask;
+            if (at_w) wlane = __ffs(at_w) - 1;
+            if (k == W) {
+                wx = x1;
+                wf = f1;
+            }
             const double e0 = __shfl_down_sync(kAll, c0, 1, G);
             const double y0 = __shfl_down_sync(kAll, x0, 1, G), y1 = __shfl_down_sync(kAll, x1, 1, G);
             const double h0 = __shfl_down_sync(kAll, f0, 1, G), h1 = __shfl_down_sync(kAll, f1, 1, G);
-            if (sub < G - 1 && k < W) {
+            const bool mine = sub < G - 1 && k < W;
+            const double mid = 0.5 * (c0 + e0);
+            const bool inner = mine && !(mid < mlo) && !(mid > mhi);
+            const unsigned inners = (__ballot_sync(kAll, inner) >> shift) & gmask;
+            const int base = k0 == 0 ? 6 : 0, slots = base + 2 * __popc(inners);
+            const int my_slot = base + 2 * __popc(inners & ((1u << sub) - 1u));
+            const int most = __reduce_max_sync(kAll, slots);
+            double qa = 0.0, qfa = 0.0, qb = 0.0, qfb = 0.0;
+            for (int s0 = 0; s0 < most; s0 += G) {
+                const int s = s0 + sub;
+                double x = 0.0, f = 0.0;
+                if (s < slots) {
+                    double edge, m;
+                    if (s < base) {
+                        edge = s & 1 ? g.hi : g.lo;
+                        m = s < 2 ? mlo : s < 4 ? mhi : clampd(0.5 * (g.lo + g.hi), mlo, mhi);
+                    } else {
+                        unsigned rest = inners;
+                        for (int r = (s - base) >> 1; r > 0; --r) rest &= rest - 1;
+                        const int kk = a + k0 + __ffs(rest) - 1;
+                        m = 0.5 * (E[kk] + E[kk + 1]);
+                        edge = E[kk + ((s - base) & 1)];
+                    }
+                    x = (edge - m) * inv_s;
+                    f = erfc(fabs(x));
+                }
+                if (base > 0 && s0 == 0) {
+                    tx = x;
+                    tf = f;
+                }
+                const int src = my_slot & (G - 1);
+                const double xa = __shfl_sync(kAll, x, src, G), fa = __shfl_sync(kAll, f, src, G);
+                const double xb = __shfl_sync(kAll, x, src + 1, G), fb = __shfl_sync(kAll, f, src + 1, G);
+                if (my_slot >= s0 && my_slot < s0 + G) {
+                    qa = xa;
+                    qfa = fa;
+                    qb = xb;
+                    qfb = fb;
+                }
+            }
+            if (mine) {
                 const double glo = mass64(x0, f0, y0, h0), ghi = mass64(x1, f1, y1, h1);
-                const double mid = 0.5 * (c0 + e0);
                 // largest factor: at the midpoint clamped to the image
-                const double U = mid < mlo ? glo : mid > mhi ? ghi : g64(c0, e0, mid, inv_s);
+                const double U = mid < mlo ? glo : mid > mhi ? ghi : mass64(qa, qfa, qb, qfb);
                 if (act) ul[k] = make_double2(U, fmin(glo, ghi));
                 if (U >= cut) {
                     first = min(first, k);
@@ -169,25 +230,21 @@ items_fp64(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
                 ow += v;
             }
         }
-        // the masses beyond the window and in the domain, one per lane
-        double part = 0.0;
-        if (sub < 5) {
-            const double mid = 0.5 * (g.lo + g.hi);
-            double ge = g.lo, gf = g.hi, gm = sub == 2 ? clampd(mid, mlo, mhi) : sub == 3 ? mlo : mhi;
-            bool on = true;
-            if (sub == 0) {
-                on = a > 0;
-                ge = E[0];
-                gf = E[on ? a : 0];
-                gm = mlo;
-            } else if (sub == 1) {
-                on = b < g.N - 1;
-                ge = E[on ? b + 1 : g.N];
-                gf = E[g.N];
-                gm = mhi;
-            }
-            if (on) part = g64(ge, gf, gm, inv_s);
+        // the masses beyond the window at m_lo and m_hi and in the domain at
+        // its clamped midpoint, m_lo and m_hi, one per lane
+        const int sa = sub == 2 ? 4 : sub == 4 ? 2 : 0, sb = sub == 2 ? 5 : sub == 3 ? 1 : 3;
+        double pa = __shfl_sync(kAll, tx, sa, G), fa = __shfl_sync(kAll, tf, sa, G);
+        double pb = __shfl_sync(kAll, tx, sb, G), fb = __shfl_sync(kAll, tf, sb, G);
+        const double qx = __shfl_sync(kAll, wx, wlane, G), qf = __shfl_sync(kAll, wf, wlane, G);
+        if (sub == 0) {
+            pb = ax;
+            fb = af;
+        } else if (sub == 1) {
+            pa = qx;
+            fa = qf;
         }
+        double part = 0.0;
+        if (sub == 0 ? a > 0 : sub == 1 ? b < g.N - 1 : sub < 5) part = mass64(pa, fa, pb, fb);
         sw = group_sum(kAll, sw, G);
         ow = group_sum(kAll, ow, G);
         for (int o = G >> 1; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(kAll, M, o, G));
@@ -208,7 +265,7 @@ items_fp64(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
             h.first = empty ? 0 : first;
             *reinterpret_cast<Item64 *>(it) = h;
         }
-        if (d != D.n - 1 || !is_sorted_dim(cut, g.w64)) continue;   // uniform in the warp
+        if (d != D.n - 1 || !is_sorted_dim(D.cutoff32, g.w64)) continue;   // uniform in the warp
         const int cs = g.w64 + 1;
         double *su = item_sorted(it, g.w64), *sl = su + cs, *pu = sl + cs, *pl = pu + cs, *sf = pl + cs;
         for (int k = sub; act && k < tw; k += G) {
@@ -313,6 +370,7 @@ struct Warp64 {
     WalkDim *h;
     double2 *ul;
     double *su, *pu, *pl, *sf;   // the last dimension's sorted arrays (count pass)
+    float *su32;                 // leading bits of su
     unsigned char *lists;
 };
 
@@ -379,13 +437,68 @@ __device__ __forceinline__ Node64 node_at(const Nodes64 &L, bool root, int i)
     return Node64{L.P[i], L.Pl[i], L.col[i]};
 }
 
-// cut <= 0 keeps every product that is not negative (a factor of rounded
-// erfc differences can be a negative last bit); else the bits of non-negative
-// doubles order like the doubles, and integer compares leave the FP64 pipe to
-// the products.
-__device__ __forceinline__ bool passes(double x, double cut, long long cutb)
+// The keep test x >= cut on the bits, which leaves the FP64 pipe to the products
+// (a compare holds it as long as a multiply): the bits of non-negative doubles
+// order like the doubles, and negative ones (a factor of rounded erfc
+// differences can be a negative last bit) stay below; cutoff 0 keeps -0 too.
+struct Cut64 {
+    long long bits, also;   // keep iff bits(x) >= bits or bits(x) == also
+    float sure, never;      // FP32 products from here on / below here decide (see search64)
+};
+
+// cut32: the smallest float that is not below cut.
+__device__ __forceinline__ Cut64 cut_of(double cut, float cut32)
 {
-    return cut > 0.0 ? __double_as_longlong(x) >= cutb : x >= cut;
+    Cut64 c;
+    c.bits = __double_as_longlong(cut);
+    c.also = cut32 > 0.0f ? c.bits : LLONG_MIN;
+    // products below the normal range decide nothing
+    const bool fine = cut32 > 1e-30f;
+    c.sure = fine ? cut32 * 1.00001f : INFINITY;
+    c.never = fine ? cut32 * 0.99999f : 0.0f;
+    return c;
+}
+
+__device__ __forceinline__ bool passes(double x, const Cut64 &c)
+{
+    const long long b = __double_as_longlong(x);
+    return b >= c.bits || b == c.also;
+}
+
+// A double's leading 24 bits as a float (rounded to zero; for values in the
+// normal range of FP32 or 0, else some small or large float), without the FP64
+// pipe's conversion.
+__device__ __forceinline__ float lead32(double x)
+{
+    const long long b = __double_as_longlong(x);
+    const int e = (int)(b >> 52);                       // sign and exponent
+    const unsigned m = (unsigned)((unsigned long long)b >> 29);
+    return e <= 896 ? 0.0f : __uint_as_float(m - (896u << 23));
+}
+
+// The bits of a non-negative float as a double (subnormals as 0).
+__device__ __forceinline__ long long wide_bits(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    return b < (1u << 23) ? 0ll : ((long long)b << 29) + (896ll << 52);
+}
+
+// How many entries of su (descending) RN(P su) >= cut keeps: FP32 products of
+// leading bits (within 2^-20 of the exact ones) decide all but those within
+// 1e-5 of the cutoff, which take the FP64 product.
+__device__ __forceinline__ int search64(double P, const double *su, const float *su32, int n,
+                                        const Cut64 &cut)
+{
+    const float p = lead32(P);
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const float f = p * su32[mid];
+        bool keep = f >= cut.sure;
+        if (!keep && f >= cut.never) keep = __double_as_longlong(P * su[mid]) >= cut.bits;
+        if (keep) lo = mid + 1; else hi = mid;
+    }
+    return lo;
 }
 
 // Children of candidates [c0, c1) of the level k - 1 list in dimension k, kept
@@ -404,14 +517,14 @@ __device__ __forceinline__ int expand64(const Warp64 &S, int k, int c0, int c1, 
         const int t = e - pi * h.tw;
         const Node64 par = node_at(Lp, k == 0, pi);
         const double2 ul = S.ul[h.off + t];
-        const double Pc = par.P * ul.x;
+        const double Pc = k > 0 ? par.P * ul.x : ul.x;
         const bool keep = act && __double_as_longlong(Pc) >= h.cp;
         if (COUNT && act && !keep) acc.drop += Pc * h.SR;
         const unsigned bal = __ballot_sync(0xffffffffu, keep);
         if (keep) {
             const int o = nout + __popc(bal & lanemask_lt());
             Lc.P[o] = Pc;
-            Lc.Pl[o] = par.Pl * ul.y;
+            Lc.Pl[o] = k > 0 ? par.Pl * ul.y : ul.y;
             Lc.col[o] = par.c + h.cb + t * h.stride;
         }
         nout += __popc(bal);
@@ -422,19 +535,14 @@ __device__ __forceinline__ int expand64(const Warp64 &S, int k, int c0, int c1, 
 
 // The targets of the last dimension under npar parents, counted and summed.
 __device__ __forceinline__ void leaf_count64(const Warp64 &S, int n, const Nodes64 &Lp, bool root,
-                                             int npar, int lane, Sums64 &acc, double cut,
-                                             long long cutb, bool sorted)
+                                             int npar, int lane, Sums64 &acc, const Cut64 &cut,
+                                             bool sorted)
 {
     const WalkDim h = S.h[n - 1];
     if (sorted) {
         for (int pi = lane; pi < npar; pi += 32) {
             const Node64 par = node_at(Lp, root, pi);
-            int lo = 0, hi = h.tw;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (__double_as_longlong(par.P * S.su[mid]) >= cutb) lo = mid + 1;
-                else hi = mid;
-            }
+            const int lo = search64(par.P, S.su, S.su32, h.tw, cut);
             acc.cnt += lo;
             acc.sup += par.P * S.pu[lo];
             acc.slo += par.Pl * S.pl[lo];
@@ -448,7 +556,7 @@ __device__ __forceinline__ void leaf_count64(const Warp64 &S, int n, const Nodes
         const Node64 par = node_at(Lp, root, pi);
         const double2 ul = S.ul[h.off + e - pi * h.tw];
         const double Pc = par.P * ul.x;
-        if (passes(Pc, cut, cutb)) {
+        if (passes(Pc, cut)) {
             acc.cnt += 1;
             acc.sup += Pc;
             acc.slo += par.Pl * ul.y;
@@ -461,7 +569,7 @@ __device__ __forceinline__ void leaf_count64(const Warp64 &S, int n, const Nodes
 // The same targets, written: one lane per candidate, kept ones compacted.
 __device__ __forceinline__ void leaf_emit64(const Warp64 &S, int n, const Nodes64 &Lp, bool root,
                                             int npar, int lane, const Out64 &out, int64_t &written,
-                                            double cut, long long cutb)
+                                            const Cut64 &cut)
 {
     const WalkDim h = S.h[n - 1];
     const int total = npar * h.tw;
@@ -472,7 +580,7 @@ __device__ __forceinline__ void leaf_emit64(const Warp64 &S, int n, const Nodes6
         const Node64 par = node_at(Lp, root, pi);
         const double2 ul = S.ul[h.off + t];
         const double Pc = par.P * ul.x;
-        const bool keep = e0 + lane < total && passes(Pc, cut, cutb);
+        const bool keep = e0 + lane < total && passes(Pc, cut);
         const unsigned bal = __ballot_sync(0xffffffffu, keep);
         const int64_t p = written + __popc(bal & lanemask_lt());
         if (keep && p < out.len) {
@@ -486,11 +594,11 @@ __device__ __forceinline__ void leaf_emit64(const Warp64 &S, int n, const Nodes6
 
 template <bool EMIT>
 __device__ bool walk_row64(const Warp64 &S, int n, int lane, Sums64 &acc, const Out64 &out,
-                           int64_t &written, double cut, long long cutb, bool sorted)
+                           int64_t &written, const Cut64 &cut, bool sorted)
 {
     auto leaves = [&](const Nodes64 &Lp, bool root, int npar) {
-        if (EMIT) leaf_emit64(S, n, Lp, root, npar, lane, out, written, cut, cutb);
-        else leaf_count64(S, n, Lp, root, npar, lane, acc, cut, cutb, sorted);
+        if (EMIT) leaf_emit64(S, n, Lp, root, npar, lane, out, written, cut);
+        else leaf_count64(S, n, Lp, root, npar, lane, acc, cut, sorted);
     };
     if (n == 1) {
         leaves(Nodes64{}, true, 1);
@@ -553,7 +661,7 @@ struct Walk64Args {
 // tables, the last dimension's sorted arrays, the node lists.
 __host__ __device__ inline int64_t warp_bytes64(int n, int64_t tsum, int wl, bool sorted)
 {
-    return 40 * n + (n & 1 ? 8 : 0) + 16 * tsum + (sorted ? 32 * (int64_t)((wl + 2) & ~1) : 0) +
+    return 40 * n + (n & 1 ? 8 : 0) + 16 * tsum + (sorted ? 40 * (int64_t)((wl + 2) & ~1) : 0) +
            list_bytes64(n);
 }
 
@@ -586,10 +694,11 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
         if (!D.walk64) continue;
         const int n = D.n;
         const double cut = D.cutoff;
-        const long long cutb = __double_as_longlong(cut);
+        const float cut32 = D.cutoff32;
+        const Cut64 keep = cut_of(cut, cut32);
         const int64_t r = row - B->row_begin[q];
         const int wl = D.dim[n - 1].w64;
-        const bool sorted = !EMIT && is_sorted_dim(cut, wl);
+        const bool sorted = !EMIT && is_sorted_dim(cut32, wl);
         Warp64 S;
         S.h = reinterpret_cast<WalkDim *>(mine);
         S.ul = reinterpret_cast<double2 *>(mine + 40 * n + (n & 1 ? 8 : 0));
@@ -611,8 +720,8 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
         const bool empty = __any_sync(0xffffffffu, lane < n && h.tw == 0);
         int off = 0, tsum = 0;
         float R = 1.0f;
-        double SR = 1.0;
-        for (int k = 0; k < n; ++k) {
+        double SR = 1.0;   // its products only where two factors meet
+        for (int k = n - 1; k >= 0; --k) {
             const int twk = __shfl_sync(0xffffffffu, h.tw, k);
             const float Mk = __shfl_sync(0xffffffffu, h.M32, k);
             if (k < lane) off += twk;
@@ -620,7 +729,8 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
             tsum += twk;
             if (!EMIT) {
                 const double SWk = __shfl_sync(0xffffffffu, h.SW, k);
-                if (k > lane) SR *= SWk;
+                if (k == n - 1) SR = lane < k ? SWk : 1.0;
+                else if (k > 0) SR = lane < k ? SR * SWk : SR;
             }
         }
         if (lane < n) {
@@ -628,8 +738,11 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
             // a node is kept iff its product is at least cutoff / R, taken
             // low enough that no rounding of the rest of the chain can lift a
             // dropped one to the cutoff; cutoff 0 keeps every node
-            const float thr = __fmul_rd(__fdiv_rd(__double2float_rd(cut), R), 0.999999f);
-            w.cp = cut > 0.0 ? __double_as_longlong((double)thr) : LLONG_MIN;
+            // (cut32 is within 2^-23 of the cutoff where it is not tiny: tiny
+            // ones prune nothing; wide_bits, not a conversion: that would take
+            // the FP64 pipe)
+            const float thr = __fmul_rd(__fdiv_rd(cut32, R), 0.999999f);
+            w.cp = cut32 > 1e-30f ? wide_bits(thr) : cut32 > 0.0f ? 0ll : LLONG_MIN;
             w.SR = SR;
             w.tw = h.tw;
             w.off = off;
@@ -644,7 +757,8 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
         S.pu = S.su + cs;
         S.pl = S.pu + cs;
         S.sf = S.pl + cs;
-        S.lists = reinterpret_cast<unsigned char *>(S.su + (sorted ? 4 * cs : 0));
+        S.su32 = reinterpret_cast<float *>(S.sf + cs);
+        S.lists = reinterpret_cast<unsigned char *>(S.su + (sorted ? 5 * cs : 0));
         if (!empty) {
             for (int k = 0; k < n; ++k) {
                 const unsigned long long p = __shfl_sync(0xffffffffu, (unsigned long long)it, k);
@@ -660,7 +774,9 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
                 const int tl = __shfl_sync(0xffffffffu, h.tw, n - 1);
                 const double *src = item_sorted(pl, wl);
                 for (int e = lane; e <= tl; e += 32) {
-                    S.su[e] = e < tl ? src[e] : 0.0;
+                    const double x = e < tl ? src[e] : 0.0;
+                    S.su[e] = x;
+                    S.su32[e] = lead32(x);
                     S.pu[e] = src[e + 2 * (wl + 1)];
                     S.pl[e] = src[e + 3 * (wl + 1)];
                     S.sf[e] = src[e + 4 * (wl + 1)];
@@ -677,7 +793,7 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
                 Sums64 none;
                 int64_t written = 0;
                 bool ok = true;
-                if (!empty) ok = walk_row64<true>(S, n, lane, none, out, written, cut, cutb, false);
+                if (!empty) ok = walk_row64<true>(S, n, lane, none, out, written, keep, false);
                 if (lane == 0 && (!ok || written != len))
                     atomicOr(A.status, ok ? IMPACT_STATUS_EMIT_MISMATCH : IMPACT_STATUS_INTERNAL);
             }
@@ -686,7 +802,7 @@ __global__ void __launch_bounds__(kWarps * 32) walk_fp64(const Walk64Args A)
             const Out64 none{nullptr, nullptr, nullptr, 0};
             int64_t w0 = 0;
             bool ok = true;
-            if (!empty) ok = walk_row64<false>(S, n, lane, acc, none, w0, cut, cutb, sorted);
+            if (!empty) ok = walk_row64<false>(S, n, lane, acc, none, w0, keep, sorted);
             const int cnt = __reduce_add_sync(0xffffffffu, acc.cnt);
             double sum[3] = {acc.drop, acc.sup, acc.slo};
             warp_sums(sum, lane);
@@ -718,7 +834,7 @@ int64_t size_items64(ImpactDesc &D, int64_t nnz_bound)
     int64_t bytes = 0, tsum = 0;
     for (int d = 0; d < n; ++d) {
         ImpactDim &g = D.dim[d];
-        const bool sorted = d == n - 1 && is_sorted_dim(D.cutoff, g.w64);
+        const bool sorted = d == n - 1 && is_sorted_dim(D.cutoff32, g.w64);
         g.group = g.w64 + 1 <= 8 ? 8 : g.w64 + 1 <= 16 ? 16 : 32;
         tsum += g.w64;
         const int64_t st = kItemHead + 16 * (int64_t)g.w64 + (sorted ? 40 * (int64_t)(g.w64 + 1) : 0);
@@ -740,7 +856,7 @@ int64_t walk64_bytes(const ImpactDesc &D)
     int64_t tsum = 0;
     for (int d = 0; d < D.n; ++d) tsum += D.dim[d].w64;
     const int wl = D.dim[D.n - 1].w64;
-    return (warp_bytes64(D.n, tsum, wl, is_sorted_dim(D.cutoff, wl)) + 15) / 16 * 16;
+    return (warp_bytes64(D.n, tsum, wl, is_sorted_dim(D.cutoff32, wl)) + 15) / 16 * 16;
 }
 
 cudaError_t launch_items64(const BatchIndex *d_index, int64_t units, uint32_t *status,

@@ -55,6 +55,10 @@ PROBLEMS = {
                               B=[[0.1, 0], [0, 0.1], [0, 0], [-0.0, 0]]),
     "dense-6d": lambda: linear([3, 2, 3, 2, 3, 2], np.eye(6) * 0.8 + 0.02, [0.5] * 6, 0.0, U1),
     "images": lambda: images_of(linear([9, 12], np.eye(2), [0.7, 0.5], 1e-8, U2), 3),
+    # cutoffs around FP32's smallest normal number (pruning and searches use FP32)
+    "cutoff-1e-39": lambda: linear([12, 9, 5], np.eye(3) * 0.9, [0.3, 0.4, 0.2], 1e-39, U1),
+    "cutoff-1e-31": lambda: linear([12, 9, 5], np.eye(3) * 0.9, [0.3, 0.4, 0.2], 1e-31, U1),
+    "cutoff-2e-30": lambda: linear([12, 9, 5], np.eye(3) * 0.9, [0.3, 0.4, 0.2], 2e-30, U1),
     "one-cell": lambda: linear([1, 1, 5], np.eye(3) * 0.5, [0.3, 1.0, 0.6], 1e-8, U1),
 }
 
