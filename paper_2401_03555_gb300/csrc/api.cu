@@ -456,8 +456,10 @@ impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int
     impact::RowOutputs o{out->row_ptr, out->col, out->lo, out->up, nullptr, nullptr, nullptr,
                          nullptr, W.status(), capacity, B.rows};
     if (B.prec == PREC_FP32_SOUND) {
-        if (!records_ready)   // rebuild the records; the row outputs stay as counted
+        if (!records_ready) {   // rebuild the records; the row outputs stay as counted
             CK(setup_pass(B, W, st));
+            CK(impact::launch_leaf_fp32(W.index(), B.leaf_begin.back(), B.leaf_smem, st));
+        }
         CK(walk_pass(B, W, WALK_EMIT, B.tune.emit_warps, o, W.counter() + 1, chunk_rows, st));
     } else {
         if (B.any64) {

@@ -86,6 +86,7 @@ struct ImpactDesc {
     // dimensions together (leaf_shared), numbered like the items
     int share32;
     int leaf_shared;
+    int lists;                // the leaf tables carry the emit pass's list blocks
     int64_t leaf_items;
     int64_t leaf_mul[IMPACT_MAX_DIM];
     int leaf_classes;

@@ -53,6 +53,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <limits.h>
+
 #include <algorithm>
 
 #include "../../include/impact.h"
@@ -633,6 +635,34 @@ __host__ __device__ inline int list_bytes(int n) { return align16((n > 2 ? n - 2
 // Entries of an emit leaf table, even: the tables are 8-byte aligned.
 __host__ __device__ constexpr int emit_cap(int leaf_cap) { return (leaf_cap + 1) & ~1; }
 
+// Emit by lists (builds with shared leaf tables, rows of kListMin to kListMax
+// entries): the leaf block of a row -- sorted upper factors, then U, L and column
+// of the entries in C order, kListMax words each, and for every kept count k
+// the k largest entries in C order, one byte each -- then the parents of a
+// chunk and the chunk's start bits. Below 20 entries a parent's search costs
+// more than the candidates that its list saves (building 6^7, 9 entries: 4.9 ms
+// by lists, 4.3 by candidates), above 48 the lists outgrow the block. The window
+// bound of a build (its rows' tables hold about a third of it) tells which side
+// most rows are on: outside kListCapMin..kListCapMax entries the smaller blocks
+// are worth more.
+constexpr int kListMin = 20, kListMax = 48, kListCapMin = 64, kListCapMax = 160;
+__host__ __device__ constexpr int list_block(int nb)   // bytes, multiple of 16
+{
+    return align16(16 * kListMax + nb * (nb + 1) / 2);
+}
+constexpr int kInfoBytes = 16 * kCap;
+constexpr int kStartWords = kCap * kListMax / 32;
+
+// Shared memory of the emit's leaf: the staged table and its trimmed copy, or a
+// list block with the parents and start bits behind it.
+__host__ __device__ inline int emit_leaf_bytes(int leaf_cap, bool lists)
+{
+    const int staged = align16(24 * emit_cap(leaf_cap));
+    if (!lists) return staged;
+    const int block = list_block(kListMax);
+    return (staged > block ? staged : block) + kInfoBytes + 4 * kStartWords;
+}
+
 __device__ __forceinline__ WarpMem carve(unsigned char *work, unsigned char *rec, int n, int leaf_cap)
 {
     WarpMem m;
@@ -894,11 +924,18 @@ __device__ void leaf_build(const WarpMem &S, int n, Leaf &f, int lane, float cut
 
 // leaf_fp32: the sorted leaf table of every distinct image of the last two
 // dimensions together, one warp each, from their items: {nb, ..} in 16 bytes,
-// then (su, sf, pu, pl) per entry k = 0..nb, su[nb] unused. Tables of more than
-// leaf_cap entries stay empty (their rows test the entries directly).
+// then (su, sf, pu, pl) per entry k = 0..nb, su[nb] unused, and the list block of
+// the emit pass. Tables of more than leaf_cap entries stay empty (their rows
+// test the entries directly).
 struct LeafHead {
     int nb, pad[3];
 };
+
+// Where the list block of a leaf table stands.
+__host__ __device__ constexpr int leaf_lists_at(int leaf_cap)
+{
+    return (int)sizeof(LeafHead) + 16 * (leaf_cap + 1);
+}
 
 __global__ void __launch_bounds__(128)
 leaf_fp32(const BatchIndex *__restrict__ B, int warp_smem)
@@ -945,11 +982,11 @@ leaf_fp32(const BatchIndex *__restrict__ B, int warp_smem)
                 RecDim rd;
                 rd.tw = o.tw;
                 rd.tb = e * wm;
-                rd.cb = 0;
+                rd.cb = (o.a + o.f0) * g.stride;
                 rd.magic = o.tw > 1
                                ? (uint32_t)((0x100000000ull + (unsigned)o.tw - 1) / (unsigned)o.tw) : 0u;
                 rd.cp = rd.SR = 0.0f;
-                rd.stride = 0;
+                rd.stride = g.stride;
                 rd.lay = 0;
                 S.h[d] = rd;
             }
@@ -964,6 +1001,42 @@ leaf_fp32(const BatchIndex *__restrict__ B, int warp_smem)
             float4 *to = reinterpret_cast<float4 *>(out + sizeof(LeafHead));
             for (int k = lane; k <= f.nb; k += 32)
                 to[k] = make_float4(k < f.nb ? f.su[k] : 0.0f, f.sf[k], f.pu[k], f.pl[k]);
+        }
+        if (D.lists && f.sorted && f.nb >= kListMin && f.nb <= kListMax) {   // the emit's list block
+            const int nb = f.nb;
+            float *const block = reinterpret_cast<float *>(mine + warp_smem - list_block(kListMax));
+            unsigned char *const lists = reinterpret_cast<unsigned char *>(block + 4 * kListMax);
+            // sorted positions of entries lane and lane + 32 (ties by index)
+            const bool h0 = lane < nb, h1 = lane + 32 < nb;
+            const float u0 = h0 ? f.bu[lane] : 0.0f, u1 = h1 ? f.bu[lane + 32] : 0.0f;
+            int r0 = 0, r1 = 0;
+            for (int i = 0; i < nb; ++i) {
+                const float v = f.bu[i];
+                r0 += v > u0 || (v == u0 && i < lane);
+                r1 += v > u1 || (v == u1 && i < lane + 32);
+            }
+            if (!h0) r0 = INT_MAX;
+            if (!h1) r1 = INT_MAX;
+            for (int j = lane; j < kListMax; j += 32) {
+                const bool in = j < nb;
+                block[j] = in ? f.su[j] : 0.0f;
+                block[j + kListMax] = in ? f.bu[j] : 0.0f;
+                block[j + 2 * kListMax] = in ? f.bl[j] : 0.0f;
+                block[j + 3 * kListMax] = in ? __int_as_float(f.bc[j]) : 0.0f;
+            }
+            for (int k = 1; k <= nb; ++k) {
+                unsigned char *const l = lists + k * (k - 1) / 2;
+                const unsigned b0 = __ballot_sync(0xffffffffu, r0 < k);
+                if (r0 < k) l[__popc(b0 & lanemask_lt())] = (unsigned char)lane;
+                if (nb > 32) {
+                    const unsigned b1 = __ballot_sync(0xffffffffu, r1 < k);
+                    if (r1 < k) l[__popc(b0) + __popc(b1 & lanemask_lt())] = (unsigned char)(lane + 32);
+                }
+            }
+            __syncwarp();
+            float4 *const to = reinterpret_cast<float4 *>(out + leaf_lists_at(D.leaf_cap));
+            for (int i = lane; i < (list_block(nb) >> 4); i += 32)
+                to[i] = reinterpret_cast<const float4 *>(block)[i];
         }
         __syncwarp();
     }
@@ -1274,6 +1347,79 @@ __device__ __forceinline__ void leaf_emit(const WarpMem &S, const EmitLeaf &f, c
     }
 }
 
+// The same from the row's list block: a parent keeps the k largest entries of
+// the table (RU(P x) is monotone in x), k from a search in the sorted table, and
+// list k holds them in C order, so every lane of every step writes a pair: the
+// chunk's pairs are numbered through, a bit marks each parent's first pair, and
+// a pair's parent is the number of bits up to it. Steps of 32 pairs and not of
+// 32 candidates (the 11^5 room: 62 and not 97 a row, about 27 instructions each
+// and not 33), for about 80 instructions per 32 parents: its emit pass 7.45 ->
+// 6.69 ms, the list blocks 0.2 ms of leaf_fp32.
+__device__ __forceinline__ void emit_lists(unsigned char *block, unsigned char *after, int nb,
+                                           const NodeList &Lp, int npar, int lane,
+                                           const EmitOut &out, int &written, float cut)
+{
+    const float *const su = reinterpret_cast<const float *>(block);
+    const unsigned char *const lists = block + 16 * kListMax;
+    float4 *const info = reinterpret_cast<float4 *>(after);
+    unsigned *const bits = reinterpret_cast<unsigned *>(after + kInfoBytes);
+    int start[kCap / 32], total = 0, nord = 0;
+    __syncwarp();   // the chunk before is written
+#pragma unroll
+    for (int h = 0; h < kCap / 32; ++h) {
+        const int pi = lane + 32 * h;
+        const float P = pi < npar ? Lp.P[pi] : 0.0f;
+        int lo = 0, hi = nb;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (__fmul_ru(P, su[mid]) >= cut) lo = mid + 1; else hi = mid;
+        }
+        int s = lo;   // pairs up to this parent
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += y;
+        }
+        const unsigned some = __ballot_sync(0xffffffffu, lo > 0);
+        start[h] = lo > 0 ? total + s - lo : -1;
+        if (lo > 0)
+            info[nord + __popc(some & lanemask_lt())] =
+                make_float4(P, Lp.Pl[pi], __int_as_float(Lp.col[pi]),
+                            __int_as_float(lo * (lo - 1) / 2 - start[h]));
+        total += __shfl_sync(0xffffffffu, s, 31);
+        nord += __popc(some);
+    }
+    for (int w = lane; w < (total + 31) >> 5; w += 32) bits[w] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < kCap / 32; ++h)
+        if (start[h] >= 0) atomicOr(&bits[start[h] >> 5], 1u << (start[h] & 31));
+    __syncwarp();
+    const int room = min(total, out.len - written);
+    int before = -1;   // parents whose first pair stands before this step, less one
+    int32_t *const col = out.col + written;
+    float *const lo = out.lo + written, *const up = out.up + written;
+    const unsigned le = lanemask_lt() | (1u << lane);
+    // two steps at once: a step is a chain of four shared-memory loads
+    for (int o0 = 0; o0 < total; o0 += 64) {
+        const unsigned wa = bits[o0 >> 5], wb = o0 + 32 < total ? bits[(o0 >> 5) + 1] : 0u;
+        const int oa = o0 + lane, ob = oa + 32;
+        const float4 pa = info[before + __popc(wa & le)];
+        before += __popc(wa);
+        const float4 pb = info[before + __popc(wb & le)];
+        before += __popc(wb);
+        const float *const ea = su + lists[__float_as_int(pa.w) + min(oa, total - 1)];
+        const float *const eb = su + lists[__float_as_int(pb.w) + min(ob, total - 1)];
+        const float ua = __fmul_ru(pa.x, ea[kListMax]), la = __fmul_rd(pa.y, ea[2 * kListMax]);
+        const int ca = __float_as_int(pa.z) + __float_as_int(ea[3 * kListMax]);
+        const float ub = __fmul_ru(pb.x, eb[kListMax]), lb = __fmul_rd(pb.y, eb[2 * kListMax]);
+        const int cb = __float_as_int(pb.z) + __float_as_int(eb[3 * kListMax]);
+        st_pair(oa < room, col + oa, lo + oa, up + oa, ca, la, ua);
+        st_pair(ob < room, col + ob, lo + ob, up + ob, cb, lb, ub);
+    }
+    written += total;
+}
+
 // The same for a table too wide to stage, and for the root (rows of at most two
 // dimensions): entries evaluated where they are read.
 __device__ __forceinline__ void leaf_emit_wide(const WarpMem &S, int n, const Leaf &f,
@@ -1336,15 +1482,16 @@ __device__ __forceinline__ void count_row(const WarpMem &S, int n, const Leaf &f
 // scheduler hide its shared-memory latency; unrolled, the 11^5 room's emit
 // pass took 7.8 ms against 7.45). Every step fills a list, runs the leaves of one
 // or leaves one whose candidates are used up, so the loop ends.
-__device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f, int lane,
-                                         const EmitOut &out, int &written, float cut)
+__device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f, bool lists,
+                                         int after, int lane, const EmitOut &out, int &written,
+                                         float cut)
 {
     if (n <= 2) {
         leaf_emit_wide(S, n, f, NodeList{}, true, 1, lane, out, written, cut);
         return;
     }
     const EmitLeaf g = emit_leaf(S, f);
-    if (g.staged)
+    if (g.staged && !lists)
         for (int j = lane; j < f.nb; j += 32) {
             const LeafEntry e = leaf_eval(S, n, f, j);
             g.u[j] = e.u;
@@ -1359,7 +1506,9 @@ __device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f,
         if (k == last + 1) {
             const NodeList L = node_list(S.work, last);
             const int npar = __shfl_sync(0xffffffffu, my_sz, last);
-            if (g.staged) leaf_emit(S, g, L, npar, lane, out, written, cut);
+            unsigned char *const block = reinterpret_cast<unsigned char *>(S.leaf);
+            if (lists) emit_lists(block, block + after, f.nb, L, npar, lane, out, written, cut);
+            else if (g.staged) leaf_emit(S, g, L, npar, lane, out, written, cut);
             else leaf_emit_wide(S, n, f, L, false, npar, lane, out, written, cut);
             k = last;
             continue;
@@ -1666,7 +1815,24 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
                 const EmitOut out{A.col + base, A.lo + base, A.up + base, (int)len};
                 int written = 0;
                 __syncwarp();   // FUSED: the count's leaf table makes room
-                if (!empty) emit_row(S, n, f, lane, out, written, cut);
+                if (!empty) {
+                    // the row's list block, where the build shares leaf tables
+                    const bool lists = MODE == MODE_EMIT && D.lists && f.nb >= kListMin &&
+                                       f.nb <= kListMax;
+                    const int after = emit_leaf_bytes(D.leaf_cap, true) - kInfoBytes - 4 * kStartWords;
+                    if (lists) {
+                        const unsigned char *src = B->leaf[q] +
+                                                   rec_row(rec, n)->leaf * D.leaf_stride +
+                                                   leaf_lists_at(D.leaf_cap);
+                        unsigned char *dst = reinterpret_cast<unsigned char *>(S.leaf);
+                        for (int i = lane; i < (list_block(f.nb) >> 4); i += 32)
+                            cp_async16(dst + 16 * i, src + 16 * i);
+                        cp_async_commit();
+                        cp_async_wait_all();
+                        __syncwarp();
+                    }
+                    emit_row(S, n, f, lists, after, lane, out, written, cut);
+                }
                 if (lane == 0 && written != len) atomicOr(A.status, IMPACT_STATUS_EMIT_MISMATCH);
             }
         }
@@ -1710,7 +1876,7 @@ int walk_work_bytes(const ImpactDesc &D, int mode)
 {
     // rows with a shared leaf table stage none of their own to count, and
     // rows of at most two dimensions none at all
-    const int emit = D.n > 2 ? 24 * emit_cap(D.leaf_cap) : 0;
+    const int emit = D.n > 2 ? emit_leaf_bytes(D.leaf_cap, mode == MODE_EMIT && D.lists) : 0;
     const int count = D.n > 2 || !(D.cutoff32 > 0.0f) ? 32 * (D.leaf_cap + 1) : 0;
     if (mode == MODE_EMIT) return list_bytes(D.n) + align16(emit);
     if (mode == MODE_COUNT) return list_bytes(D.n) + align16(D.leaf_shared ? 0 : count);
@@ -1745,16 +1911,19 @@ void size_items32(ImpactDesc &D, int64_t &item_bytes, int64_t &leaf_bytes)
     }
     D.share32 = D.kind != KIND_IMAGES && items * 3 <= D.rows * n;
     item_bytes = D.share32 ? bytes : 0;
-    D.leaf_stride = (int)sizeof(LeafHead) + 16 * (D.leaf_cap + 1);
+    const bool lists = D.leaf_cap >= kListCapMin && D.leaf_cap <= kListCapMax;
+    D.leaf_stride = leaf_lists_at(D.leaf_cap) + (lists ? list_block(kListMax) : 0);
     D.leaf_shared = D.share32 && n >= 3 && D.cutoff32 > 0.0f && D.leaf_items * 4 <= D.rows &&
                     D.leaf_items * D.leaf_stride <= D.rows * (int64_t)D.rec_stride;
+    D.lists = D.leaf_shared && lists;
     leaf_bytes = D.leaf_shared ? D.leaf_items * D.leaf_stride : 0;
 }
 
 int leaf32_bytes(const ImpactDesc &D)
 {
     const int w = ((D.dim[D.n - 2].wcap + 1) & ~1) + ((D.dim[D.n - 1].wcap + 1) & ~1);
-    return 2 * (int)sizeof(RecDim) + 8 * w + align16(32 * (D.leaf_cap + 1));
+    return 2 * (int)sizeof(RecDim) + 8 * w + align16(32 * (D.leaf_cap + 1)) +
+           (D.lists ? list_block(kListMax) : 0);
 }
 
 cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, bool shared, bool own,

@@ -55,6 +55,12 @@ PROBLEMS = {
                               B=[[0.1, 0], [0, 0.1], [0, 0], [-0.0, 0]]),
     "dense-6d": lambda: linear([3, 2, 3, 2, 3, 2], np.eye(6) * 0.8 + 0.02, [0.5] * 6, 0.0, U1),
     "images": lambda: images_of(linear([9, 12], np.eye(2), [0.7, 0.5], 1e-8, U2), 3),
+    # shared leaf tables around the sizes the emit pass takes by lists (20 and 48
+    # entries, window bounds 64 and 160), with rows of all sizes at the border
+    "lists-4x5": lambda: linear([6, 8, 8], np.eye(3) * 0.9, [0.4, 0.3, 0.4], 1e-8, U1),
+    "lists-6x7": lambda: linear([5, 9, 12], np.eye(3) * 0.9, [0.5, 0.45, 0.5], 1e-8, U2),
+    "lists-7x7": lambda: linear([6, 12, 12], np.eye(3) * 0.9, [0.9, 0.52, 0.5], 1e-8, U1),
+    "lists-5d": lambda: linear([4, 3, 5, 9, 9], np.eye(5) * 0.9, [0.8, 0.4, 0.6, 0.45, 0.4], 1e-8, U1),
     # cutoffs around FP32's smallest normal number (pruning and searches use FP32)
     "cutoff-1e-39": lambda: linear([12, 9, 5], np.eye(3) * 0.9, [0.3, 0.4, 0.2], 1e-39, U1),
     "cutoff-1e-31": lambda: linear([12, 9, 5], np.eye(3) * 0.9, [0.3, 0.4, 0.2], 1e-31, U1),
