@@ -178,8 +178,8 @@ BatchLayout batch_layout(const Batch &B)
         L.tl[q] = impact::table_layout(B.plans[q]);
         L.tables[q] = put(L.tl[q].total);
     }
-    L.upload_end = o;
     L.status = put(64);
+    L.upload_end = L.status + 64;   // its zeros go up with the tables
     L.scan = put((size_t)impact::scan_scratch_elems(B.rows) * 8);
     L.lb = put(!B.walks                    ? 0
                : B.prec == PREC_FP32_SOUND ? (size_t)B.rows * 16
@@ -267,7 +267,8 @@ void free_owned(impact_csr *out, cudaStream_t st)
     out->workspace_bytes = wsb;
 }
 
-// Copies the batch index, the descriptors and the tables into the workspace.
+// Copies the batch index, the descriptors, the tables and a zeroed status block
+// into the workspace.
 impact_status upload(const Batch &B, Work &W, cudaStream_t st)
 {
     const BatchLayout &L = W.L;
@@ -422,29 +423,33 @@ cudaError_t setup_pass(const Batch &B, const Work &W, cudaStream_t st)
 // row_flags: per-row counts, then the scan. FP64 builds whose tables are too
 // large for the walk (ImpactDesc.walk64) are counted by the per-pair kernel.
 impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cudaStream_t st,
-                        int64_t chunk_rows)
+                        int64_t chunk_rows, bool fresh)
 {
-    CK(cudaMemsetAsync(W.status(), 0, 64, st));
+    if (!fresh) CK(cudaMemsetAsync(W.status(), 0, 64, st));
     impact::RowOutputs o{out->row_ptr, nullptr, nullptr, nullptr, out->sink_lo, out->sink_up,
                          out->trunc, out->row_flags, W.status(), -1, B.rows};
+    const impact::ScanHead scan = impact::scan_head(out->row_ptr, B.rows, W.scan(), W.total());
     if (B.prec == PREC_FP32_SOUND) {
         CK(setup_pass(B, W, st));
         CK(impact::launch_leaf_fp32(W.index(), B.leaf_begin.back(), B.leaf_smem, st));
         CK(walk_pass(B, W, WALK_COUNT, B.tune.count_warps, o, W.counter(), chunk_rows, st));
-        CK(impact::launch_terms_fp32(W.index(), B.rows, W.lb(), B.tune.faults.fault_row, o, st));
-        CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st, W.total()));
+        CK(impact::launch_terms_fp32(W.index(), B.rows, W.lb(), B.tune.faults.fault_row, o, scan,
+                                     st));
+        CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st, W.total(), scan.tiles > 0));
         return IMPACT_OK;
     }
     if (B.any64) {
         CK(impact::launch_items64(W.index(), B.item_begin.back(), W.status(), st));
         CK(walk_pass64(B, W, false, o, W.counter(), chunk_rows, st));
-        CK(impact::launch_terms64(W.index(), B.rows, (const double *)W.lb(), o, st));
     }
     for (int q = 0; q < B.count(); ++q)
         if (!B.plans[q].desc.walk64)
             CK(impact::launch_rows(W.desc(q), B.prec, false, 0, B.plans[q].rows,
                                    shifted(o, B.row_begin[q], B.rows), st));
-    CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st, W.total()));
+    if (B.any64)   // after every count: its blocks begin the scan
+        CK(impact::launch_terms64(W.index(), B.rows, (const double *)W.lb(), o, scan, st));
+    CK(impact::launch_scan(out->row_ptr, B.rows, W.scan(), st, W.total(),
+                           B.any64 && scan.tiles > 0));
     return IMPACT_OK;
 }
 
@@ -481,20 +486,20 @@ impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int
 // tuning one_pass a single walk in which each row finds its offset by the
 // look-back and writes its pairs
 impact_status run_fused(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
-                        cudaStream_t st, int64_t chunk_rows)
+                        cudaStream_t st, int64_t chunk_rows, bool fresh)
 {
     if (B.prec != PREC_FP32_SOUND || !B.tune.one_pass) {
-        impact_status s = run_count(B, W, out, st, chunk_rows);
+        impact_status s = run_count(B, W, out, st, chunk_rows, fresh);
         if (s != IMPACT_OK) return s;
         return run_emit(B, W, out, capacity, true, st, chunk_rows);
     }
-    CK(cudaMemsetAsync(W.status(), 0, 64, st));
+    if (!fresh) CK(cudaMemsetAsync(W.status(), 0, 64, st));
     CK(setup_pass(B, W, st));
     if (B.rows > 0) CK(cudaMemsetAsync(W.lb(), 0, (size_t)B.rows * 8, st));
     else CK(cudaMemsetAsync(out->row_ptr, 0, 8, st));
     impact::RowOutputs o{out->row_ptr, out->col, out->lo, out->up, out->sink_lo, out->sink_up,
                          out->trunc, out->row_flags, W.status(), capacity, B.rows};
-    CK(impact::launch_terms_fp32(W.index(), B.rows, nullptr, -1, o, st));
+    CK(impact::launch_terms_fp32(W.index(), B.rows, nullptr, -1, o, impact::ScanHead(), st));
     CK(walk_pass(B, W, WALK_FUSED, B.tune.count_warps, o, W.counter(), chunk_rows, st));
     return IMPACT_OK;
 }
@@ -543,7 +548,7 @@ impact_status do_count(const Batch &B, impact_csr *out, cudaStream_t st)
     WorkHold hold{W, st};
     if (!W.owned) ws_tag(W.base, 0);
     if ((s = upload(B, W, st)) != IMPACT_OK) return s;
-    if ((s = run_count(B, W, out, st)) != IMPACT_OK) return s;
+    if ((s = run_count(B, W, out, st, 0, true)) != IMPACT_OK) return s;
     Outcome r;
     CK(cudaMemcpyAsync(&r, W.status(), sizeof(r), cudaMemcpyDeviceToHost, st));
     if ((s = release(W, st)) != IMPACT_OK) return s;
@@ -603,7 +608,7 @@ impact_status build_into(const Batch &B, impact_csr *out, bool lib_owned, cudaSt
     if ((s = upload(B, W, st)) != IMPACT_OK) return s;
     int64_t capacity = out->nnz;
     if (lib_owned) {   // the output size is known after the count pass
-        if ((s = run_count(B, W, out, st)) != IMPACT_OK) return s;
+        if ((s = run_count(B, W, out, st, 0, true)) != IMPACT_OK) return s;
         int64_t nnz = 0;
         CK(cudaMemcpyAsync(&nnz, W.total(), 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
@@ -618,7 +623,7 @@ impact_status build_into(const Batch &B, impact_csr *out, bool lib_owned, cudaSt
     } else {   // caller capacity: no host round trip
         impact_csr view;
         if ((s = pair_view(out, view)) != IMPACT_OK) return s;
-        if ((s = run_fused(B, W, &view, capacity, st)) != IMPACT_OK) return s;
+        if ((s = run_fused(B, W, &view, capacity, st, 0, true)) != IMPACT_OK) return s;
     }
     Outcome r;
     CK(cudaMemcpyAsync(&r, W.status(), sizeof(r), cudaMemcpyDeviceToHost, st));

@@ -41,6 +41,15 @@ cudaError_t launch_rows(const ImpactDesc *d_desc, int prec, bool emit, int64_t r
 
 int64_t scan_scratch_elems(int64_t n);
 
+// The row-pointer scan's first pass, for a kernel that does it beside its own
+// work (scan.cuh); tiles 0: none, there are too many.
+struct ScanHead {
+    int64_t *row_ptr = nullptr, *tsum = nullptr, *also = nullptr;
+    int64_t n = 0;
+    int tiles = 0;
+};
+ScanHead scan_head(int64_t *row_ptr, int64_t n, int64_t *scratch, int64_t *also);
+
 // Sets the message impact_last_error() returns on this host thread.
 void set_last_error(const std::string &msg);
 
@@ -142,8 +151,10 @@ cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, bool sha
                               int64_t item_units, uint32_t *status, cudaStream_t stream);
 // FP64 row terms of every row from its windows' numbers; acc: the sums that a
 // COUNT pass left in `lb` (null: only the sinks and the mass outside).
+// Its first `scan.tiles` blocks do the first pass of the scan.
 cudaError_t launch_terms_fp32(const BatchIndex *d_index, int64_t rows, const void *acc,
-                              int64_t fault_row, const RowOutputs &o, cudaStream_t stream);
+                              int64_t fault_row, const RowOutputs &o, const ScanHead &scan,
+                              cudaStream_t stream);
 // Leaf tables of the builds that share them (after the items, before a count
 // pass); leaf_smem: the largest leaf32_bytes of the batch.
 int leaf32_bytes(const ImpactDesc &D);
@@ -163,13 +174,14 @@ int64_t walk64_bytes(const ImpactDesc &D);   // shared memory of one warp
 cudaError_t launch_items64(const BatchIndex *d_index, int64_t units, uint32_t *status,
                            cudaStream_t stream);
 cudaError_t launch_terms64(const BatchIndex *d_index, int64_t rows, const double *acc,
-                           const RowOutputs &o, cudaStream_t stream);
+                           const RowOutputs &o, const ScanHead &scan, cudaStream_t stream);
 cudaError_t launch_walk64(const BatchIndex *d_index, int64_t row_begin, int64_t row_end,
                           int warp_smem, bool emit, const RowOutputs &o, double *acc,
                           int64_t rows, unsigned long long *counter, cudaStream_t stream);
 // Row pointers from per-row counts, in place; the total goes to row_ptr[n] and
-// to *also (may be null).
+// to *also (may be null). begun: a kernel given scan_head's value did the first
+// pass.
 cudaError_t launch_scan(int64_t *row_ptr, int64_t n, int64_t *scratch, cudaStream_t stream,
-                        int64_t *also = nullptr);
+                        int64_t *also = nullptr, bool begun = false);
 
 }  // namespace impact

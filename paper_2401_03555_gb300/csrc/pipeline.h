@@ -75,23 +75,25 @@ struct Work {
     }
 };
 
-// Copies the batch index, the descriptors and the tables into W (stream-ordered).
+// Copies the batch index, the descriptors, the tables and a zeroed status block
+// into W (stream-ordered).
 impact_status upload(const Batch &B, Work &W, cudaStream_t st);
 // The passes below launch the FP32 walk over all rows at once, or in chunks
 // of `chunk_rows` rows one after another on `st` (so that work on other
 // streams can take SMs between chunks); the FP64 kernels ignore chunk_rows.
-// count pass into out's row arrays (row pointers included).
+// count pass into out's row arrays (row pointers included). `fresh`: W's status
+// block is as an upload left it (zeroed).
 impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cudaStream_t st,
-                        int64_t chunk_rows = 0);
+                        int64_t chunk_rows = 0, bool fresh = false);
 // emit pass into out's pair arrays at the row pointers of a count pass
 // (`records_ready`: W holds the records or items of that count pass; `fresh`:
 // W's status block is as a count left it, or zeroed).
 impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
                        bool records_ready, cudaStream_t st, int64_t chunk_rows = 0,
                        bool fresh = true);
-// FP32: count and emit in one pass (capacity known); FP64: count, scan, emit.
+// The whole build into arrays of known capacity (`fresh` as in run_count).
 impact_status run_fused(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
-                        cudaStream_t st, int64_t chunk_rows = 0);
+                        cudaStream_t st, int64_t chunk_rows = 0, bool fresh = false);
 // Maps the device status word of a finished pipeline to a status code.
 impact_status status_result(uint32_t status);
 void configure_pool_once();

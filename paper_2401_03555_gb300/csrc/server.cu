@@ -259,7 +259,7 @@ void impact_server::admit()
     out.trunc = g->trunc;
     out.row_flags = g->flags;
     s = impact::upload(g->B, g->W, st);
-    if (s == IMPACT_OK) s = impact::run_count(g->B, g->W, &out, st, g->chunk_rows);
+    if (s == IMPACT_OK) s = impact::run_count(g->B, g->W, &out, st, g->chunk_rows, true);
     if (s == IMPACT_OK) {
         for (size_t q = 0; q <= take.size(); ++q)
             cudaMemcpyAsync(g->h_ptr + q, g->row_ptr + g->B.row_begin[q], 8,

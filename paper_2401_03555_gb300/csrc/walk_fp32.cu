@@ -61,6 +61,7 @@
 #include "impact_desc.h"
 #include "kernels.h"
 #include "rowmath.cuh"
+#include "scan.cuh"
 #include "sound_fp32.cuh"
 
 namespace {
@@ -443,13 +444,19 @@ __device__ __forceinline__ double widen(float x)
 // FP64 issues two lanes per clock and SM here, whatever share of a warp's
 // lanes is active: in the setup (n lanes per row) and at the end of a row's
 // walk (one lane) the same operations took 1.1 ms of the 11^5 room's 12.
-__global__ void __launch_bounds__(256)
+constexpr int kTermThreads = 256;
+__global__ void __launch_bounds__(kTermThreads)
 terms_fp32(const BatchIndex *__restrict__ B, const float4 *__restrict__ acc, int64_t fault_row,
            double *__restrict__ sink_lo, double *__restrict__ sink_up, double *__restrict__ trunc,
-           uint32_t *__restrict__ flags, uint32_t *__restrict__ status)
+           uint32_t *__restrict__ flags, uint32_t *__restrict__ status, impact::ScanHead scan)
 {
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < B->rows;
-         row += (int64_t)gridDim.x * blockDim.x) {
+    if (blockIdx.x < scan.tiles) {   // the row-pointer scan, in blocks of its own
+        rowscan::first_pass<kTermThreads>(scan);
+        return;
+    }
+    const int64_t rows = B->rows, step = (int64_t)(gridDim.x - scan.tiles) * kTermThreads;
+    for (int64_t row = (int64_t)(blockIdx.x - scan.tiles) * kTermThreads + threadIdx.x; row < rows;
+         row += step) {
         const int q = find_problem(B->row_begin, B->count, row);
         const ImpactDesc &D = *B->desc[q];
         const int n = D.n;
@@ -1955,12 +1962,14 @@ cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, bool sha
 }
 
 cudaError_t launch_terms_fp32(const BatchIndex *d_index, int64_t rows, const void *acc,
-                              int64_t fault_row, const RowOutputs &o, cudaStream_t stream)
+                              int64_t fault_row, const RowOutputs &o, const ScanHead &scan,
+                              cudaStream_t stream)
 {
     if (rows <= 0) return cudaSuccess;
-    const int g = occupancy_grid((const void *)terms_fp32, 256, 0, rows, 256);
-    terms_fp32<<<g, 256, 0, stream>>>(d_index, (const float4 *)acc, fault_row, o.sink_lo,
-                                      o.sink_up, o.trunc, o.flags, o.status);
+    const int g = occupancy_grid((const void *)terms_fp32, kTermThreads, 0, rows, kTermThreads);
+    terms_fp32<<<scan.tiles + g, kTermThreads, 0, stream>>>(
+        d_index, (const float4 *)acc, fault_row, o.sink_lo, o.sink_up, o.trunc, o.flags, o.status,
+        scan);
     return cudaGetLastError();
 }
 

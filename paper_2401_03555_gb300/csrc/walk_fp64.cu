@@ -39,6 +39,7 @@
 #include "impact_desc.h"
 #include "kernels.h"
 #include "rowmath.cuh"
+#include "scan.cuh"
 
 namespace {
 
@@ -304,13 +305,19 @@ items_fp64(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
 
 // Row terms after the count walk (acc: its dropped mass, upper and lower sums
 // per row).
-__global__ void __launch_bounds__(256)
+constexpr int kTermThreads = 256;
+__global__ void __launch_bounds__(kTermThreads)
 terms_fp64(const BatchIndex *__restrict__ B, const double *__restrict__ acc,
            double *__restrict__ sink_lo, double *__restrict__ sink_up, double *__restrict__ trunc,
-           uint32_t *__restrict__ flags, uint32_t *__restrict__ status)
+           uint32_t *__restrict__ flags, uint32_t *__restrict__ status, impact::ScanHead scan)
 {
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < B->rows;
-         row += (int64_t)gridDim.x * blockDim.x) {
+    if (blockIdx.x < scan.tiles) {   // the row-pointer scan, in blocks of its own
+        rowscan::first_pass<kTermThreads>(scan);
+        return;
+    }
+    const int64_t rows = B->rows, step = (int64_t)(gridDim.x - scan.tiles) * kTermThreads;
+    for (int64_t row = (int64_t)(blockIdx.x - scan.tiles) * kTermThreads + threadIdx.x; row < rows;
+         row += step) {
         const int q = find_problem(B->row_begin, B->count, row);
         const ImpactDesc &D = *B->desc[q];
         if (!D.walk64) continue;
@@ -869,12 +876,12 @@ cudaError_t launch_items64(const BatchIndex *d_index, int64_t units, uint32_t *s
 }
 
 cudaError_t launch_terms64(const BatchIndex *d_index, int64_t rows, const double *acc,
-                           const RowOutputs &o, cudaStream_t stream)
+                           const RowOutputs &o, const ScanHead &scan, cudaStream_t stream)
 {
     if (rows <= 0) return cudaSuccess;
-    const int g = blocks_for((const void *)terms_fp64, 256, 0, rows, 256);
-    terms_fp64<<<g, 256, 0, stream>>>(d_index, acc, o.sink_lo, o.sink_up, o.trunc, o.flags,
-                                      o.status);
+    const int g = blocks_for((const void *)terms_fp64, kTermThreads, 0, rows, kTermThreads);
+    terms_fp64<<<scan.tiles + g, kTermThreads, 0, stream>>>(
+        d_index, acc, o.sink_lo, o.sink_up, o.trunc, o.flags, o.status, scan);
     return cudaGetLastError();
 }
 

@@ -92,3 +92,22 @@ def test_mixed_batch_equals_its_builds(orc):
         one, part = impact.build(p, "fp64"), batch.part(q)
         for k in ("row_ptr", "col", "lo", "up", "sink_lo", "sink_up", "trunc", "row_flags"):
             assert torch.equal(getattr(one, k), getattr(part, k)), (q, k)
+
+
+# rows around one tile of the row-pointer scan (4096 rows) and around the most
+# tiles that the row-terms kernels begin the scan for (152)
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("cells,inputs", [(1, 1), (64, 64), (17, 241), (64, 9728), (3, 207531)])
+def test_row_pointers_at_the_scan_tiles(cells, inputs, precision):
+    """Row pointers against running sums of the kept pairs of the dense build
+    (exact: FP64 keeps by the same values; FP32 is checked dense)."""
+    U = np.resize([[-0.3], [0.4], [0.0], [1.2]], (inputs, 1))
+    dense = linear([cells], [[0.9]], [0.8], 0.0, U)
+    csr = impact.build(dense, precision)
+    want = torch.arange(dense.rows + 1, device="cuda") * cells
+    assert torch.equal(csr.row_ptr, want)
+    if precision == "fp64":
+        kept = (csr.up.view(dense.rows, cells) >= 1e-3).sum(1).cumsum(0)
+        got = impact.build(linear([cells], [[0.9]], [0.8], 1e-3, U), "fp64")
+        assert int(got.row_ptr[0]) == 0 and torch.equal(got.row_ptr[1:], kept)
+        assert got.nnz == int(kept[-1])
