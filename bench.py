@@ -58,7 +58,7 @@ WORKLOAD = workload_name()
 LAUNCHES_PER_STEP = 8
 BATCHED_LAUNCHES = 6
 # FP64 rate of the GB300 FMA pipe, measured with a dependent-chain DFMA
-# probe (2 flops per DFMA): the bound of the FP64-plain path
+# probe (2 flops per DFMA)
 FP64_PEAK_GFLOPS = 1200.0
 L2_FLUSH_BYTES = 512 << 20
 
@@ -240,19 +240,18 @@ def walk_traffic(alg_bytes):
     return None if r is None else int(r * alg_bytes)
 
 
-def fp64_roofline(pairs, ms):
-    """The FP64-plain build against the FP64 pipe: its FP64 flops per pair
-    (2 per DFMA + DADD + DMUL, counted by ncu over both passes on the 7^5 room)
-    times the pairs, over the build's time."""
-    f = profile_figure("room5d_fp64_rows_ncu.txt", "kernels.cu", "fp64_flops_per_pair")
-    out = {"bound": "fp64", "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
-           "peak_source": "measured (dependent-chain DFMA probe on GB300)",
-           "flops_per_pair": f}
-    if f is None:
-        out.update({"achieved": None, "frac": None})
-    else:
-        ach = f * pairs / (ms / 1e3) / 1e9
-        out.update({"achieved": round(ach, 1), "frac": round(ach / FP64_PEAK_GFLOPS, 4)})
+def fp64_roofline(pairs, rows, ms, peak, peak_kind):
+    """The FP64-plain build against the bytes it writes (20 B/pair, 36 B/row),
+    and against the FP64 pipe by its flops per pair (2 per DFMA + DADD + DMUL,
+    counted by ncu over a whole build of the 7^5 room)."""
+    ach = (pairs * 20 + rows * 36) / (ms / 1e3) / 1e9
+    out = {"bound": "hbm", "achieved": round(ach, 1), "peak": peak, "unit": "GB/s",
+           "frac": round(ach / peak, 4), "peak_source": peak_kind,
+           "bytes_model": "20 B/pair + 36 B/row written, over the build's time"}
+    f = profile_figure("room5d_fp64_walk_ncu.txt", "walk_fp64.cu", "fp64_flops_per_pair")
+    if f is not None:
+        out["fp64_flops_per_pair"] = f
+        out["fp64_pipe_frac"] = round(f * pairs / (ms / 1e3) / 1e9 / FP64_PEAK_GFLOPS, 4)
     return out
 
 
@@ -458,9 +457,9 @@ def run_ours(args, rank, world, local_rank):
                 "bytes_model": "12 B/pair written + 16 B/row read",
                 "step_frac": round(step_bytes / (ms_local / 1e3) / 1e9 / peak, 4),
                 "step_bytes_model": "12 B/pair + 36 B/row written, over ms_per_step",
-                # every erf/erfc evaluation of the build is in setup_fp32, which
+                # every erf/erfc evaluation of the build is in items_fp32, which
                 # runs inside impact_count: the count call's time bounds it
-                "erfc_term": {"kernel": "setup_fp32 (within impact_count)",
+                "erfc_term": {"kernel": "items_fp32 (within impact_count)",
                               "ms_upper_bound": two["count_ms"],
                               "hbm_term_ms": round(emit_bytes / peak / 1e6, 3)}}
 
@@ -495,8 +494,11 @@ def run_ours(args, rank, world, local_rank):
                              mode=args.e2e_mode)
         torch.cuda.empty_cache()
 
-    # FP64-plain GPU path on the same workload (one build, rank-local)
+    # FP64-plain GPU path on the same workload (one build after a warm-up, whose
+    # output blocks stay in the library's pool; rank-local)
     if not args.no_fp64 and rank == 0:
+        c64 = impact.build(prob, "fp64")
+        del c64
         torch.cuda.synchronize(dev)
         s = torch.cuda.Event(enable_timing=True)
         e = torch.cuda.Event(enable_timing=True)
@@ -507,7 +509,7 @@ def run_ours(args, rank, world, local_rank):
         ms64 = s.elapsed_time(e)
         out["fp64_plain"] = {"value": c64.nnz / (ms64 / 1e3), "unit": UNIT, "ms": ms64,
                              "pairs": c64.nnz, "fp32_over_fp64": value / world / (c64.nnz / (ms64 / 1e3)),
-                             "roofline": fp64_roofline(c64.nnz, ms64)}
+                             "roofline": fp64_roofline(c64.nnz, rows, ms64, peak, peak_kind)}
         del c64
         torch.cuda.empty_cache()
 
@@ -650,7 +652,7 @@ def run_batched(dev, stream, reps=2, cap_pairs=8_000_000_000):
                         "peak_source": peak_kind, "algorithmic_bytes_per_pass": alg_bytes,
                         "bytes_model": "12 B/pair + 36 B/row written",
                         "time": "every group's graph replay, back to back"},
-           "path": "impact_graph_launch per group (setup, count, scan and emit, each one "
+           "path": "impact_graph_launch per group (setup, count, terms, scan and emit, each one "
                    "persistent launch over every system of the group)"}
     out["fp64_plain"] = batched_fp64_sample(probs, dev)
     return out
@@ -658,8 +660,7 @@ def run_batched(dev, stream, reps=2, cap_pairs=8_000_000_000):
 
 def batched_fp64_sample(probs, dev, pairs_target=150_000_000):
     """FP32-sound against FP64 plain on the first systems of the batched
-    workload (about `pairs_target` pairs: the FP64 plain kernel evaluates erfc
-    in FP64 per pair and dimension, so the whole workload would take minutes)."""
+    workload (about `pairs_target` pairs)."""
     import torch
     from paper_2401_03555_gb300 import impact
     take, acc = [], 0
@@ -765,8 +766,8 @@ def run_mc(draws=1024, oracle_rows=4):
     dt = time.perf_counter() - t0
     out = {"workload": MC_WORKLOAD, "rows": int(prob.rows), "pairs": int(g.nnz), "ms": dt * 1e3,
            "value": g.nnz / dt, "unit": "pairs/s", "row_draws_per_s": prob.rows * draws / dt,
-           "path": "impact_build_mc (one block per row: shared-memory histograms of the cells "
-                   "each moved image box meets / lies in; count, scan, emit)"}
+           "path": "impact_build_mc (per distinct image and cell a mask of the draws, one warp "
+                   "per row over the masks' products; count, scan, emit)"}
     del g
     try:
         import oracle
@@ -805,7 +806,8 @@ def run_regions(reps=5, oracle_rows=16):
         torch.cuda.synchronize()
         ms = (time.perf_counter() - t0) * 1e3 / reps
         out[mode] = {"ms": ms, "value": prob.rows / (ms * 1e-3),
-                     "path": "impact_region_vectors (plan upload + one thread per row)"}
+                     "path": "impact_region_vectors (plan upload, factors of every distinct image, "
+                            "products per row)"}
     try:
         import oracle
         rows = W.sample_rows(prob, oracle_rows, seed=5, include_boundary=False)

@@ -188,9 +188,10 @@ impact_status impact_build(const impact_system *sys, const impact_grid *grid,
                            impact_precision precision, impact_csr *out, void *stream);
 
 /*
- * impact_workspace_bytes -- host-only: the device scratch one build uses (the
- * uploaded descriptor and tables, the scan partial sums and, for
- * IMPACT_FP32_SOUND, one 8-byte offset word per row).
+ * impact_workspace_bytes -- host-only: the device scratch one build uses: the
+ * uploaded descriptor and tables, the scan partial sums, the windows of the
+ * distinct images and, per row, 16 bytes and the row's record
+ * (IMPACT_FP32_SOUND) or 24 bytes (IMPACT_FP64_PLAIN).
  */
 impact_status impact_workspace_bytes(const impact_system *sys, const impact_grid *grid,
                                      const impact_inputs *inputs, const double *sigma,
@@ -644,8 +645,8 @@ impact_status impact_debug_live_bytes(int64_t *device_bytes, int64_t *host_bytes
 #define IMPACT_SCAN_STATIC_MAX_ROWS (1LL << 27)
 
 /*
- * impact_scan_rows_static -- the row-pointer scan (the one the FP64-plain count
- * pass and impact_build_mc run), for callers that must not allocate device
+ * impact_scan_rows_static -- the row-pointer scan (the one every build runs
+ * after its count pass), for callers that must not allocate device
  * memory. The paper has no counterpart: this is
  * a deployment convenience, not part of the method.
  *

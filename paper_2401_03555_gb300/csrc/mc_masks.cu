@@ -423,7 +423,10 @@ namespace impact {
 
 // The masks pay per tree node, so: a cutoff (kmin >= 1 prunes the tree), rows
 // that share images, up to 4096 draws (four words per lane) and masks that stay
-// near the L2 (256 MB at most). Else bytes stays 0.
+// near the L2 (256 MB at most). Else bytes stays 0. Room 6^5, 100 / 1000 / 4096
+// draws, masks against histograms: cutoff 1e-6 (every met cell kept) 1.8 / 2.1 /
+// 5.0 against 13.3 / 38.6 / 232 ms, cutoff 2e-2 1.7 / 1.6 / 3.4 against 13.1 /
+// 38.6 / 232.
 McMasks mc_masks(const ImpactDesc &D, int64_t S, double cutoff)
 {
     McMasks K{};

@@ -1,7 +1,7 @@
 // static_scan.cu -- the row-pointer scan for callers that cannot allocate.
 //
 // impact_scan_rows_static turns per-row pair counts into CSR row pointers in
-// place, like the scan of the FP64-plain count pass, but its scratch (one partial sum
+// place, like the scan after a count pass, but its scratch (one partial sum
 // per tile of rows) lives in a fixed file-scope device array instead of
 // memory allocated per call. Nothing here calls cudaMalloc, cudaFree or any
 // allocating library routine.

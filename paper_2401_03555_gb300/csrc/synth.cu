@@ -32,9 +32,10 @@
 // What bounds it: the row kernel's FP64 multiplies and adds (2 lanes per clock
 // and SM on this part), about five per successor and vector; their order is
 // part of the result (ties between inputs), so it is kept. Dense robot 21x21
-// (3969 rows of 441 successors, about 270 iterations): 54 -> 23.8 ms; a 62-step
+// (3969 rows of 441 successors, about 270 iterations): 44 -> 16 ms; a 62-step
 // bisection over the doubles for each vector took 140 us of an iteration's 200,
-// the host's stopping test 50.
+// the host's stopping test 50. Now 37 for the rows, 6 for the cells, 4 for the
+// ranks.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>

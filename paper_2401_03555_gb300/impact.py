@@ -306,7 +306,7 @@ def plan(prob, precision="fp32"):
 
 
 def workspace_bytes(prob, precision="fp32") -> int:
-    """Device scratch bytes of one build (descriptor, tables, scan, offset words)."""
+    """Device scratch bytes of one build (descriptor, tables, scan, records or items, row sums)."""
     a = _Args(prob, need_images=False)
     if prob.kind == 2:
         a.sys.dev_images = 1
