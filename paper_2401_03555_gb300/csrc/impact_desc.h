@@ -37,7 +37,7 @@ struct ImpactDim {
     int64_t item_mul[IMPACT_MAX_DIM];   // 0: the image does not read dimension k
     int n_classes;        // classes of inputs
     int w64;              // FP64: targets an item's table holds (largest window)
-    int group;            // lanes that make one item (FP64: 8, 16 or 32; FP32: 1)
+    int group;            // lanes that make one item (FP64: 8, 16 or 32; FP32: 1 or 8)
     int item_stride;      // bytes of one item
     int64_t item_off;     // bytes of the build's items before this dimension's
 };

@@ -381,21 +381,179 @@ __device__ DimOut setup_dim(const ImpactDesc &D, int64_t row, const int *idx, in
     return o;
 }
 
+// The pieces of setup_dim for a window that several lanes make. (setup_dim keeps
+// its own text: built from these, setup_fp32 took 1.06 ms for 24 random systems,
+// not 1.01.) Bounds of a target's factor from its edges c, e at the image's lower
+// (0) and upper (1) end.
+__device__ __forceinline__ float2 target_factor(const ImpactDim &g, const EdgePt &c0,
+                                                const EdgePt &e0, const EdgePt &c1,
+                                                const EdgePt &e1)
+{
+    if (mid_below(c0, e0))              // target midpoint <= m_lo
+        return make_float2(sound::cell_hi(c0.a, c0.t, e0.a, e0.t),
+                           sound::cell_lo(c1.a, c1.t, e1.a, e1.t));
+    if (mid_above(c1, e1))              // target midpoint >= m_hi
+        return make_float2(sound::cell_hi(c1.a, c1.t, e1.a, e1.t),
+                           sound::cell_lo(c0.a, c0.t, e0.a, e0.t));
+    return make_float2(g.plateau_hi,    // midpoint may be inside
+                       fminf(sound::cell_lo(c0.a, c0.t, e0.a, e0.t),
+                             sound::cell_lo(c1.a, c1.t, e1.a, e1.t)));
+}
+
+// The trimmed window and its sums, targets taken in order.
+struct Trim {
+    int first = -1, last = -1;
+    float pre = 0.0f, mid = 0.0f, post = 0.0f, M = 0.0f;
+    __device__ __forceinline__ void take(int k, float U, float cut)
+    {
+        if (U >= cut) {
+            if (first < 0) {
+                first = k;
+                mid = U;
+            } else {
+                mid = __fadd_ru(mid, __fadd_ru(post, U));
+                post = 0.0f;
+            }
+            last = k;
+            M = fmaxf(M, U);
+        } else if (first < 0) {
+            pre = __fadd_ru(pre, U);
+        } else {
+            post = __fadd_ru(post, U);
+        }
+    }
+};
+
+// The rest of a window: the mass outside it and the out-of-domain bounds, from
+// its first edge at m_lo (w0), its last at m_hi (w1) and the domain's edges.
+__device__ __forceinline__ DimOut dim_out(const ImpactDim &g, const Win &h, const Trim &s,
+                                          const EdgePt &w0, const EdgePt &w1, const EdgePt &lo0,
+                                          const EdgePt &hi0, const EdgePt &lo1, const EdgePt &hi1)
+{
+    DimOut o;
+    o.a = h.a;
+    float O = __fadd_ru(s.pre, s.post);
+    if (h.a > 0)   // cells 0..a-1 lie left of the image: their mass at m_lo
+        O = __fadd_ru(O, sound::cell_hi(lo0.a, lo0.t, w0.a, w0.t));
+    if (h.a + h.W < g.N)   // cells right of the window: their mass at m_hi
+        O = __fadd_ru(O, sound::cell_hi(w1.a, w1.t, hi1.a, hi1.t));
+    // out-of-domain mass Q(m) = T(-alpha(lo_D)) + T(alpha(hi_D))
+    const float q0 = __fadd_ru(lo0.t.m_hi, hi0.t.p_hi);
+    const float q1 = __fadd_ru(lo1.t.m_hi, hi1.t.p_hi);
+    o.qhi = fminf(fmaxf(q0, q1), 1.0f);
+    float qlo;
+    if (mid_below(lo0, hi0))
+        qlo = __fadd_rd(lo0.t.m_lo, hi0.t.p_lo);
+    else if (mid_above(lo1, hi1))
+        qlo = __fadd_rd(lo1.t.m_lo, hi1.t.p_lo);
+    else
+        qlo = g.qmin_lo;
+    o.qlo = fminf(qlo, 1.0f);
+    o.tw = s.first >= 0 ? s.last - s.first + 1 : 0;
+    o.f0 = s.first >= 0 ? s.first : 0;
+    o.M = s.M;
+    o.SW = s.mid;
+    o.O = O;
+    return o;
+}
+
+// A lane's edge point seen by the others of its group of G.
+template <int G>
+__device__ __forceinline__ EdgePt edge_from(const EdgePt &e, int src)
+{
+    EdgePt r;
+    r.a = __shfl_sync(0xffffffffu, e.a, src, G);
+    r.da = __shfl_sync(0xffffffffu, e.da, src, G);
+    r.t.p_lo = __shfl_sync(0xffffffffu, e.t.p_lo, src, G);
+    r.t.p_hi = __shfl_sync(0xffffffffu, e.t.p_hi, src, G);
+    r.t.m_lo = __shfl_sync(0xffffffffu, e.t.m_lo, src, G);
+    r.t.m_hi = __shfl_sync(0xffffffffu, e.t.m_hi, src, G);
+    return r;
+}
+
+// setup_dim by a group of G lanes (4 or 8), one edge each per round: the same
+// values, all lanes of the warp together (inactive groups: act false). Few
+// windows leave most of the chip idle and take as long as the longest chain of
+// tails, which this cuts to the rounds; many are cheaper one lane each, since
+// here every lane of a group repeats the image and the sums.
+template <int G>
+__device__ DimOut setup_dim_split(const ImpactDesc &D, int64_t row, const int *idx, int j, int d,
+                                  float2 *ul, uint32_t *status, bool act)
+{
+    const int lane = threadIdx.x & (G - 1);
+    Win h;
+    h.W = -1;
+    h.a = 0;
+    if (act && !dim_window(D, row, idx, j, d, h)) {
+        if (lane == 0) atomicOr(status, IMPACT_STATUS_TABLE_OVERFLOW);
+        act = false;
+    }
+    const ImpactDim &g = D.dim[d];
+    const int W = act ? h.W : -1;   // edges 0..W
+    const int rounds = __reduce_max_sync(0xffffffffu, (W + G) / G);
+    EdgePt x{}, y{}, last0{}, last1{};
+    Trim s;
+    for (int r = 0; r < rounds; ++r) {
+        const int k = r * G + lane;
+        x = EdgePt{};
+        y = EdgePt{};
+        if (k <= W) {
+            x = edge_at(h, k, false);
+            y = edge_at(h, k, true);
+        }
+        // target k - 1 lies between the edges of the lane before and this one
+        EdgePt c0 = edge_from<G>(x, (lane + G - 1) & (G - 1));
+        EdgePt c1 = edge_from<G>(y, (lane + G - 1) & (G - 1));
+        const EdgePt n0 = edge_from<G>(x, G - 1), n1 = edge_from<G>(y, G - 1);
+        if (lane == 0) {
+            c0 = last0;
+            c1 = last1;
+        }
+        last0 = n0;
+        last1 = n1;
+        float2 f = make_float2(0.0f, 0.0f);
+        if (k >= 1 && k <= W) {
+            f = target_factor(g, c0, x, c1, y);
+            ul[k - 1] = f;
+        }
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            const float U = __shfl_sync(0xffffffffu, f.x, i, G);
+            const int kk = r * G + i;
+            if (kk >= 1 && kk <= W) s.take(kk - 1, U, D.cutoff32);
+        }
+    }
+    // the window's and the domain's edges, one lane each
+    auto end = [&](int i) {
+        const int k = i < 4 ? (i & 1 ? g.N : 0) - h.a : i == 4 ? 0 : h.W;
+        return edge_at(h, k, i == 2 || i == 3 || i == 5);
+    };
+    x = EdgePt{};
+    y = EdgePt{};
+    if (act && lane < 6) x = end(lane);
+    if (G == 4 && act && lane < 2) y = end(4 + lane);
+    const EdgePt w0 = G == 4 ? edge_from<G>(y, 0) : edge_from<G>(x, 4);
+    const EdgePt w1 = G == 4 ? edge_from<G>(y, 1) : edge_from<G>(x, 5);
+    const EdgePt lo0 = edge_from<G>(x, 0), hi0 = edge_from<G>(x, 1);
+    const EdgePt lo1 = edge_from<G>(x, 2), hi1 = edge_from<G>(x, 3);
+    return act ? dim_out(g, h, s, w0, w1, lo0, hi0, lo1, hi1) : DimOut();
+}
+
 // What one lane of a row's dimensions finishes with the row's others (the
-// lanes of a row are `base` .. `base + n - 1`): its record entry with the
+// lanes of a row are `base`, `base + step`, .. one per dimension): its record entry with the
 // pruning threshold (a child t of a node with product P survives iff
 // RU(RU(P U[t]) R') >= cutoff, R' the product of the later dimensions' largest
 // factors grown by 2^-18 to cover the rounding of the rest of the chain; cp is
 // the least such child product).
 __device__ __forceinline__ void finish_dim(const ImpactDesc &D, const DimOut &o, int d, int base,
-                                           bool act, unsigned char *rr)
+                                           bool act, unsigned char *rr, int step = 1)
 {
     const int n = D.n;
     float R = 1.0f, SR = 1.0f;
 #pragma unroll
     for (int k = 0; k < IMPACT_MAX_DIM; ++k) {
         if (k < n) {   // n is the same for the whole warp
-            const int src = (base + k) & 31;
+            const int src = (base + k * step) & 31;
             const float Mk = __shfl_sync(0xffffffffu, o.M, src);
             const float SWk = __shfl_sync(0xffffffffu, o.SW, src);
             if (k > d) {
@@ -540,8 +698,43 @@ setup_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
     }
 }
 
+// The same for few rows: four lanes per (row, dimension), a unit's 32/n rows in
+// parts of 8/n.
+__global__ void __launch_bounds__(128)
+setup_split_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
+{
+    constexpr int G = 4, kParts = 6;   // (32/n) / (8/n) rounded up, at most
+    const int lane = threadIdx.x & 31;
+    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t v = warp0; v < B->units * kParts; v += nwarps) {
+        const int64_t u = v / kParts;
+        const int q = find_problem(B->unit_begin, B->count, u);
+        const ImpactDesc &D = *B->desc[q];
+        if (D.share32) continue;
+        const int n = D.n;
+        const int rpw = 32 / n, rpp = 32 / (G * n);
+        const int slot = lane / (G * n), d = (lane - slot * G * n) / G;
+        const int r = (int)(v - u * kParts) * rpp + slot;   // row of the unit
+        if (r - slot >= rpw) continue;
+        const int64_t rows_q = B->row_begin[q + 1] - B->row_begin[q];
+        const int64_t rl = (u - B->unit_begin[q]) * rpw + r;
+        const bool act = slot < rpp && r < rpw && rl < rows_q;
+        unsigned char *rr = act ? B->rec[q] + rl * (int64_t)D.rec_stride : nullptr;
+        int idx[IMPACT_MAX_DIM], j = 0;
+        if (act) rowmath::decode_row(D, rl, idx, j);
+        const DimOut o = setup_dim_split<G>(D, rl, idx, j, d,
+                                            act ? rec_table(rr, n) + D.dim[d].rec_off : nullptr,
+                                            status, act);
+        const bool head = act && (lane & (G - 1)) == 0;
+        if (head) reinterpret_cast<float4 *>(B->terms[q])[rl * n + d] = term_of(o);
+        finish_dim(D, o, d, slot * G * n, head, rr, G);
+    }
+}
+
 // items_fp32: the window and factor table of every distinct image
-// (impact_desc.h), one lane each: DimOut, then the window's (U, L) pairs.
+// (impact_desc.h), one lane or (few items, ImpactDim.group) eight lanes each:
+// DimOut, then the window's (U, L) pairs.
 __device__ __forceinline__ float2 *item_table(unsigned char *it)
 {
     return reinterpret_cast<float2 *>(it + sizeof(DimOut));
@@ -552,11 +745,21 @@ items_fp32(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
 {
     const int64_t total = B->item_units * 32;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
+         i += (int64_t)gridDim.x * blockDim.x) {   // a warp's lanes share a unit
         const int seg = find_problem(B->item_begin, B->count * IMPACT_MAX_DIM, i >> 5);
         const int q = seg / IMPACT_MAX_DIM, d = seg % IMPACT_MAX_DIM;
         const ImpactDesc &D = *B->desc[q];
         const ImpactDim &g = D.dim[d];
+        if (g.group == 8) {
+            const int64_t c = (i - B->item_begin[seg] * 32) / 8;
+            const bool act = c < g.n_items;
+            int idx[IMPACT_MAX_DIM], j = 0;
+            if (act) rowmath::decode_item(D, d, c, idx, j);
+            unsigned char *it = B->items[q] + g.item_off + c * g.item_stride;
+            const DimOut o = setup_dim_split<8>(D, c, idx, j, d, item_table(it), status, act);
+            if (act && (i & 7) == 0) *reinterpret_cast<DimOut *>(it) = o;
+            continue;
+        }
         const int64_t c = i - B->item_begin[seg] * 32;
         if (c >= g.n_items) continue;
         int idx[IMPACT_MAX_DIM], j;
@@ -1907,6 +2110,14 @@ int walk_core_bytes(int n, int tsum_cap, int leaf_cap)
     return (int)std::min<int64_t>(b, INT32_MAX / 2);
 }
 
+// Windows by groups of lanes (setup_dim_split) while they leave the chip idle. One
+// lane each against groups: items_fp32 22.6 against 10.8 us (robot 21^2, 4k rows),
+// 13.1 against 10.4 (room 9^5, 11k items), 14.1 against 16.3 (room 11^5, 20k);
+// per row 18.5 against 12.0 us (33x31 cells, 4 inputs, 256 units), 16.6 against
+// 11.5 (9^3, 292), 18.1 against 24.0 (64^2, 1024), 48.7 against 119 (160^2, 6400).
+constexpr int64_t kSplitItems = 12288;
+constexpr int64_t kSplitUnits = 456;   // three warps of setup_fp32 per SM
+
 // Shared windows pay when a window serves three rows or more (below that the
 // items' write and read back cost about what they save): the 11^5 room's 20k
 // windows take 0.014 ms and the gather of 1.45M records 0.37 ms, one setup per
@@ -1921,7 +2132,6 @@ void size_items32(ImpactDesc &D, int64_t &item_bytes, int64_t &leaf_bytes)
     int64_t bytes = 0, items = 0;
     for (int d = 0; d < n; ++d) {
         ImpactDim &g = D.dim[d];
-        g.group = 1;
         g.item_stride = (int)sizeof(DimOut) + 8 * ((g.wcap + 1) & ~1);
         g.item_off = bytes;
         bytes += g.n_items * (int64_t)g.item_stride;
@@ -1929,6 +2139,7 @@ void size_items32(ImpactDesc &D, int64_t &item_bytes, int64_t &leaf_bytes)
     }
     D.share32 = D.kind != KIND_IMAGES && items * 3 <= D.rows * n;
     item_bytes = D.share32 ? bytes : 0;
+    for (int d = 0; d < n; ++d) D.dim[d].group = items <= kSplitItems ? 8 : 1;
     const bool lists = D.leaf_cap >= kListCapMin && D.leaf_cap <= kListCapMax;
     D.leaf_stride = leaf_lists_at(D.leaf_cap) + (lists ? list_block(kListMax) : 0);
     D.leaf_shared = D.share32 && n >= 3 && D.cutoff32 > 0.0f && D.leaf_items * 4 <= D.rows &&
@@ -1948,7 +2159,10 @@ cudaError_t launch_setup_fp32(const BatchIndex *d_index, int64_t units, bool sha
                               int64_t item_units, uint32_t *status, cudaStream_t stream)
 {
     if (units <= 0) return cudaSuccess;
-    if (own) {
+    if (own && units <= kSplitUnits) {
+        const int g = occupancy_grid((const void *)setup_split_fp32, 128, 0, units * 6, 128 / 32);
+        setup_split_fp32<<<g, 128, 0, stream>>>(d_index, status);
+    } else if (own) {
         const int g = occupancy_grid((const void *)setup_fp32, 256, 0, units, 256 / 32);
         setup_fp32<<<g, 256, 0, stream>>>(d_index, status);
     }

@@ -111,3 +111,21 @@ def test_row_pointers_at_the_scan_tiles(cells, inputs, precision):
         got = impact.build(linear([cells], [[0.9]], [0.8], 1e-3, U), "fp64")
         assert int(got.row_ptr[0]) == 0 and torch.equal(got.row_ptr[1:], kept)
         assert got.nnz == int(kept[-1])
+
+
+@pytest.mark.parametrize("cells", [[1], [2, 3], [3, 4], [5, 7], [8, 9], [2, 3, 4], [3, 2, 3, 2],
+                                   [3, 2, 2, 2, 2], [2, 2, 3, 2, 2, 2], [2] * 7, [2] * 8])
+def test_windows_by_lane_groups_equal_those_by_lanes(cells):
+    """Few rows of distinct images make their windows by groups of lanes, rows
+    beside many others by single lanes: bitwise the same. Window widths (the
+    grid's, up to 9) around the group of 4; dimensions that fill a warp unevenly."""
+    n = len(cells)
+    A = np.eye(n) * 0.7 + 0.05
+    small = linear(cells, A, [2.0] * n, 1e-9, U2)
+    images = images_of(small, 5)
+    big = linear([80, 80], np.eye(2) * 0.7 + 0.05, [0.6] * 2, 1e-6, U2)   # 25600 rows
+    batch = impact.Batch([small, big, images], "fp32").build()
+    for q, p in ((0, small), (2, images)):
+        one, part = impact.build(p, "fp32"), batch.part(q)
+        for k in ("row_ptr", "col", "lo", "up", "sink_lo", "sink_up", "trunc", "row_flags"):
+            assert torch.equal(getattr(one, k), getattr(part, k)), (q, k)
