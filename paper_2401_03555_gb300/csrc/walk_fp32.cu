@@ -60,6 +60,7 @@
 #include "../../include/impact.h"
 #include "impact_desc.h"
 #include "kernels.h"
+#include "launch.h"
 #include "rowmath.cuh"
 #include "scan.cuh"
 #include "sound_fp32.cuh"
@@ -2192,8 +2193,7 @@ cudaError_t launch_leaf_fp32(const BatchIndex *d_index, int64_t tables, int leaf
 {
     if (tables <= 0) return cudaSuccess;
     const size_t smem = (size_t)leaf_smem * 4;
-    cudaError_t e = cudaFuncSetAttribute((const void *)leaf_fp32,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void *)leaf_fp32);
     if (e != cudaSuccess) return e;
     const int g = occupancy_grid((const void *)leaf_fp32, 128, smem, tables, 4);
     leaf_fp32<<<g, 128, smem, stream>>>(d_index, leaf_smem);
@@ -2221,7 +2221,7 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
     const void *k = mode == MODE_COUNT  ? (const void *)walk_fp32<MODE_COUNT>
                     : mode == MODE_EMIT ? (const void *)walk_fp32<MODE_EMIT>
                                         : (const void *)walk_fp32<MODE_FUSED>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     WalkArgs A;
     A.B = d_index;

@@ -38,6 +38,7 @@
 
 #include "impact_desc.h"
 #include "kernels.h"
+#include "launch.h"
 #include "rowmath.cuh"
 #include "scan.cuh"
 
@@ -894,7 +895,7 @@ cudaError_t launch_walk64(const BatchIndex *d_index, int64_t row_begin, int64_t 
     const int warps = std::max(1, std::min(kWarps, 200 * 1024 / std::max(warp_smem, 1)));
     const size_t smem = (size_t)warp_smem * warps;
     const void *k = emit ? (const void *)walk_fp64<true> : (const void *)walk_fp64<false>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     Walk64Args A;
     A.B = d_index;
