@@ -38,6 +38,18 @@ void track(void *p, size_t bytes, bool host)
     (host ? g_host_bytes : g_dev_bytes) += (int64_t)bytes;
 }
 
+// A failed allocation leaves neither a pointer nor an error that the check after
+// the next launch would take for its own.
+void settle(cudaError_t e, void **p, size_t bytes, bool host)
+{
+    if (e == cudaSuccess) {
+        track(*p, bytes, host);
+    } else {
+        *p = nullptr;
+        cudaGetLastError();
+    }
+}
+
 void untrack(void *p)
 {
     if (!p) return;
@@ -57,8 +69,7 @@ cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t st)
     *p = nullptr;
     if (injected_failure()) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaMallocAsync(p, bytes, st);
-    if (e == cudaSuccess) track(*p, bytes, false);
-    else *p = nullptr;
+    settle(e, p, bytes, false);
     return e;
 }
 
@@ -74,8 +85,7 @@ cudaError_t dev_malloc(void **p, size_t bytes)
     *p = nullptr;
     if (injected_failure()) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaSuccess) track(*p, bytes, false);
-    else *p = nullptr;
+    settle(e, p, bytes, false);
     return e;
 }
 
@@ -91,8 +101,7 @@ cudaError_t host_malloc(void **p, size_t bytes)
     *p = nullptr;
     if (injected_failure()) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaMallocHost(p, bytes);
-    if (e == cudaSuccess) track(*p, bytes, true);
-    else *p = nullptr;
+    settle(e, p, bytes, true);
     return e;
 }
 

@@ -83,43 +83,22 @@ impact_status tuning_of(const impact_tuning *t, Tuning &T)
 // ---------------------------------------------------------------------------
 
 
-impact_status make_batch(const impact_request *reqs, int count, impact_precision precision,
-                         const impact_tuning *tuning, Batch &B)
+// What the passes of the planned builds need: item and leaf table numbering,
+// shared memory.
+void size_batch(Batch &B)
 {
-    if (!reqs) return fail(IMPACT_ERR_ARG, "null request array");
-    if (count < 1 || count > kBatchMax)
-        return fail(IMPACT_ERR_ARG, "request count must be in [1, 65536]");
-    impact_status s = tuning_of(tuning, B.tune);
-    if (s != IMPACT_OK) return s;
-    B.plans.assign(count, Plan());
-    B.images.assign(count, nullptr);
-    B.row_begin.assign(count + 1, 0);
-    B.unit_begin.assign(count + 1, 0);
+    const int count = B.count();
     B.item_begin.assign((size_t)count * IMPACT_MAX_DIM + 1, 0);
     B.leaf_begin.assign(count + 1, 0);
-    B.prec = precision;
-    uint64_t h = 1469598103934665603ull;
+    B.rec_max = B.leaf_smem = B.shared32 = B.any64 = B.warp64 = 0;
+    for (int &w : B.work_max) w = 0;
     for (int q = 0; q < count; ++q) {
-        const impact_request &r = reqs[q];
-        s = impact::make_plan(r.sys, r.grid, r.inputs, r.sigma, r.cutoff, precision, B.plans[q]);
-        if (s != IMPACT_OK) {
-            if (count > 1) g_last_error = "request " + std::to_string(q) + ": " + g_last_error;
-            return s;
-        }
-        const Plan &P = B.plans[q];
-        B.images[q] = r.sys->dev_images;
-        B.row_begin[q + 1] = B.row_begin[q] + P.rows;
-        const int64_t rpw = 32 / P.desc.n;
-        B.unit_begin[q + 1] = B.unit_begin[q] + (P.rows + rpw - 1) / rpw;
-        B.nnz_bound = (B.nnz_bound > INT64_MAX - P.nnz_bound) ? INT64_MAX
-                                                              : B.nnz_bound + P.nnz_bound;
-        if (precision == IMPACT_FP32_SOUND) {
-            B.rec_max = std::max(B.rec_max, P.desc.rec_stride);
+        const ImpactDesc &D = B.plans[q].desc;
+        if (B.prec == IMPACT_FP32_SOUND) {
+            B.rec_max = std::max(B.rec_max, D.rec_stride);
             for (int mode = 0; mode < 3; ++mode)
-                B.work_max[mode] =
-                    std::max(B.work_max[mode], impact::walk_work_bytes(P.desc, mode));
+                B.work_max[mode] = std::max(B.work_max[mode], impact::walk_work_bytes(D, mode));
         }
-        const ImpactDesc &D = P.desc;
         for (int d = 0; d < IMPACT_MAX_DIM; ++d) {
             const size_t i = (size_t)q * IMPACT_MAX_DIM + d;
             int64_t units = 0;
@@ -136,11 +115,63 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
             ++B.any64;
             B.warp64 = std::max(B.warp64, (int)impact::walk64_bytes(D));
         }
+    }
+}
+
+// Less than this is not worth a second try at an allocation.
+constexpr int64_t kSpareMin = (int64_t)16 << 20;
+
+bool make_lean(Batch &B, int only)
+{
+    const int from = only < 0 ? 0 : only, to = only < 0 ? B.count() : only + 1;
+    int64_t spare = 0;
+    for (int q = from; q < to; ++q)
+        spare += B.plans[q].leaf_bytes + (B.plans[q].desc.walk64 ? B.plans[q].item_bytes : 0);
+    if (!B.walks || spare < kSpareMin) return false;
+    for (int q = from; q < to; ++q) {
+        Plan &P = B.plans[q];
+        if (P.desc.walk64) P.item_bytes = 0;
+        P.leaf_bytes = 0;
+        P.desc.walk64 = P.desc.leaf_shared = P.desc.lists = 0;
+    }
+    size_batch(B);
+    return true;
+}
+
+impact_status make_batch(const impact_request *reqs, int count, impact_precision precision,
+                         const impact_tuning *tuning, Batch &B)
+{
+    if (!reqs) return fail(IMPACT_ERR_ARG, "null request array");
+    if (count < 1 || count > kBatchMax)
+        return fail(IMPACT_ERR_ARG, "request count must be in [1, 65536]");
+    impact_status s = tuning_of(tuning, B.tune);
+    if (s != IMPACT_OK) return s;
+    B.plans.assign(count, Plan());
+    B.images.assign(count, nullptr);
+    B.row_begin.assign(count + 1, 0);
+    B.unit_begin.assign(count + 1, 0);
+    B.prec = precision;
+    uint64_t h = 1469598103934665603ull;
+    for (int q = 0; q < count; ++q) {
+        const impact_request &r = reqs[q];
+        s = impact::make_plan(r.sys, r.grid, r.inputs, r.sigma, r.cutoff, precision, B.plans[q]);
+        if (s != IMPACT_OK) {
+            if (count > 1) g_last_error = "request " + std::to_string(q) + ": " + g_last_error;
+            return s;
+        }
+        const Plan &P = B.plans[q];
+        B.images[q] = r.sys->dev_images;
+        B.row_begin[q + 1] = B.row_begin[q] + P.rows;
+        const int64_t rpw = 32 / P.desc.n;
+        B.unit_begin[q + 1] = B.unit_begin[q] + (P.rows + rpw - 1) / rpw;
+        B.nnz_bound = (B.nnz_bound > INT64_MAX - P.nnz_bound) ? INT64_MAX
+                                                              : B.nnz_bound + P.nnz_bound;
         h = mix(h, P.hash);
     }
     B.rows = B.row_begin[count];
     B.units = B.unit_begin[count];
     B.hash = h;   // launch shapes change no result: they are not part of the identity
+    size_batch(B);
     if (precision == IMPACT_FP32_SOUND &&
         2 * (int64_t)B.rec_max + B.work_max[WALK_FUSED] > IMPACT_WALK_SMEM_MAX)
         return fail(IMPACT_ERR_ARG,
@@ -218,7 +249,7 @@ bool ws_has(const void *ws, uint64_t h)
     return it != g_ws_tag.end() && it->second == h;
 }
 
-impact_status get_work(const Batch &B, const impact_csr *out, cudaStream_t st, Work &W)
+impact_status get_work(Batch &B, const impact_csr *out, cudaStream_t st, Work &W)
 {
     W.L = batch_layout(B);
     if (out && out->workspace) {
@@ -232,7 +263,14 @@ impact_status get_work(const Batch &B, const impact_csr *out, cudaStream_t st, W
         W.owned = false;
         return IMPACT_OK;
     }
-    CK(dev_malloc_async(&W.base, W.L.total, st));
+    cudaError_t e = dev_malloc_async(&W.base, W.L.total, st);
+    if (e == cudaErrorMemoryAllocation && make_lean(B)) {
+        W.L = batch_layout(B);
+        e = dev_malloc_async(&W.base, W.L.total, st);
+    }
+    if (e != cudaSuccess)
+        return fail(e == cudaErrorMemoryAllocation ? IMPACT_ERR_OOM : IMPACT_ERR_CUDA,
+                    std::string("workspace: ") + cudaGetErrorString(e));
     W.owned = true;
     return IMPACT_OK;
 }
@@ -538,7 +576,7 @@ struct Outcome {
     int64_t nnz = 0;
 };
 
-impact_status do_count(const Batch &B, impact_csr *out, cudaStream_t st)
+impact_status do_count(Batch &B, impact_csr *out, cudaStream_t st)
 {
     impact_status s;
     if ((s = check_row_arrays(out)) != IMPACT_OK) return s;
@@ -560,7 +598,7 @@ impact_status do_count(const Batch &B, impact_csr *out, cudaStream_t st)
     return s;
 }
 
-impact_status do_emit(const Batch &B, impact_csr *out, cudaStream_t st)
+impact_status do_emit(Batch &B, impact_csr *out, cudaStream_t st)
 {
     impact_status s;
     if (!is_device_ptr(out->row_ptr)) return fail(IMPACT_ERR_ARG, "row_ptr must be a device array");
@@ -590,7 +628,7 @@ impact_status do_emit(const Batch &B, impact_csr *out, cudaStream_t st)
     return status_result(status);
 }
 
-impact_status build_into(const Batch &B, impact_csr *out, bool lib_owned, cudaStream_t st)
+impact_status build_into(Batch &B, impact_csr *out, bool lib_owned, cudaStream_t st)
 {
     impact_status s;
     const size_t vbytes = B.prec == PREC_FP32_SOUND ? 4 : 8;
@@ -637,7 +675,7 @@ impact_status build_into(const Batch &B, impact_csr *out, bool lib_owned, cudaSt
     return status_result(r.status);
 }
 
-impact_status do_build(const Batch &B, impact_csr *out, cudaStream_t st)
+impact_status do_build(Batch &B, impact_csr *out, cudaStream_t st)
 {
     configure_pool_once();
     const bool lib_owned = (out->col == nullptr);
@@ -929,6 +967,10 @@ impact_status impact_graph_create(const impact_request *reqs, int count,
         ws_tag(W.base, 0);
     } else {
         cudaError_t e = dev_malloc(&g->own_ws, W.L.total);
+        if (e == cudaErrorMemoryAllocation && make_lean(B)) {
+            W.L = batch_layout(B);
+            e = dev_malloc(&g->own_ws, W.L.total);
+        }
         if (e != cudaSuccess) return cleanup(fail(IMPACT_ERR_OOM, cudaGetErrorString(e)));
         W.base = g->own_ws;
     }

@@ -169,7 +169,7 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
 // per row in `acc`, [3][rows of the batch]), then the per-row terms. The
 // planner calls size_items64 (item layout and whether the build takes this
 // path: ImpactDesc.walk64; returns the bytes of the build's items).
-int64_t size_items64(ImpactDesc &D, int64_t nnz_bound);
+int64_t size_items64(ImpactDesc &D);
 int64_t walk64_bytes(const ImpactDesc &D);   // shared memory of one warp
 cudaError_t launch_items64(const BatchIndex *d_index, int64_t units, uint32_t *status,
                            cudaStream_t stream);

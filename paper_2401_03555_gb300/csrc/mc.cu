@@ -22,7 +22,7 @@ namespace impact {
 impact_status fail(impact_status s, const std::string &msg);
 impact_request single(const impact_system *sys, const impact_grid *grid,
                       const impact_inputs *inputs, const double *sigma, double cutoff);
-impact_status get_work(const Batch &B, const impact_csr *out, cudaStream_t st, Work &W);
+impact_status get_work(Batch &B, const impact_csr *out, cudaStream_t st, Work &W);
 impact_status release(Work &W, cudaStream_t st);
 bool is_device_ptr(const void *p);
 impact_status check_row_arrays(const impact_csr *out);

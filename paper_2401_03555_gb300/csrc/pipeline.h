@@ -37,6 +37,12 @@ struct Batch {
 impact_status make_batch(const impact_request *reqs, int count, impact_precision precision,
                          const impact_tuning *tuning, Batch &B);
 
+// Plans the builds `only` (or all, < 0) again without the tables that only save
+// time, FP64 items and FP32 leaf tables: the per-pair kernel and per-row tables
+// take their place, as at sizes beyond them (the same pairs; the FP64 truncated
+// mass is summed in another order). False: too little to give up.
+bool make_lean(Batch &B, int only = -1);
+
 // Offsets (bytes, 256-aligned) of everything in the device workspace.
 struct BatchLayout {
     size_t index = 0, row_begin = 0, unit_begin = 0, descs = 0, recs = 0, item_begin = 0;

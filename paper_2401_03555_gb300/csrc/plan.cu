@@ -505,7 +505,7 @@ impact_status make_plan(const impact_system *sys, const impact_grid *grid,
     }
     number_items(sys, inputs, P);
     if (precision == IMPACT_FP32_SOUND) impact::size_items32(D, P.item_bytes, P.leaf_bytes);
-    if (precision == IMPACT_FP64_PLAIN) P.item_bytes = impact::size_items64(D, P.nnz_bound);
+    if (precision == IMPACT_FP64_PLAIN) P.item_bytes = impact::size_items64(D);
     // identity of the arguments, for reusing a caller's workspace
     uint64_t h = 1469598103934665603ull;
     int hdr[5] = {sys->kind, n, m, (int)precision, n_inputs};

@@ -61,6 +61,7 @@ struct Request {
     std::string error;
     struct Group *group = nullptr;
     int index = 0;             // position in its group
+    bool lean = false;         // built without the tables that only save time (pipeline.h)
     int64_t nnz = 0;
     bool released = false;
 
@@ -209,6 +210,8 @@ void impact_server::admit()
         groups.push_back(g);
     };
     if (s != IMPACT_OK) return bail(s, impact_last_error());
+    for (size_t q = 0; q < take.size(); ++q)
+        if (take[q]->lean) impact::make_lean(g->B, (int)q);
     // small groups go to the high-priority stream, large ones take turns on
     // the others and run in chunks of rows, so that the SMs a large group
     // frees between its chunks go to the small groups first
@@ -223,9 +226,13 @@ void impact_server::admit()
     cudaStream_t st = g->stream;
     g->rows = g->B.rows;
     g->W.L = impact::batch_layout(g->B);
-    g->ws_bytes = align_up((int64_t)g->W.L.total);
     g->row_bytes = align_up(row_bytes_of(g->rows));
     cudaError_t e = impact::dev_malloc_async(&g->W.base, g->W.L.total, st);
+    if (e == cudaErrorMemoryAllocation && impact::make_lean(g->B)) {
+        g->W.L = impact::batch_layout(g->B);
+        e = impact::dev_malloc_async(&g->W.base, g->W.L.total, st);
+    }
+    g->ws_bytes = align_up((int64_t)g->W.L.total);
     if (e == cudaSuccess) e = impact::dev_malloc_async(&g->row_ptr, (g->rows + 1) * 8, st);
     if (e == cudaSuccess) e = impact::dev_malloc_async(&g->sink_lo, g->rows * 8, st);
     if (e == cudaSuccess) e = impact::dev_malloc_async(&g->sink_up, g->rows * 8, st);
@@ -478,8 +485,14 @@ impact_status impact_server_submit(impact_server *S, const impact_request *reque
     r->sigma = copy(q.sigma, n);
     r->cutoff = q.cutoff;
     r->rows = B.rows;
-    r->admit_bytes = align_up((int64_t)impact::batch_layout(B).total) +
-                     align_up(row_bytes_of(B.rows));
+    auto need = [&] {
+        return align_up((int64_t)impact::batch_layout(B).total) + align_up(row_bytes_of(B.rows));
+    };
+    r->admit_bytes = need();
+    if (r->admit_bytes > S->budget && impact::make_lean(B)) {   // does it fit without its tables?
+        r->lean = true;
+        r->admit_bytes = need();
+    }
     r->t_submit = Clock::now();
     {
         std::lock_guard<std::mutex> lock(S->mu);

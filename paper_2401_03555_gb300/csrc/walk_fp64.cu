@@ -51,6 +51,7 @@ constexpr int kSortMax = 256;         // widest last-dimension window that is so
 constexpr int kTablesMax = 2048;      // widest window box (targets, all dimensions)
 constexpr int kWarps = 8;             // warps per block at most
 constexpr int kSmemWarp = 64 * 1024;  // shared memory of one warp at most
+constexpr int64_t kItemsMax = (int64_t)1 << 30;   // item tables of one build at most
 
 // One item: the header, the window's (U, L) pairs and, in the last dimension
 // of a build with a cutoff, five sorted arrays of w64 + 1 doubles (su, sl, pu,
@@ -836,7 +837,7 @@ int blocks_for(const void *kernel, int threads, size_t smem, int64_t items, int 
 
 namespace impact {
 
-int64_t size_items64(ImpactDesc &D, int64_t nnz_bound)
+int64_t size_items64(ImpactDesc &D)
 {
     const int n = D.n;
     int64_t bytes = 0, tsum = 0;
@@ -850,12 +851,10 @@ int64_t size_items64(ImpactDesc &D, int64_t nnz_bound)
         g.item_off = bytes;
         bytes += g.n_items * (int64_t)g.item_stride;
     }
-    // a window box too wide for a warp's shared memory, or tables out of
-    // proportion to the output (one wide dimension of distinct images), keep
-    // the per-pair evaluation
-    D.walk64 = tsum <= kTablesMax && walk64_bytes(D) <= kSmemWarp &&
-               bytes <= std::max<int64_t>((int64_t)1 << 30,
-                                          nnz_bound > INT64_MAX / 4 ? INT64_MAX : nnz_bound * 5 / 2);
+    // a window box too wide for a warp's shared memory, or tables beyond a fixed
+    // size (images that are nearly all distinct, on large grids), keep the
+    // per-pair evaluation, which needs no scratch
+    D.walk64 = tsum <= kTablesMax && walk64_bytes(D) <= kSmemWarp && bytes <= kItemsMax;
     return D.walk64 ? bytes : 0;
 }
 

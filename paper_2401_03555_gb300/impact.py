@@ -374,7 +374,10 @@ def build(prob, precision="fp32", stream=None, check_unsound: bool = True) -> CS
     _check(lib.impact_workspace_bytes(ctypes.byref(a.sys), ctypes.byref(a.grid),
                                       ctypes.byref(a.inp), a.sigma_ptr, a.cutoff, prec,
                                       ctypes.byref(wb)))
-    ws = torch.empty(max(wb.value, 256), dtype=torch.uint8, device="cuda")
+    try:
+        ws = torch.empty(max(wb.value, 256), dtype=torch.uint8, device="cuda")
+    except torch.OutOfMemoryError:
+        ws = None   # the library's own scratch, which can do with less
     c = _csr_struct(rb, workspace=ws)
     st = _stream_handle(stream)
     status = lib.impact_count(ctypes.byref(a.sys), ctypes.byref(a.grid), ctypes.byref(a.inp),
