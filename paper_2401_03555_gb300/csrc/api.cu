@@ -118,9 +118,6 @@ void size_batch(Batch &B)
     }
 }
 
-// Less than this is not worth a second try at an allocation.
-constexpr int64_t kSpareMin = (int64_t)16 << 20;
-
 bool make_lean(Batch &B, int only)
 {
     const int from = only < 0 ? 0 : only, to = only < 0 ? B.count() : only + 1;
@@ -1182,14 +1179,19 @@ impact_status impact_region_vectors(const impact_system *sys, const impact_grid 
     batch.extra = region_scratch(batch.plans[0].desc, B);
     Work W;
     s = get_work(batch, nullptr, st, W);
+    if (s == IMPACT_ERR_OOM && batch.extra >= kSpareMin) {
+        batch.extra = 0;
+        s = get_work(batch, nullptr, st, W);
+    }
     if (s != IMPACT_OK) return s;
     WorkHold hold{W, st};
     s = upload(batch, W, st);
     if (s == IMPACT_OK) {
         cudaError_t e = launch_regions(batch.plans[0].desc, W.desc(0), batch.rows, B,
                                        mode == IMPACT_REGION_CELL_SUM,
-                                       precision == IMPACT_FP32_SOUND, W.base + W.L.extra, r_lo,
-                                       r_up, a_lo, a_up, st);
+                                       precision == IMPACT_FP32_SOUND,
+                                       batch.extra > 0 ? W.base + W.L.extra : nullptr, r_lo, r_up,
+                                       a_lo, a_up, st);
         if (e != cudaSuccess) s = fail(IMPACT_ERR_CUDA, cudaGetErrorString(e));
     }
     impact_status r = release(W, st);

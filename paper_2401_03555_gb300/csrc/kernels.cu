@@ -999,12 +999,16 @@ cudaError_t launch_labels(const RegionBoxes &boxes, int64_t total_cells, uint8_t
 // Items only where rows share them: below two rows per item the table's
 // write and read back cost about what they save. FP64 erfc per row, dimension
 // and cell bounded the per-row kernel: the 11^5 room's cell sums (1.45M rows,
-// 22k items) took 50.7 ms and take 0.32 ms.
+// 22k items) took 50.7 ms and take 0.32 ms. Tables beyond a fixed size (it holds
+// a million items of 16 boxes) are not made either: the rows need no scratch.
+constexpr int64_t kRegionItemsMax = (int64_t)256 << 20;
+
 int64_t region_scratch(const ImpactDesc &D, const RegionBoxes &boxes)
 {
     int64_t items = 0;
     for (int d = 0; d < D.n; ++d) items += D.dim[d].n_items;
-    return items <= D.rows * D.n / 2 ? items * (boxes.count + 1) * (int64_t)sizeof(double2) : 0;
+    const int64_t bytes = items * (boxes.count + 1) * (int64_t)sizeof(double2);
+    return items <= D.rows * D.n / 2 && bytes <= kRegionItemsMax ? bytes : 0;
 }
 
 cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_t rows,
@@ -1013,7 +1017,7 @@ cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_
                            cudaStream_t stream)
 {
     if (rows <= 0) return cudaSuccess;
-    if (region_scratch(D, boxes) > 0) {
+    if (scratch) {
         RegionItems I;
         I.first[0] = 0;
         for (int d = 0; d < D.n; ++d) I.first[d + 1] = I.first[d] + D.dim[d].n_items;

@@ -115,7 +115,8 @@ cudaError_t launch_labels(const RegionBoxes &boxes, int64_t total_cells, uint8_t
 // Region vectors of rows [0, rows) of the build described by D (FP64 tables):
 // cell_sum selects the paper's sums of per-cell bounds, else one relaxation
 // per box; sound selects the enclosing evaluation. scratch: device memory of
-// region_scratch bytes (0: rows are evaluated one by one).
+// region_scratch bytes, or null (it is 0, or cannot be had): rows are evaluated
+// one by one.
 int64_t region_scratch(const ImpactDesc &D, const RegionBoxes &boxes);
 cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_t rows,
                            const RegionBoxes &boxes, bool cell_sum, bool sound, void *scratch,

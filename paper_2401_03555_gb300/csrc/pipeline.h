@@ -42,6 +42,8 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
 // take their place, as at sizes beyond them (the same pairs; the FP64 truncated
 // mass is summed in another order). False: too little to give up.
 bool make_lean(Batch &B, int only = -1);
+// Scratch that a call can do without and whose lack is worth a second try.
+constexpr int64_t kSpareMin = (int64_t)16 << 20;
 
 // Offsets (bytes, 256-aligned) of everything in the device workspace.
 struct BatchLayout {

@@ -122,3 +122,24 @@ def test_images_beyond_the_item_tables_match_the_oracle():
     orc = oracle.default()
     rows = W.sample_rows(prob, 200, seed=2)
     PA.compare(prob, csr, orc.build_rows(prob, rows), orc, "fp64").assert_ok()
+
+
+@pytest.mark.parametrize("mode", ["box", "cells"])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_region_vectors_without_tables_have_the_same_bits(mode, precision):
+    """200 x 200 x 2 cells, 4 inputs: 320,000 images of two coordinates, whose
+    factors of the domain and 3 boxes take 20 MB."""
+    prob = W.Problem(name="regions", kind=W.AFFINE, lo=np.full(3, -1.0), hi=np.full(3, 1.0),
+                     cells=np.array([200, 200, 2], np.int32),
+                     inputs=np.linspace(-0.5, 0.5, 4)[:, None], sigma=np.array([0.02, 0.02, 0.5]),
+                     cutoff=1e-8, A=np.array([[0.9, 0.05, 0], [-0.03, 0.8, 0], [0, 0, 0.7]]),
+                     B=np.array([[0.2], [0.1], [0.3]]), c=np.zeros(3))
+
+    def vectors(boxes):
+        r = impact.region_vectors(prob, target=boxes[:1], avoid=boxes[1:], mode=mode,
+                                  precision=precision)
+        return [r.r_lo, r.r_up, r.a_lo, r.a_up]
+
+    boxes = [([-1.0 + 0.4 * i, -0.9, -1.0], [-0.8 + 0.4 * i, 0.3, 1.0]) for i in range(3)]
+    ref = vectors(boxes)
+    assert all(torch.equal(a, b) for a, b in zip(without_tables(lambda: vectors(boxes)), ref))
