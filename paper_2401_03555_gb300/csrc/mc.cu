@@ -70,11 +70,14 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     impact_status s = make_batch(&req, 1, IMPACT_FP64_PLAIN, nullptr, B);
     if (s != IMPACT_OK) return s;
     B.walks = false;
-    const McMasks masks = mc_masks(B.plans[0].desc, n_samples, cutoff);
+    McMasks masks = mc_masks(B.plans[0].desc, n_samples, cutoff);
     // the masks, the entries a count keeps for the emit, a segment per row
-    const int64_t keep_cap = masks.bytes > 0 ? mc_keep_entries(B.rows) : 0;
+    int64_t keep_cap = masks.bytes > 0 ? mc_keep_entries(B.rows) : 0;
     const int64_t mask_end = (masks.bytes + 255) / 256 * 256;
-    if (masks.bytes > 0) B.extra = mask_end + 8 * keep_cap + 8 * B.rows;
+    auto size_extra = [&] {
+        B.extra = masks.bytes > 0 ? mask_end + 8 * keep_cap + 8 * B.rows : 0;
+    };
+    size_extra();
     B.plans[0].desc.cutoff = cutoff;
     B.plans[0].desc.prec = precision;
     configure_pool_once();
@@ -103,7 +106,18 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
     Work W;
     impact_csr no_ws = *out;
     no_ws.workspace = nullptr;
-    if ((s = get_work(B, &no_ws, st, W)) != IMPACT_OK) return give_back(s);
+    s = get_work(B, &no_ws, st, W);
+    if (s == IMPACT_ERR_OOM && 8 * keep_cap >= kSpareMin) {   // the emit walks every row again
+        keep_cap = 0;
+        size_extra();
+        s = get_work(B, &no_ws, st, W);
+    }
+    if (s == IMPACT_ERR_OOM && masks.bytes >= kSpareMin) {    // the per-row histogram
+        masks.bytes = 0;
+        size_extra();
+        s = get_work(B, &no_ws, st, W);
+    }
+    if (s != IMPACT_OK) return give_back(s);
     // per-call tables: draw keys [n][S], range [n][2], values u / S for
     // u = 0..S (FP64, FP32 down, FP32 up), the non-finite flag
     const int64_t S = n_samples;

@@ -143,3 +143,28 @@ def test_region_vectors_without_tables_have_the_same_bits(mode, precision):
     boxes = [([-1.0 + 0.4 * i, -0.9, -1.0], [-0.8 + 0.4 * i, 0.3, 1.0]) for i in range(3)]
     ref = vectors(boxes)
     assert all(torch.equal(a, b) for a, b in zip(without_tables(lambda: vectors(boxes)), ref))
+
+
+# room for the kept entries refused (286 MB): every row is walked again; the masks
+# refused (25 MB, fewer entries): the per-row histograms
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("name,draws", [("room", 300), ("cube", 2100)])
+def test_sampled_noise_without_its_scratch_has_the_same_bits(name, draws, precision):
+    if name == "room":
+        prob = W.room_5d(cells_per_dim=6)
+    else:
+        prob = W.Problem(name="cube", kind=W.AFFINE, lo=np.full(4, -1.0), hi=np.full(4, 1.0),
+                         cells=np.array([8, 8, 8, 7], np.int32), inputs=np.zeros((1, 1)),
+                         sigma=np.full(4, 0.1), cutoff=1e-3, A=0.9 * np.eye(4) + 0.05 *
+                         (np.ones((4, 4)) - np.eye(4) - np.roll(np.eye(4), 1, axis=1)),
+                         B=np.zeros((4, 1)), c=np.zeros(4))
+    w = np.random.default_rng(draws).normal(size=(draws, prob.n)) * np.asarray(prob.sigma)
+    ref = impact.build_mc(prob, w, precision, cutoff=4e-3)
+    impact.fail_alloc(6)   # the five row arrays, then the scratch
+    try:
+        got = impact.build_mc(prob, w, precision, cutoff=4e-3)
+    finally:
+        impact.fail_alloc(0)
+    assert ref.nnz > prob.rows
+    for f in ("row_ptr", "col", "lo", "up", "sink_lo", "sink_up", "trunc", "row_flags"):
+        assert torch.equal(getattr(got, f), getattr(ref, f)), f
