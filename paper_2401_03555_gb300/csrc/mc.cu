@@ -214,5 +214,5 @@ extern "C" impact_status impact_build_mc(const impact_system *sys, const impact_
         return done(fail(IMPACT_ERR_CUDA, "emit pass failed"));
     if (status & IMPACT_STATUS_CAPACITY)
         return done(fail(IMPACT_ERR_CAPACITY, "output capacity too small"));
-    return done(IMPACT_OK);
+    return done(status_result(status));   // a row written otherwise than it was counted
 }
