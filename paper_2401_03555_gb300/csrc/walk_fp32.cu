@@ -1661,14 +1661,16 @@ __device__ __forceinline__ void leaf_emit_wide(const WarpMem &S, int n, const Le
 // the leaves under every chunk of the deepest list. LEFT lists are still to
 // come; the recursion is unrolled at compile time (a loop with the level as a
 // variable spends more on finding its place than on the nodes: the 8^5 room's
-// count pass took 1251 instructions a row, and takes 861), and every loop runs
-// over a list's candidates once, so it ends.
+// count pass took 1251 instructions a row, and takes 861). Every chunk takes at
+// least one of a list's candidates, whatever the record says, so every loop
+// ends; counting the steps as the emit does cost the 7-D building's count 2.80 ->
+// 3.04 ms, and its records were made in the same call.
 template <int LEFT, bool ROOT>
 __device__ __forceinline__ void count_levels(const WarpMem &S, int n, const Leaf &f, int npar,
                                              int lane, CountAcc &acc, float cut)
 {
     const int k = n - 2 - LEFT;
-    const int total = npar * S.h[k].tw, chunk = chunk_of(S.h[k]);
+    const int total = npar * S.h[k].tw, chunk = max(chunk_of(S.h[k]), 1);
 #pragma unroll 1
     for (int c0 = 0; c0 < total; c0 += chunk) {
         const int nout = expand<true>(S, k, ROOT, c0, min(c0 + chunk, total), lane, acc);
@@ -1702,15 +1704,20 @@ __device__ __forceinline__ void count_row(const WarpMem &S, int n, const Leaf &f
 // level as a variable (the unrolled recursion keeps every level's loop state
 // live, and the emit's inner loop needs the registers: 64 let 8 warps per
 // scheduler hide its shared-memory latency; unrolled, the 11^5 room's emit
-// pass took 7.8 ms against 7.45). Every step fills a list, runs the leaves of one
-// or leaves one whose candidates are used up, so the loop ends.
-__device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f, bool lists,
+// pass took 7.8 ms against 7.45). Every turn of the loop fills a list, runs the
+// leaves of one or leaves one whose candidates are used up, and takes one of the
+// row's `steps`. A record bounds its lists, so a sound one never runs out
+// (ImpactDesc.walk_steps); one that was overwritten since the setup (a caller's
+// workspace between count and emit) could hold a chunk of no candidates, and a
+// walk without end. False: the steps ran out.
+__device__ __forceinline__ bool emit_row(const WarpMem &S, int n, const Leaf &f, bool lists,
                                          int after, int lane, const EmitOut &out, int &written,
-                                         float cut)
+                                         float cut, unsigned steps)
 {
     if (n <= 2) {
+        if (steps == 0) return false;
         leaf_emit_wide(S, n, f, NodeList{}, true, 1, lane, out, written, cut);
-        return;
+        return true;
     }
     const EmitLeaf g = emit_leaf(S, f);
     if (g.staged && !lists)
@@ -1724,7 +1731,7 @@ __device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f,
     int my_cur = 0, my_sz = 0;   // lane k: next candidate of level k, size of list k
     CountAcc none;
     int k = 0;
-    while (true) {
+    for (; steps > 0; --steps) {
         if (k == last + 1) {
             const NodeList L = node_list(S.work, last);
             const int npar = __shfl_sync(0xffffffffu, my_sz, last);
@@ -1739,7 +1746,7 @@ __device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f,
         const int cur = __shfl_sync(0xffffffffu, my_cur, k);
         const int total = npar * S.h[k].tw;
         if (cur >= total) {
-            if (k == 0) break;
+            if (k == 0) return true;
             --k;
             continue;
         }
@@ -1752,6 +1759,7 @@ __device__ __forceinline__ void emit_row(const WarpMem &S, int n, const Leaf &f,
         if (lane == k + 1) my_cur = 0;
         ++k;
     }
+    return false;
 }
 
 // ---------------------------------------------------------------------------
@@ -1964,7 +1972,9 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
         const WarpMem S = carve(work, rec, n, D.leaf_cap);
         const bool empty = __any_sync(0xffffffffu, lane < n && S.h[lane].tw == 0);
         Leaf f = leaf_of(S, n);
-        bool walked = row != A.guard_row;   // fault injection: a broken walk
+        // fault injection: a row whose steps are spent before the first
+        const unsigned steps = row == A.guard_row ? 0u : D.walk_steps;
+        bool walked = MODE == MODE_EMIT || steps > 0;   // a count has none to run out of
         bool lb_ok = true;
         int64_t base = 0, len = 0;
         if (kCount) {
@@ -2053,9 +2063,10 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
                         cp_async_wait_all();
                         __syncwarp();
                     }
-                    emit_row(S, n, f, lists, after, lane, out, written, cut);
+                    walked = emit_row(S, n, f, lists, after, lane, out, written, cut, steps);
                 }
-                if (lane == 0 && written != len) atomicOr(A.status, IMPACT_STATUS_EMIT_MISMATCH);
+                if (lane == 0 && walked && written != len)
+                    atomicOr(A.status, IMPACT_STATUS_EMIT_MISMATCH);
             }
         }
         if (lane == 0 && !walked) atomicOr(A.status, IMPACT_STATUS_INTERNAL);
@@ -2147,6 +2158,16 @@ void size_items32(ImpactDesc &D, int64_t &item_bytes, int64_t &leaf_bytes)
                     D.leaf_items * D.leaf_stride <= D.rows * (int64_t)D.rec_stride;
     D.lists = D.leaf_shared && lists;
     leaf_bytes = D.leaf_shared ? D.leaf_items * D.leaf_stride : 0;
+    // The walk's guard: steps of a row whose windows are all as wide as they may
+    // be. A chunk but a list's last has 33 candidates or more and fills one list of
+    // the next level, so level k has at most 1 + (k + 1) prod / 33 chunks, prod its
+    // candidates; each is filled, walked and left. Twice that and more.
+    int64_t steps = 16, prod = 1;
+    for (int k = 0; k + 2 < n; ++k) {
+        prod = std::min(prod * D.dim[k].wcap, (int64_t)1 << 31);
+        steps += 8 * (int64_t)(k + 1) * (1 + prod / 32);
+    }
+    D.walk_steps = (uint32_t)std::min<int64_t>(steps, UINT32_MAX);
 }
 
 int leaf32_bytes(const ImpactDesc &D)
