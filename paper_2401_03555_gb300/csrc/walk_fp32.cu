@@ -1700,7 +1700,8 @@ __device__ __forceinline__ void count_row(const WarpMem &S, int n, const Leaf &f
     }
 }
 
-// Writes the pairs of one row whose record is in S: the same lists, with the
+// Writes the pairs of one row whose record is in S, or (COUNT: the one-pass walk,
+// which does both) counts them: the same lists, with the
 // level as a variable (the unrolled recursion keeps every level's loop state
 // live, and the emit's inner loop needs the registers: 64 let 8 warps per
 // scheduler hide its shared-memory latency; unrolled, the 11^5 room's emit
@@ -1710,17 +1711,19 @@ __device__ __forceinline__ void count_row(const WarpMem &S, int n, const Leaf &f
 // (ImpactDesc.walk_steps); one that was overwritten since the setup (a caller's
 // workspace between count and emit) could hold a chunk of no candidates, and a
 // walk without end. False: the steps ran out.
-__device__ __forceinline__ bool emit_row(const WarpMem &S, int n, const Leaf &f, bool lists,
-                                         int after, int lane, const EmitOut &out, int &written,
-                                         float cut, unsigned steps)
+template <bool COUNT>
+__device__ __forceinline__ bool walk_row(const WarpMem &S, int n, const Leaf &f, bool lists,
+                                         int after, int lane, CountAcc &acc, const EmitOut &out,
+                                         int &written, float cut, unsigned steps)
 {
     if (n <= 2) {
         if (steps == 0) return false;
-        leaf_emit_wide(S, n, f, NodeList{}, true, 1, lane, out, written, cut);
+        if (COUNT) leaf_count(S, n, f, NodeList{}, true, 1, lane, acc, cut);
+        else leaf_emit_wide(S, n, f, NodeList{}, true, 1, lane, out, written, cut);
         return true;
     }
     const EmitLeaf g = emit_leaf(S, f);
-    if (g.staged && !lists)
+    if (!COUNT && g.staged && !lists)
         for (int j = lane; j < f.nb; j += 32) {
             const LeafEntry e = leaf_eval(S, n, f, j);
             g.u[j] = e.u;
@@ -1729,14 +1732,14 @@ __device__ __forceinline__ bool emit_row(const WarpMem &S, int n, const Leaf &f,
         }
     const int last = n - 3;      // deepest list level
     int my_cur = 0, my_sz = 0;   // lane k: next candidate of level k, size of list k
-    CountAcc none;
     int k = 0;
     for (; steps > 0; --steps) {
         if (k == last + 1) {
             const NodeList L = node_list(S.work, last);
             const int npar = __shfl_sync(0xffffffffu, my_sz, last);
             unsigned char *const block = reinterpret_cast<unsigned char *>(S.leaf);
-            if (lists) emit_lists(block, block + after, f.nb, L, npar, lane, out, written, cut);
+            if (COUNT) leaf_count(S, n, f, L, false, npar, lane, acc, cut);
+            else if (lists) emit_lists(block, block + after, f.nb, L, npar, lane, out, written, cut);
             else if (g.staged) leaf_emit(S, g, L, npar, lane, out, written, cut);
             else leaf_emit_wide(S, n, f, L, false, npar, lane, out, written, cut);
             k = last;
@@ -1751,7 +1754,7 @@ __device__ __forceinline__ bool emit_row(const WarpMem &S, int n, const Leaf &f,
             continue;
         }
         const int end = min(cur + chunk_of(S.h[k]), total);
-        const int nout = expand<false>(S, k, k == 0, cur, end, lane, none);
+        const int nout = expand<COUNT>(S, k, k == 0, cur, end, lane, acc);
         if (lane == k) {
             my_cur = end;
             my_sz = nout;
@@ -1906,11 +1909,14 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
     // persistent: each warp takes rows from the batch's row counter,
     // A.row_block consecutive rows per atomic (one counter serves every warp
     // of the grid: claiming short rows one by one queues the atomics), in
-    // ascending order. The passes that count take
+    // ascending order. The count pass takes
     // rows one ahead: while a warp walks a row, the next row's record is copied
     // (cp.async) into the warp's other record buffer. The emit pass (more
-    // registers live in its walk) copies each record when it starts it.
-    constexpr bool kAhead = MODE != MODE_EMIT;
+    // registers live in its walk) copies each record when it starts it. So does the
+    // one-pass walk, one row at a time: a row taken and not yet counted holds up
+    // every row after it while its warp waits for the rows before the one it is at
+    // (a row ahead: the 11^5 room 85 ms, the unicycle 139; none: 14.5 and 22.5).
+    constexpr bool kAhead = MODE == MODE_COUNT;
     const int64_t row_end = A.row_end;
     unsigned char *const work = wbase + (kAhead ? 2 : 1) * A.rec_max;
     // the claimed rows [claim[0], claim[1]) stand in the last bytes of the
@@ -1974,7 +1980,7 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
         Leaf f = leaf_of(S, n);
         // fault injection: a row whose steps are spent before the first
         const unsigned steps = row == A.guard_row ? 0u : D.walk_steps;
-        bool walked = MODE == MODE_EMIT || steps > 0;   // a count has none to run out of
+        bool walked = MODE != MODE_COUNT || steps > 0;   // that count has none to run out of
         bool lb_ok = true;
         int64_t base = 0, len = 0;
         if (kCount) {
@@ -1995,7 +2001,13 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
                     }
                 }
                 if (!f.shared) leaf_build(S, n, f, lane, cut);
-                count_row(S, n, f, lane, acc, cut);
+                if (MODE == MODE_FUSED) {
+                    int none = 0;
+                    walked = walk_row<true>(S, n, f, false, 0, lane, acc, EmitOut{}, none, cut, steps);
+                    if (!walked) acc = CountAcc();
+                } else {
+                    count_row(S, n, f, lane, acc, cut);
+                }
             }
             const int c = __reduce_add_sync(0xffffffffu, acc.cnt);
             const float drop = warp_sum_ru(acc.drop);
@@ -2063,7 +2075,9 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
                         cp_async_wait_all();
                         __syncwarp();
                     }
-                    walked = emit_row(S, n, f, lists, after, lane, out, written, cut, steps);
+                    CountAcc none;
+                    walked = walk_row<false>(S, n, f, lists, after, lane, none, out, written, cut,
+                                             steps);
                 }
                 if (lane == 0 && walked && written != len)
                     atomicOr(A.status, IMPACT_STATUS_EMIT_MISMATCH);
@@ -2232,7 +2246,7 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
     // multiples of 16)
     rec_max = (rec_max + 15) & ~15;
     const int work = work_max[mode];
-    const int warp_smem = (mode == MODE_EMIT ? 1 : 2) * rec_max + ((work + 15) & ~15) + kClaimBytes;
+    const int warp_smem = (mode == MODE_COUNT ? 2 : 1) * rec_max + ((work + 15) & ~15) + kClaimBytes;
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -2270,11 +2284,12 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
     // persistent grid: as many blocks as fit at once (rows are taken dynamically)
     const int g = occupancy_grid(k, threads, smem, rows, warps);
     // rows per claim: 4 in the count pass (its rows are short: the atomics
-    // cost more than the last claims' imbalance), else up to 4 while that
+    // cost more than the last claims' imbalance), in the emit up to 4 while that
     // imbalance (up to 3 rows per warp) stays under 1/256 of each warp's rows
-    A.row_block = mode == MODE_COUNT
-                      ? 4
-                      : (int)std::max<int64_t>(1, std::min<int64_t>(4, rows / ((int64_t)g * warps * 256)));
+    A.row_block = mode == MODE_COUNT   ? 4
+                  : mode == MODE_FUSED ? 1
+                      : (int)std::max<int64_t>(
+                            1, std::min<int64_t>(4, rows / ((int64_t)g * warps * 256)));
     if (mode == MODE_COUNT)
         walk_fp32<MODE_COUNT><<<g, threads, smem, stream>>>(A);
     else if (mode == MODE_EMIT)
