@@ -129,3 +129,29 @@ def test_windows_by_lane_groups_equal_those_by_lanes(cells):
         one, part = impact.build(p, "fp32"), batch.part(q)
         for k in ("row_ptr", "col", "lo", "up", "sink_lo", "sink_up", "trunc", "row_flags"):
             assert torch.equal(getattr(one, k), getattr(part, k)), (q, k)
+
+
+@pytest.mark.parametrize("cells,sigma", [([12, 11, 10], 0.3), ([12, 11, 10], 0.6), ([7, 8, 9], 4.0),
+                                         ([16, 17], 5.0), ([3, 31, 10], 1.1)])
+def test_shared_windows_by_lane_groups_equal_those_by_lanes(cells, sigma):
+    """A build of few distinct images makes its shared windows by eight lanes each, one
+    of more than 12,288 by single lanes: the same inputs among many others have
+    the same rows, bitwise. Widths below, at and beyond the group."""
+    n, few = len(cells), 8
+    many = few + 12289 // sum(cells) + 1
+    U = np.random.default_rng(3).uniform(-0.5, 0.5, (many, 1))
+    B = np.full((n, 1), 0.3)
+    small = linear(cells, np.eye(n) * 0.9, [sigma] * n, 1e-9, U[:few], B=B)
+    large = linear(cells, np.eye(n) * 0.9, [sigma] * n, 1e-9, U, B=B)
+    a, b = impact.build(small, "fp32"), impact.build(large, "fp32")
+    total = small.total_cells
+    rows = (torch.arange(total, device="cuda")[:, None] * many
+            + torch.arange(few, device="cuda")[None]).flatten()
+    for k in ("sink_lo", "sink_up", "trunc", "row_flags"):
+        assert torch.equal(getattr(a, k), getattr(b, k)[rows]), k
+    len_a = a.row_ptr[1:] - a.row_ptr[:-1]
+    assert torch.equal(len_a, b.row_ptr[rows + 1] - b.row_ptr[rows])
+    at = torch.repeat_interleave(b.row_ptr[rows] - a.row_ptr[:-1], len_a) + torch.arange(
+        a.nnz, device="cuda")
+    for k in ("col", "lo", "up"):
+        assert torch.equal(getattr(a, k), getattr(b, k)[at]), k
