@@ -83,38 +83,31 @@ impact_status tuning_of(const impact_tuning *t, Tuning &T)
 // ---------------------------------------------------------------------------
 
 
-// What the passes of the planned builds need: item and leaf table numbering,
-// shared memory.
-void size_batch(Batch &B)
+// What the passes of build q need beside those before it: item and leaf table
+// numbering, shared memory.
+void size_build(Batch &B, int q)
 {
-    const int count = B.count();
-    B.item_begin.assign((size_t)count * IMPACT_MAX_DIM + 1, 0);
-    B.leaf_begin.assign(count + 1, 0);
-    B.rec_max = B.leaf_smem = B.shared32 = B.any64 = B.warp64 = 0;
-    for (int &w : B.work_max) w = 0;
-    for (int q = 0; q < count; ++q) {
-        const ImpactDesc &D = B.plans[q].desc;
-        if (B.prec == IMPACT_FP32_SOUND) {
-            B.rec_max = std::max(B.rec_max, D.rec_stride);
-            for (int mode = 0; mode < 3; ++mode)
-                B.work_max[mode] = std::max(B.work_max[mode], impact::walk_work_bytes(D, mode));
+    const ImpactDesc &D = B.plans[q].desc;
+    if (B.prec == IMPACT_FP32_SOUND) {
+        B.rec_max = std::max(B.rec_max, D.rec_stride);
+        for (int mode = 0; mode < 3; ++mode)
+            B.work_max[mode] = std::max(B.work_max[mode], impact::walk_work_bytes(D, mode));
+    }
+    for (int d = 0; d < IMPACT_MAX_DIM; ++d) {
+        const size_t i = (size_t)q * IMPACT_MAX_DIM + d;
+        int64_t units = 0;
+        if ((D.walk64 || D.share32) && d < D.n) {
+            const int ipw = 32 / D.dim[d].group;
+            units = (D.dim[d].n_items + ipw - 1) / ipw;
         }
-        for (int d = 0; d < IMPACT_MAX_DIM; ++d) {
-            const size_t i = (size_t)q * IMPACT_MAX_DIM + d;
-            int64_t units = 0;
-            if ((D.walk64 || D.share32) && d < D.n) {
-                const int ipw = 32 / D.dim[d].group;
-                units = (D.dim[d].n_items + ipw - 1) / ipw;
-            }
-            B.item_begin[i + 1] = B.item_begin[i] + units;
-        }
-        B.leaf_begin[q + 1] = B.leaf_begin[q] + (D.leaf_shared ? D.leaf_items : 0);
-        if (D.leaf_shared) B.leaf_smem = std::max(B.leaf_smem, impact::leaf32_bytes(D));
-        if (D.share32) ++B.shared32;
-        if (D.walk64) {
-            ++B.any64;
-            B.warp64 = std::max(B.warp64, (int)impact::walk64_bytes(D));
-        }
+        B.item_begin[i + 1] = B.item_begin[i] + units;
+    }
+    B.leaf_begin[q + 1] = B.leaf_begin[q] + (D.leaf_shared ? D.leaf_items : 0);
+    if (D.leaf_shared) B.leaf_smem = std::max(B.leaf_smem, impact::leaf32_bytes(D));
+    if (D.share32) ++B.shared32;
+    if (D.walk64) {
+        ++B.any64;
+        B.warp64 = std::max(B.warp64, (int)impact::walk64_bytes(D));
     }
 }
 
@@ -131,7 +124,9 @@ bool make_lean(Batch &B, int only)
         P.leaf_bytes = 0;
         P.desc.walk64 = P.desc.leaf_shared = P.desc.lists = 0;
     }
-    size_batch(B);
+    B.rec_max = B.leaf_smem = B.shared32 = B.any64 = B.warp64 = 0;
+    for (int &w : B.work_max) w = 0;
+    for (int q = 0; q < B.count(); ++q) size_build(B, q);
     return true;
 }
 
@@ -147,6 +142,8 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
     B.images.assign(count, nullptr);
     B.row_begin.assign(count + 1, 0);
     B.unit_begin.assign(count + 1, 0);
+    B.item_begin.assign((size_t)count * IMPACT_MAX_DIM + 1, 0);
+    B.leaf_begin.assign(count + 1, 0);
     B.prec = precision;
     uint64_t h = 1469598103934665603ull;
     for (int q = 0; q < count; ++q) {
@@ -163,12 +160,12 @@ impact_status make_batch(const impact_request *reqs, int count, impact_precision
         B.unit_begin[q + 1] = B.unit_begin[q] + (P.rows + rpw - 1) / rpw;
         B.nnz_bound = (B.nnz_bound > INT64_MAX - P.nnz_bound) ? INT64_MAX
                                                               : B.nnz_bound + P.nnz_bound;
+        size_build(B, q);
         h = mix(h, P.hash);
     }
     B.rows = B.row_begin[count];
     B.units = B.unit_begin[count];
     B.hash = h;   // launch shapes change no result: they are not part of the identity
-    size_batch(B);
     if (precision == IMPACT_FP32_SOUND &&
         2 * (int64_t)B.rec_max + B.work_max[WALK_FUSED] > IMPACT_WALK_SMEM_MAX)
         return fail(IMPACT_ERR_ARG,
