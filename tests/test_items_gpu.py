@@ -155,3 +155,28 @@ def test_shared_windows_by_lane_groups_equal_those_by_lanes(cells, sigma):
         a.nnz, device="cuda")
     for k in ("col", "lo", "up"):
         assert torch.equal(getattr(a, k), getattr(b, k)[at]), k
+
+
+def repeated(count, distinct):
+    return np.resize(np.random.default_rng(6).uniform(-0.4, 0.4, (distinct, 1)), (count, 1))
+
+
+# input lists around the longest whose classes are all found, with few and many
+# distinct points
+MORE = {
+    "inputs-2048": lambda: linear([5, 4], np.eye(2) * 0.9, [0.6, 0.5], 1e-8, repeated(2048, 2048)),
+    "inputs-2049": lambda: linear([5, 4], np.eye(2) * 0.9, [0.6, 0.5], 1e-8, repeated(2049, 2049)),
+    "inputs-cycle": lambda: linear([5, 4, 3], np.eye(3) * 0.9, [0.6, 0.5, 0.4], 1e-8, repeated(5001, 7)),
+    "inputs-long-cycle": lambda: linear([5, 4, 3], np.eye(3) * 0.9, [0.6, 0.5, 0.4], 1e-8,
+                                        repeated(9000, 4500)),
+}
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("name", list(MORE))
+def test_long_input_lists_match_the_oracle(orc, name, precision):
+    prob = MORE[name]()
+    csr = impact.build(prob, precision)
+    torch.cuda.synchronize()
+    rows = np.arange(prob.rows) if prob.rows <= 2000 else W.sample_rows(prob, 200, seed=2)
+    PA.compare(prob, csr, orc.build_rows(prob, rows), orc, precision).assert_ok()
