@@ -162,19 +162,23 @@ def repeated(count, distinct):
 
 
 # input lists around the longest whose classes are all found, with few and many
-# distinct points
+# distinct points; caller images whose windows are far narrower than the grid, of
+# different widths side by side
 MORE = {
     "inputs-2048": lambda: linear([5, 4], np.eye(2) * 0.9, [0.6, 0.5], 1e-8, repeated(2048, 2048)),
     "inputs-2049": lambda: linear([5, 4], np.eye(2) * 0.9, [0.6, 0.5], 1e-8, repeated(2049, 2049)),
     "inputs-cycle": lambda: linear([5, 4, 3], np.eye(3) * 0.9, [0.6, 0.5, 0.4], 1e-8, repeated(5001, 7)),
     "inputs-long-cycle": lambda: linear([5, 4, 3], np.eye(3) * 0.9, [0.6, 0.5, 0.4], 1e-8,
                                         repeated(9000, 4500)),
+    "images-70": lambda: images_of(linear([70], np.eye(1), [1.0], 1e-8, U2), 3),
+    "images-40x300": lambda: images_of(linear([40, 300], np.eye(2), [0.6, 5.0], 1e-8, U1), 4),
+    "images-outside": lambda: images_of(linear([33, 35], np.eye(2), [0.02, 0.02], 1e-3, U1), 5),
 }
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("name", list(MORE))
-def test_long_input_lists_match_the_oracle(orc, name, precision):
+def test_long_input_lists_and_narrow_windows_match_the_oracle(orc, name, precision):
     prob = MORE[name]()
     csr = impact.build(prob, precision)
     torch.cuda.synchronize()
