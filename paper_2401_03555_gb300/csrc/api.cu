@@ -451,6 +451,9 @@ cudaError_t setup_pass(const Batch &B, const Work &W, cudaStream_t st)
                                      B.item_begin.back(), W.status(), st);
 }
 
+// The builds of B into arrays of known capacity run as one walk.
+bool one_pass(const Batch &B) { return B.prec == PREC_FP32_SOUND && B.tune.one_pass; }
+
 // count pass: row_ptr (row pointers and the total), sink_lo, sink_up, trunc,
 // row_flags: per-row counts, then the scan. FP64 builds whose tables are too
 // large for the walk (ImpactDesc.walk64) are counted by the per-pair kernel.
@@ -520,7 +523,7 @@ impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int
 impact_status run_fused(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
                         cudaStream_t st, int64_t chunk_rows, bool fresh)
 {
-    if (B.prec != PREC_FP32_SOUND || !B.tune.one_pass) {
+    if (!one_pass(B)) {
         impact_status s = run_count(B, W, out, st, chunk_rows, fresh);
         if (s != IMPACT_OK) return s;
         return run_emit(B, W, out, capacity, true, st, chunk_rows);
@@ -634,6 +637,7 @@ impact_status build_into(Batch &B, impact_csr *out, bool lib_owned, cudaStream_t
         CK(dev_malloc_async(&out->row_flags, B.rows * 4, st));
     }
     Work W;
+    if (!lib_owned && one_pass(B) && !out->workspace) make_lean(B);   // it reads no leaf table
     if ((s = get_work(B, out, st, W)) != IMPACT_OK) return s;
     WorkHold hold{W, st};
     if (!W.owned) ws_tag(W.base, 0);
@@ -945,6 +949,7 @@ impact_status impact_graph_create(const impact_request *reqs, int count,
     g->rows = B.rows;
     g->capacity = out->nnz;
     Work W;
+    if (one_pass(B) && !out->workspace) make_lean(B);   // it reads no leaf table
     W.L = batch_layout(B);
     auto cleanup = [&](impact_status r) {
         if (g->exec) cudaGraphExecDestroy(g->exec);

@@ -79,6 +79,29 @@ def test_builds_without_tables_make_the_same_pairs(precision, make):
     assert impact.live_bytes() == base
 
 
+def test_one_pass_scratch_holds_no_leaf_tables():
+    """The one-pass walk reads none: its own scratch is smaller than the two-pass
+    build's by the leaf tables (16 MB of them or more), and the pairs are the same."""
+    prob = W.unicycle_3d(nx=31, ny=31, nth=17)
+    ref = impact.build(prob, "fp32")
+    rb, pb = impact.alloc_rows(prob.rows), impact.alloc_pairs(ref.nnz, "fp32")
+    base = impact.live_bytes()[0]
+    held = []
+    for one_pass in (False, True):
+        batch = impact.Batch([prob], "fp32", tune=impact.tuning(one_pass=one_pass))
+        graph = batch.graph(rb, pb, ref.nnz)
+        held.append(impact.live_bytes()[0] - base)
+        graph.launch()
+        torch.cuda.synchronize()
+        assert graph.result() == ref.nnz
+        graph.close()
+        assert torch.equal(pb["col"], ref.col) and torch.equal(pb["up"], ref.up)
+        pb["col"].fill_(-3)
+        assert batch.build_into(rb, pb, ref.nnz) == ref.nnz
+        assert torch.equal(pb["col"], ref.col) and torch.equal(rb["trunc"], ref.trunc)
+    assert held[1] <= held[0] - (16 << 20)
+
+
 def test_build_without_the_callers_scratch(monkeypatch):
     """impact.build when torch cannot give the workspace: the library's own."""
     prob = dense_2d()
