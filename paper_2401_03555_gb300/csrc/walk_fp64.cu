@@ -61,12 +61,11 @@ struct Item64 {
     double SW;             // sum of U over the trimmed window
     double O;              // mass outside the trimmed window
     double gmax, gmin;     // in-domain mass: largest, smallest over the image
-    double M;              // largest U of the trimmed window
-    float M32;             // M rounded up
+    float M32;             // largest U of the trimmed window, rounded up
     int ta, tw;            // trimmed window [ta, ta + tw)
     int first;             // its first entry in the table
 };
-static_assert(sizeof(Item64) == 56, "Item64 layout");
+static_assert(sizeof(Item64) == 48, "Item64 layout");
 constexpr int kItemHead = 64;
 
 __host__ __device__ inline bool is_sorted_dim(float cutoff32, int w64)
@@ -265,7 +264,6 @@ items_fp64(const BatchIndex *__restrict__ B, uint32_t *__restrict__ status)
             h.O = ow + left + right;
             h.gmax = gmax;
             h.gmin = gmin;
-            h.M = M;
             h.M32 = __double2float_ru(M);
             h.ta = empty ? a : a + first;
             h.tw = tw;
