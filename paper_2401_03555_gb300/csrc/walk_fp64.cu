@@ -851,7 +851,8 @@ int64_t size_items64(ImpactDesc &D)
         const int64_t st = kItemHead + 16 * (int64_t)g.w64 + (sorted ? 40 * (int64_t)(g.w64 + 1) : 0);
         g.item_stride = (int)std::min<int64_t>((st + 15) / 16 * 16, INT32_MAX / 2 / 16 * 16);
         g.item_off = bytes;
-        bytes += g.n_items * (int64_t)g.item_stride;
+        bytes = g.n_items > kItemsMax / g.item_stride || bytes > kItemsMax
+                    ? kItemsMax + 1 : bytes + g.n_items * (int64_t)g.item_stride;
     }
     // a window box too wide for a warp's shared memory, or tables beyond a fixed
     // size (images that are nearly all distinct, on large grids), keep the
