@@ -715,7 +715,7 @@ def run_synthesis(eps=1e-6, oracle_iters=2):
     out = {"workload": SYNTH_WORKLOAD, "iterations": list(g.iterations), "ms": dt * 1e3,
            "ms_per_iteration": dt * 1e3 / its, "value": row_lps / dt, "unit": "row LPs/s",
            "p_min_max": float(g.p_min.max().item()),
-           "path": "impact_synthesize (sorting-method LP by warp bisection, one warp per row, "
+           "path": "impact_synthesize (sorting-method LP by bisection over ranks, one warp per row, "
                    "then one thread per cell)"}
     # the same controller with the region vectors (one box relaxation per region)
     rv = impact.region_vectors(prob, target, avoid, "box", "fp64")

@@ -189,9 +189,20 @@ impact_status impact_build(const impact_system *sys, const impact_grid *grid,
 
 /*
  * impact_workspace_bytes -- host-only: the device scratch one build uses: the
- * uploaded descriptor and tables, the scan partial sums, the windows of the
- * distinct images and, per row, 16 bytes and the row's record
- * (IMPACT_FP32_SOUND) or 24 bytes (IMPACT_FP64_PLAIN).
+ * uploaded descriptor and tables, the scan partial sums and
+ *   IMPACT_FP32_SOUND  per row 16 bytes and its record; where rows share images
+ *                      the windows of the distinct ones (about a third of the
+ *                      records at most), else 16 bytes per row and dimension;
+ *                      the shared leaf tables (together no more than the
+ *                      records), which the one-pass build does not read;
+ *   IMPACT_FP64_PLAIN  per row 24 bytes and the factor tables of the distinct
+ *                      images, 1 GiB at most: a build that needs more of them
+ *                      is made pair by pair, slower, without.
+ * A call that allocates its own scratch (workspace NULL) and cannot have it with
+ * leaf or factor tables of 16 MiB or more runs without them: the same pairs, the
+ * FP64 truncated mass within the rounding of its sum. Region vectors (tables of
+ * 256 MiB at most) and sampled noise (masks of 256 MiB, kept entries of 1 GiB at
+ * most) likewise.
  */
 impact_status impact_workspace_bytes(const impact_system *sys, const impact_grid *grid,
                                      const impact_inputs *inputs, const double *sigma,
@@ -216,8 +227,8 @@ impact_status impact_count(const impact_system *sys, const impact_grid *grid,
  * Synchronizes `stream` once at the end to read the status. If
  * out->workspace is the one impact_count filled for these arguments, its
  * uploaded tables are reused; otherwise (NULL, or filled for other arguments:
- * IMPACT_ERR_ARG) pass NULL and the tables are uploaded again. Each row's factor tables are recomputed
- * on the device either way.
+ * IMPACT_ERR_ARG) pass NULL: the tables are uploaded and the records or factor
+ * tables made again.
  * Errors: IMPACT_ERR_ARG; IMPACT_ERR_CAPACITY when row_ptr[rows] > out->nnz
  *         (nothing written); IMPACT_ERR_CUDA when row_ptr does not match the
  *         arguments (a row whose pair count differs from its row_ptr range,
@@ -266,9 +277,12 @@ typedef struct {
  *   fault_row     r + 1: row r's row check sees a lower-bound sum of 2, so it
  *                 is flagged IMPACT_ROW_LO_SUM_ABOVE_ONE and the call returns
  *                 IMPACT_ERR_UNSOUND (needs row_flags; 0: off)
- *   guard_row     r + 1: row r's walk starts with its step guard spent, as if
- *                 an invariant of the walk had broken: the call returns
- *                 IMPACT_ERR_CUDA ("internal") (FP32 walks; 0: off)
+ *   guard_row     r + 1: row r's walk starts with its step guard spent, as one
+ *                 whose record was overwritten runs out of steps: the call
+ *                 returns IMPACT_ERR_CUDA ("internal"). The emit and the
+ *                 one-pass walk count their steps; the count pass, whose every
+ *                 step makes progress, reports the row at once (FP32 walks;
+ *                 0: off)
  * Shapes change speed only: results are bitwise identical for every shape.
  */
 typedef struct {
@@ -627,8 +641,10 @@ int impact_version(void);
  * impact_debug_fail_alloc -- the n-th device or pinned-host allocation the
  * library makes from now on (counting across all threads) fails as if the
  * device were out of memory, without allocating; the entry point that made it
- * returns IMPACT_ERR_OOM after releasing everything it took. n = 0 turns the
- * injection off; after the failure it is off again.
+ * returns IMPACT_ERR_OOM after releasing everything it took, or runs with less
+ * where what failed was scratch that it can do without
+ * (impact_workspace_bytes). n = 0 turns the injection off; after the failure it
+ * is off again.
  * Errors: IMPACT_ERR_ARG when n < 0.
  */
 impact_status impact_debug_fail_alloc(int64_t n);

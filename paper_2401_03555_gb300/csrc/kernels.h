@@ -18,7 +18,7 @@
 #define IMPACT_STATUS_CAPACITY 0x4u       // emit skipped: output capacity too small
 #define IMPACT_STATUS_EMIT_MISMATCH 0x8u  // emit found a different pair count than count
 #define IMPACT_STATUS_TIMEOUT 0x20u       // a bounded look-back wait gave up
-#define IMPACT_STATUS_INTERNAL 0x40u      // the walk's step guard ran out (broken invariant)
+#define IMPACT_STATUS_INTERNAL 0x40u      // a row's walk ran out of steps (damaged record)
 
 namespace impact {
 
@@ -128,8 +128,8 @@ cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_
 // the walk kernels read the records. A walk launch covers
 // the global rows [row_begin, row_end) of a batch (the pass's row counter
 // zeroed before each launch; launches of one pass in row order on one
-// stream). A warp's shared memory holds two record buffers of `rec_max`
-// bytes (the largest record_stride of the batch: the row being walked and the
+// stream). A warp's shared memory holds a record buffer of `rec_max` bytes (the
+// largest record_stride of the batch; COUNT two: the row being walked and the
 // next one, prefetched) and work space: `work_max` = the largest
 // walk_work_bytes of the batch per mode; `lb`: 16 bytes per row, for FUSED
 // one 8-byte look-back word per row, zeroed before the first launch of the
@@ -140,7 +140,7 @@ struct WalkFaults {
     int spin_limit = 0;        // look-back sleeps before giving up (0: the default)
     int64_t stall_row = -1;    // this row never publishes its count (-1: none)
     int64_t fault_row = -1;    // this row's checks see an impossible sum (-1: none)
-    int64_t guard_row = -1;    // this row's walk starts with its step guard spent (-1: none)
+    int64_t guard_row = -1;    // this row's walk has no steps (COUNT: fails at once; -1: none)
 };
 int64_t record_stride(int n, int tsum_cap);
 int walk_core_bytes(int n, int tsum_cap, int leaf_cap);   // both buffers and the work space

@@ -86,9 +86,9 @@ struct Work {
 // Copies the batch index, the descriptors, the tables and a zeroed status block
 // into W (stream-ordered).
 impact_status upload(const Batch &B, Work &W, cudaStream_t st);
-// The passes below launch the FP32 walk over all rows at once, or in chunks
-// of `chunk_rows` rows one after another on `st` (so that work on other
-// streams can take SMs between chunks); the FP64 kernels ignore chunk_rows.
+// The passes below launch the walks over all rows at once, or in chunks of
+// `chunk_rows` rows one after another on `st` (so that work on other streams can
+// take SMs between chunks); the per-pair FP64 kernel ignores chunk_rows.
 // count pass into out's row arrays (row pointers included). `fresh`: W's status
 // block is as an upload left it (zeroed).
 impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cudaStream_t st,

@@ -14,7 +14,7 @@
 //               dimension). The lanes of a row exchange their window maxima and
 //               sums by shuffles for the pruning thresholds.
 //   leaf_fp32   the sorted leaf tables (below) of the distinct images of the
-//               last two dimensions, for the count pass.
+//               last two dimensions, and their entries by kept count.
 //   terms_fp32  after the count pass, one thread per row: sink bounds, mass of
 //               the targets outside the window box, truncated mass and row
 //               checks (FP64, outward).
@@ -34,9 +34,10 @@
 //               product RU(P B[a, b]). The count pass finds how many entries of
 //               B pass under each parent by a binary search in B sorted by
 //               value, with prefix sums for the row sums (B from the row's shared
-//               leaf table, else sorted by the warp); the emit pass tests
-//               every entry of B under each parent, one lane each, and stores
-//               the kept pairs warp-contiguously.
+//               leaf table, else sorted by the warp). The emit pass stores
+//               the kept pairs warp-contiguously: from the lists of a shared
+//               table of 20 to 48 entries, one lane per kept pair, else every
+//               entry of B tested under each parent, one lane each.
 //
 // Kernel modes: COUNT (pairs per row, truncated mass, row checks), EMIT
 // (pairs at given row offsets) and FUSED (both: each row publishes its pair
@@ -831,8 +832,8 @@ constexpr int kSlots = kCap + 1;           // and a spare slot
 constexpr int kClaimBytes = 16;            // per warp: the claimed row range
 constexpr int kTrimMin = 512;              // emit: candidates of a chunk worth trimming its table for
 
-// Warp shared memory: two record buffers of the batch's largest record (the
-// row being walked and the next one, copied in meanwhile), then the work
+// Warp shared memory: a record buffer of the batch's largest record (in the count
+// pass two: the row being walked and the next one, copied in meanwhile), then the work
 // space (offsets fixed per problem by leaf_cap):
 //   h      RecDim[n]                 the row record's per-dimension entries
 //   ul     (U, L) x tsum_cap         the record's window tables
