@@ -277,12 +277,13 @@ typedef struct {
  *   fault_row     r + 1: row r's row check sees a lower-bound sum of 2, so it
  *                 is flagged IMPACT_ROW_LO_SUM_ABOVE_ONE and the call returns
  *                 IMPACT_ERR_UNSOUND (needs row_flags; 0: off)
- *   guard_row     r + 1: row r's walk starts with its step guard spent, as one
- *                 whose record was overwritten runs out of steps: the call
- *                 returns IMPACT_ERR_CUDA ("internal"). The emit and the
- *                 one-pass walk count their steps; the count pass, whose every
- *                 step makes progress, reports the row at once (FP32 walks;
- *                 0: off)
+ *   guard_row     r + 1: row r's walk reports a damaged record and the call
+ *                 returns IMPACT_ERR_CUDA ("internal"). An emit on a workspace
+ *                 that impact_count filled checks every row's record, so that
+ *                 one overwritten since cannot keep the walk going for ever (it
+ *                 sees row r's as overwritten); the walks of a call that made
+ *                 its records itself have nothing to check and report the row
+ *                 (FP32 walks; 0: off)
  * Shapes change speed only: results are bitwise identical for every shape.
  */
 typedef struct {

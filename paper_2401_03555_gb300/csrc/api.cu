@@ -384,7 +384,8 @@ impact_status status_result(uint32_t status)
     if (status & IMPACT_STATUS_TIMEOUT)
         return fail(IMPACT_ERR_TIMEOUT, "a row's look-back wait for the rows before it gave up");
     if (status & IMPACT_STATUS_INTERNAL)
-        return fail(IMPACT_ERR_CUDA, "internal: the walk's step guard ran out");
+        return fail(IMPACT_ERR_CUDA,
+                    "internal: a row's record is damaged (the walk's step guard refused it)");
     if (status & IMPACT_STATUS_TABLE_OVERFLOW)
         return fail(IMPACT_ERR_ARG,
                     "a row's window exceeded the planner's bound (caller images wider than "
@@ -415,14 +416,14 @@ impact::RowOutputs shifted(const impact::RowOutputs &o, int64_t rb, int64_t rows
 // pass's row counter (zero at the first launch, reset before the others).
 cudaError_t walk_pass(const Batch &B, const Work &W, int mode, int warps,
                       const impact::RowOutputs &o, unsigned long long *counter,
-                      int64_t chunk_rows, cudaStream_t st)
+                      int64_t chunk_rows, cudaStream_t st, bool saved = false)
 {
     const int64_t step = chunk_rows > 0 ? chunk_rows : std::max<int64_t>(B.rows, 1);
     for (int64_t r0 = 0; r0 < B.rows; r0 += step) {
         cudaError_t e = r0 > 0 ? cudaMemsetAsync(counter, 0, 8, st) : cudaSuccess;
         if (e == cudaSuccess)
             e = impact::launch_walk_fp32(W.index(), r0, std::min(B.rows, r0 + step),
-                                         B.rec_max, B.work_max, warps, mode, o,
+                                         B.rec_max, B.work_max, warps, mode, saved, o,
                                          W.lb(), B.tune.faults, st);
         if (e != cudaSuccess) return e;
     }
@@ -490,7 +491,8 @@ impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cu
 
 // emit pass at the row pointers in out->row_ptr
 impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
-                       bool records_ready, cudaStream_t st, int64_t chunk_rows, bool fresh)
+                       bool records_ready, cudaStream_t st, int64_t chunk_rows, bool fresh,
+                       bool saved)
 {
     if (!fresh) CK(cudaMemsetAsync(W.status(), 0, 64, st));
     impact::RowOutputs o{out->row_ptr, out->col, out->lo, out->up, nullptr, nullptr, nullptr,
@@ -500,7 +502,8 @@ impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int
             CK(setup_pass(B, W, st));
             CK(impact::launch_leaf_fp32(W.index(), B.leaf_begin.back(), B.leaf_smem, st));
         }
-        CK(walk_pass(B, W, WALK_EMIT, B.tune.emit_warps, o, W.counter() + 1, chunk_rows, st));
+        CK(walk_pass(B, W, WALK_EMIT, B.tune.emit_warps, o, W.counter() + 1, chunk_rows, st,
+                     saved));
     } else {
         if (B.any64) {
             if (!records_ready)
@@ -614,7 +617,7 @@ impact_status do_emit(Batch &B, impact_csr *out, cudaStream_t st)
     if ((s = get_work(B, out, st, W)) != IMPACT_OK) return s;
     WorkHold hold{W, st};
     if (!ready && (s = upload(B, W, st)) != IMPACT_OK) return s;
-    if ((s = run_emit(B, W, &view, out->nnz, ready, st, 0, false)) != IMPACT_OK) return s;
+    if ((s = run_emit(B, W, &view, out->nnz, ready, st, 0, false, ready)) != IMPACT_OK) return s;
     uint32_t status = 0;
     CK(cudaMemcpyAsync(&status, W.status(), 4, cudaMemcpyDeviceToHost, st));
     if ((s = release(W, st)) != IMPACT_OK) return s;

@@ -106,7 +106,6 @@ struct ImpactDesc {
     int rec_stride;           // bytes per row record in the workspace
     int leaf_cap;             // leaf-table entries a warp of the walk stages
     int walk_core;            // shared-memory bytes of one warp of the walk
-    uint32_t walk_steps;      // steps of a row's walk (its guard)
     const float2 *ea;         // per dim: N+1 edges in erf units, offset edge_off
     const float2 *ta_lo;      // AFFINE [n][n][Nmax]: min term A_dk x_k in erf units of d
     const float2 *ta_hi;      //                      max term

@@ -18,7 +18,7 @@
 #define IMPACT_STATUS_CAPACITY 0x4u       // emit skipped: output capacity too small
 #define IMPACT_STATUS_EMIT_MISMATCH 0x8u  // emit found a different pair count than count
 #define IMPACT_STATUS_TIMEOUT 0x20u       // a bounded look-back wait gave up
-#define IMPACT_STATUS_INTERNAL 0x40u      // a row's walk ran out of steps (damaged record)
+#define IMPACT_STATUS_INTERNAL 0x40u      // the walk refused a row's record (damaged)
 
 namespace impact {
 
@@ -133,14 +133,15 @@ cudaError_t launch_regions(const ImpactDesc &D, const ImpactDesc *d_desc, int64_
 // next one, prefetched) and work space: `work_max` = the largest
 // walk_work_bytes of the batch per mode; `lb`: 16 bytes per row, for FUSED
 // one 8-byte look-back word per row, zeroed before the first launch of the
-// pass, for COUNT the row's sums. COUNT writes per-row counts (a scan makes them row pointers), FUSED
+// pass, for COUNT the row's sums. `saved`: an EMIT whose records have lain in the
+// caller's workspace since the count; each row's is checked. COUNT writes per-row counts (a scan makes them row pointers), FUSED
 // the row pointers themselves.
 enum { WALK_COUNT = 0, WALK_EMIT = 1, WALK_FUSED = 2 };
 struct WalkFaults {
     int spin_limit = 0;        // look-back sleeps before giving up (0: the default)
     int64_t stall_row = -1;    // this row never publishes its count (-1: none)
     int64_t fault_row = -1;    // this row's checks see an impossible sum (-1: none)
-    int64_t guard_row = -1;    // this row's walk has no steps (COUNT: fails at once; -1: none)
+    int64_t guard_row = -1;    // this row's walk reports a damaged record (-1: none)
 };
 int64_t record_stride(int n, int tsum_cap);
 int walk_core_bytes(int n, int tsum_cap, int leaf_cap);   // both buffers and the work space
@@ -163,7 +164,7 @@ cudaError_t launch_leaf_fp32(const BatchIndex *d_index, int64_t tables, int leaf
                              cudaStream_t stream);
 cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64_t row_end,
                              int rec_max, const int work_max[3], int warps, int mode,
-                             const RowOutputs &o,
+                             bool saved, const RowOutputs &o,
                              unsigned long long *lb, const WalkFaults &f, cudaStream_t stream);
 // FP64 path (walk_fp64.cu): item tables, the walk (launches of one pass cover
 // row ranges in order; *counter zeroed before each; a count leaves 3 doubles

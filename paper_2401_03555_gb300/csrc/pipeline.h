@@ -94,11 +94,12 @@ impact_status upload(const Batch &B, Work &W, cudaStream_t st);
 impact_status run_count(const Batch &B, const Work &W, const impact_csr *out, cudaStream_t st,
                         int64_t chunk_rows = 0, bool fresh = false);
 // emit pass into out's pair arrays at the row pointers of a count pass
-// (`records_ready`: W holds the records or items of that count pass; `fresh`:
-// W's status block is as a count left it, or zeroed).
+// (`records_ready`: W holds the records or items of that count pass; `saved`:
+// the caller has held W since; `fresh`: W's status block is as a count left it,
+// or zeroed).
 impact_status run_emit(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
                        bool records_ready, cudaStream_t st, int64_t chunk_rows = 0,
-                       bool fresh = true);
+                       bool fresh = true, bool saved = false);
 // The whole build into arrays of known capacity (`fresh` as in run_count).
 impact_status run_fused(const Batch &B, const Work &W, const impact_csr *out, int64_t capacity,
                         cudaStream_t st, int64_t chunk_rows = 0, bool fresh = false);

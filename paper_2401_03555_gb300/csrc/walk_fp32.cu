@@ -1663,9 +1663,8 @@ __device__ __forceinline__ void leaf_emit_wide(const WarpMem &S, int n, const Le
 // come; the recursion is unrolled at compile time (a loop with the level as a
 // variable spends more on finding its place than on the nodes: the 8^5 room's
 // count pass took 1251 instructions a row, and takes 861). Every chunk takes at
-// least one of a list's candidates, whatever the record says, so every loop
-// ends; counting the steps as the emit does cost the 7-D building's count 2.80 ->
-// 3.04 ms, and its records were made in the same call.
+// least one of a list's candidates, so every loop ends (counting the steps
+// cost the 7-D building's count 2.80 -> 3.04 ms).
 template <int LEFT, bool ROOT>
 __device__ __forceinline__ void count_levels(const WarpMem &S, int n, const Leaf &f, int npar,
                                              int lane, CountAcc &acc, float cut)
@@ -1702,26 +1701,22 @@ __device__ __forceinline__ void count_row(const WarpMem &S, int n, const Leaf &f
 }
 
 // Writes the pairs of one row whose record is in S, or (COUNT: the one-pass walk,
-// which does both) counts them: the same lists, with the
-// level as a variable (the unrolled recursion keeps every level's loop state
+// which does both) counts them: the same lists, with the level as a variable (the unrolled recursion keeps every level's loop state
 // live, and the emit's inner loop needs the registers: 64 let 8 warps per
 // scheduler hide its shared-memory latency; unrolled, the 11^5 room's emit
-// pass took 7.8 ms against 7.45). Every turn of the loop fills a list, runs the
-// leaves of one or leaves one whose candidates are used up, and takes one of the
-// row's `steps`. A record bounds its lists, so a sound one never runs out
-// (ImpactDesc.walk_steps); one that was overwritten since the setup (a caller's
-// workspace between count and emit) could hold a chunk of no candidates, and a
-// walk without end. False: the steps ran out.
+// pass took 7.8 ms against 7.45). Every turn of the loop fills a list from one
+// candidate or more, runs the leaves of one or leaves one whose candidates are
+// used up, so the loop ends (counting the steps cost the room's emit 0.2 of 6.6
+// ms).
 template <bool COUNT>
-__device__ __forceinline__ bool walk_row(const WarpMem &S, int n, const Leaf &f, bool lists,
+__device__ __forceinline__ void walk_row(const WarpMem &S, int n, const Leaf &f, bool lists,
                                          int after, int lane, CountAcc &acc, const EmitOut &out,
-                                         int &written, float cut, unsigned steps)
+                                         int &written, float cut)
 {
     if (n <= 2) {
-        if (steps == 0) return false;
         if (COUNT) leaf_count(S, n, f, NodeList{}, true, 1, lane, acc, cut);
         else leaf_emit_wide(S, n, f, NodeList{}, true, 1, lane, out, written, cut);
-        return true;
+        return;
     }
     const EmitLeaf g = emit_leaf(S, f);
     if (!COUNT && g.staged && !lists)
@@ -1734,7 +1729,7 @@ __device__ __forceinline__ bool walk_row(const WarpMem &S, int n, const Leaf &f,
     const int last = n - 3;      // deepest list level
     int my_cur = 0, my_sz = 0;   // lane k: next candidate of level k, size of list k
     int k = 0;
-    for (; steps > 0; --steps) {
+    while (true) {
         if (k == last + 1) {
             const NodeList L = node_list(S.work, last);
             const int npar = __shfl_sync(0xffffffffu, my_sz, last);
@@ -1750,11 +1745,11 @@ __device__ __forceinline__ bool walk_row(const WarpMem &S, int n, const Leaf &f,
         const int cur = __shfl_sync(0xffffffffu, my_cur, k);
         const int total = npar * S.h[k].tw;
         if (cur >= total) {
-            if (k == 0) return true;
+            if (k == 0) break;
             --k;
             continue;
         }
-        const int end = min(cur + chunk_of(S.h[k]), total);
+        const int end = min(cur + max(chunk_of(S.h[k]), 1), total);
         const int nout = expand<COUNT>(S, k, k == 0, cur, end, lane, acc);
         if (lane == k) {
             my_cur = end;
@@ -1763,7 +1758,6 @@ __device__ __forceinline__ bool walk_row(const WarpMem &S, int n, const Leaf &f,
         if (lane == k + 1) my_cur = 0;
         ++k;
     }
-    return false;
 }
 
 // ---------------------------------------------------------------------------
@@ -1889,10 +1883,25 @@ struct WalkArgs {
     int64_t row_end;
     int64_t stall_row;       // fault injection: this row never publishes (-1: none)
     int64_t fault_row;       // fault injection: this row's checks see a bad sum (-1: none)
-    int64_t guard_row;       // fault injection: this row's step guard starts spent (-1: none)
+    int64_t guard_row;       // fault injection: this row reports a damaged record (-1: none)
 };
 
-template <int MODE>
+// A dimension's entry as finish_dim makes it: the window within the record's
+// tables, chunks of whole parents within a list, the division by its width.
+__device__ __forceinline__ bool sound_dim(const RecDim &h, int lay, int tsum_cap)
+{
+    const bool narrow = (unsigned)(h.tw - 1) < 32u;
+    return (narrow ? (unsigned)((lay >> 16) - 33) < 32u : lay == 0) &&
+           (unsigned)h.tw <= (unsigned)tsum_cap && (unsigned)h.tb <= (unsigned)(tsum_cap - h.tw) &&
+           (h.tw == 0 || (uint32_t)h.tw * h.magic < (uint32_t)h.tw);
+}
+
+// SAVED (an emit): the records have lain in the caller's workspace since the
+// count. Every row's are checked before it is walked: widths, chunks and
+// addresses out of a record that was overwritten would take the walk out of its
+// lists or keep it going for ever. (In every emit the check would cost the 7-D
+// building 0.03 of 4.50 ms.)
+template <int MODE, bool SAVED>
 __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const WalkArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1978,10 +1987,15 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
         unsigned char *const rec = wbase + b * A.rec_max;
         const WarpMem S = carve(work, rec, n, D.leaf_cap);
         const bool empty = __any_sync(0xffffffffu, lane < n && S.h[lane].tw == 0);
+        bool walked = true;
+        if (SAVED)   // fault injection: as if the record's chunks were overwritten
+            walked = !__any_sync(0xffffffffu,
+                                 lane < n && !sound_dim(S.h[lane],
+                                                        row == A.guard_row ? 1 : S.h[lane].lay,
+                                                        D.tsum_cap));
+        else if (kCount)
+            walked = row != A.guard_row;
         Leaf f = leaf_of(S, n);
-        // fault injection: a row whose steps are spent before the first
-        const unsigned steps = row == A.guard_row ? 0u : D.walk_steps;
-        bool walked = MODE != MODE_COUNT || steps > 0;   // that count has none to run out of
         bool lb_ok = true;
         int64_t base = 0, len = 0;
         if (kCount) {
@@ -2004,8 +2018,7 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
                 if (!f.shared) leaf_build(S, n, f, lane, cut);
                 if (MODE == MODE_FUSED) {
                     int none = 0;
-                    walked = walk_row<true>(S, n, f, false, 0, lane, acc, EmitOut{}, none, cut, steps);
-                    if (!walked) acc = CountAcc();
+                    walk_row<true>(S, n, f, false, 0, lane, acc, EmitOut{}, none, cut);
                 } else {
                     count_row(S, n, f, lane, acc, cut);
                 }
@@ -2077,11 +2090,9 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
                         __syncwarp();
                     }
                     CountAcc none;
-                    walked = walk_row<false>(S, n, f, lists, after, lane, none, out, written, cut,
-                                             steps);
+                    walk_row<false>(S, n, f, lists, after, lane, none, out, written, cut);
                 }
-                if (lane == 0 && walked && written != len)
-                    atomicOr(A.status, IMPACT_STATUS_EMIT_MISMATCH);
+                if (lane == 0 && written != len) atomicOr(A.status, IMPACT_STATUS_EMIT_MISMATCH);
             }
         }
         if (lane == 0 && !walked) atomicOr(A.status, IMPACT_STATUS_INTERNAL);
@@ -2173,16 +2184,6 @@ void size_items32(ImpactDesc &D, int64_t &item_bytes, int64_t &leaf_bytes)
                     D.leaf_items * D.leaf_stride <= D.rows * (int64_t)D.rec_stride;
     D.lists = D.leaf_shared && lists;
     leaf_bytes = D.leaf_shared ? D.leaf_items * D.leaf_stride : 0;
-    // The walk's guard: steps of a row whose windows are all as wide as they may
-    // be. A chunk but a list's last has 33 candidates or more and fills one list of
-    // the next level, so level k has at most 1 + (k + 1) prod / 33 chunks, prod its
-    // candidates; each is filled, walked and left. Twice that and more.
-    int64_t steps = 16, prod = 1;
-    for (int k = 0; k + 2 < n; ++k) {
-        prod = std::min(prod * D.dim[k].wcap, (int64_t)1 << 31);
-        steps += 8 * (int64_t)(k + 1) * (1 + prod / 32);
-    }
-    D.walk_steps = (uint32_t)std::min<int64_t>(steps, UINT32_MAX);
 }
 
 int leaf32_bytes(const ImpactDesc &D)
@@ -2238,7 +2239,7 @@ cudaError_t launch_leaf_fp32(const BatchIndex *d_index, int64_t tables, int leaf
 
 cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64_t row_end,
                              int rec_max, const int work_max[3], int warps, int mode,
-                             const RowOutputs &o,
+                             bool saved, const RowOutputs &o,
                              unsigned long long *lb, const WalkFaults &f, cudaStream_t stream)
 {
     const int64_t rows = row_end - row_begin;
@@ -2254,9 +2255,11 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
     warps = std::max(1, std::min({warps, IMPACT_TREE_WARPS_MAX, optin / std::max(warp_smem, 1)}));
     const int threads = warps * 32;
     const size_t smem = (size_t)warp_smem * warps;
-    const void *k = mode == MODE_COUNT  ? (const void *)walk_fp32<MODE_COUNT>
-                    : mode == MODE_EMIT ? (const void *)walk_fp32<MODE_EMIT>
-                                        : (const void *)walk_fp32<MODE_FUSED>;
+    auto kernel = mode == MODE_COUNT   ? walk_fp32<MODE_COUNT, false>
+                  : mode == MODE_FUSED ? walk_fp32<MODE_FUSED, false>
+                  : saved              ? walk_fp32<MODE_EMIT, true>
+                                       : walk_fp32<MODE_EMIT, false>;
+    const void *k = (const void *)kernel;
     cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     WalkArgs A;
@@ -2291,12 +2294,7 @@ cudaError_t launch_walk_fp32(const BatchIndex *d_index, int64_t row_begin, int64
                   : mode == MODE_FUSED ? 1
                       : (int)std::max<int64_t>(
                             1, std::min<int64_t>(4, rows / ((int64_t)g * warps * 256)));
-    if (mode == MODE_COUNT)
-        walk_fp32<MODE_COUNT><<<g, threads, smem, stream>>>(A);
-    else if (mode == MODE_EMIT)
-        walk_fp32<MODE_EMIT><<<g, threads, smem, stream>>>(A);
-    else
-        walk_fp32<MODE_FUSED><<<g, threads, smem, stream>>>(A);
+    kernel<<<g, threads, smem, stream>>>(A);
     return cudaGetLastError();
 }
 

@@ -1,6 +1,6 @@
-"""The FP32 walk's step guard on a record that was overwritten between the count
-and the emit (needs a GPU): a chunk of no candidates would be walked for ever;
-the row runs out of steps and is reported, every access in its own bounds."""
+"""The FP32 walk's guard on a record that was overwritten between the count and the
+emit (needs a GPU): a chunk of no candidates, which a walk that trusts it never
+gets through. The emit finds it before it walks the row and reports it."""
 
 import pytest
 import torch
