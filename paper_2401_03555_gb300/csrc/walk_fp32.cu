@@ -1925,7 +1925,7 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
     // registers live in its walk) copies each record when it starts it. So does the
     // one-pass walk, one row at a time: a row taken and not yet counted holds up
     // every row after it while its warp waits for the rows before the one it is at
-    // (a row ahead: the 11^5 room 85 ms, the unicycle 139; none: 14.5 and 22.5).
+    // (a row ahead: the 11^5 room 85 ms, the unicycle 139; none: 14.1 and 22.4).
     constexpr bool kAhead = MODE == MODE_COUNT;
     const int64_t row_end = A.row_end;
     unsigned char *const work = wbase + (kAhead ? 2 : 1) * A.rec_max;
@@ -1992,7 +1992,8 @@ __global__ void __launch_bounds__(IMPACT_TREE_WARPS_MAX * 32, 4) walk_fp32(const
             walked = !__any_sync(0xffffffffu,
                                  lane < n && !sound_dim(S.h[lane],
                                                         row == A.guard_row ? 1 : S.h[lane].lay,
-                                                        D.tsum_cap));
+                                                        D.tsum_cap)) &&
+                     (!D.lists || (uint64_t)rec_row(rec, n)->leaf < (uint64_t)D.leaf_items);
         else if (kCount)
             walked = row != A.guard_row;
         Leaf f = leaf_of(S, n);

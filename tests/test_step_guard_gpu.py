@@ -10,9 +10,14 @@ from paper_2401_03555_gb300 import impact, workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("prob", [W.room_5d(cells_per_dim=5), W.unicycle_3d(nx=15, ny=13, nth=7)],
-                         ids=lambda p: p.name)
-def test_a_chunk_of_no_candidates_ends_the_walk(prob):
+ROOM, CAR = W.room_5d(cells_per_dim=9), W.unicycle_3d(nx=15, ny=13, nth=7)
+FIELDS = ["chunk", "width", "magic", "table"]
+
+
+# the leaf table's number is read where the emit takes lists: in the rooms
+@pytest.mark.parametrize("prob,field", [(p, f) for p in (ROOM, CAR) for f in FIELDS] + [(ROOM, "leaf")],
+                         ids=lambda x: x if isinstance(x, str) else x.name)
+def test_an_overwritten_record_is_refused(prob, field):
     ref = impact.build(prob, "fp32")
     batch = impact.Batch([prob], "fp32")
     rb, pb = impact.alloc_rows(prob.rows), impact.alloc_pairs(ref.nnz, "fp32")
@@ -30,8 +35,17 @@ def test_a_chunk_of_no_candidates_ends_the_walk(prob):
               + ((torch.div(64, tw, rounding_mode="floor") * tw) << 16)))
     at = torch.nonzero(hit).flatten()
     assert len(at) >= prob.rows // 2
-    k = int(at[len(at) // 2]) + 1
-    v[k, 3] &= 0xffff
+    k = int(at[len(at) // 2])
+    if field == "chunk":
+        v[k + 1, 3] &= 0xffff
+    elif field == "width":
+        v[k, 0] = 1 << 20
+    elif field == "magic":
+        v[k, 3] += 1 << 24
+    elif field == "table":
+        v[k, 1] = 1 << 20
+    else:   # behind the dimensions' entries
+        v[k + 2 * prob.n, 1] = 1 << 8
     torch.cuda.synchronize()
     with pytest.raises(impact.ImpactError) as e:
         batch.emit(rb, pb, ref.nnz, ws)
